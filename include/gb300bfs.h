@@ -217,10 +217,12 @@ gb_status graph_prepare_batched(gb_graph *g, gb_stream s);
  *   timeout_ms         limit of every device-side wait (grid barriers, the
  *                      radix-sort look-back); on expiry the kernel records
  *                      GB_ERR_TIMEOUT and returns.
- *   blocks_per_sm      1, 2 or 3: blocks of the single-source kernel per SM
- *                      (3 trades register spills for more warps; 1 halves the
- *                      grid of 2, which makes the per-level grid barrier
- *                      cheaper on small graphs). */
+ *   blocks_per_sm      1, 2 or 3: warps of the single-source kernel per SM,
+ *                      in units of 16 (3 trades register spills for more
+ *                      warps; 1 makes the per-level grid barrier cheaper).
+ *                      With 1 and 2 the grid also follows the graph: graphs
+ *                      of up to 100 * 2^20 column entries run on at most one
+ *                      block per SM, small ones on fewer. */
 typedef struct gb_bfs_options {
     int canonical_parents;
     double alpha;

@@ -47,14 +47,21 @@
 namespace gb {
 namespace {
 
-constexpr int BFS_THREADS = 512;
+constexpr int BFS_THREADS = 512;    // threads of a block; BFS_WIDE of one when it has an SM to itself
+constexpr int BFS_WIDE = 1024;
 constexpr int BIG_CHUNK = 128;      // edges per chunk of a big frontier vertex (one round)
 constexpr int BU_LANE_FIRST = 8;    // bottom-up: each lane probes this many neighbours itself
 constexpr int BU_WORDS = 2;         // bottom-up hub pass: visited words (or 32-entry list groups) per warp step
 constexpr int PBUF = 256;           // per-warp ring of vertices left for the row pass
-constexpr int BFS_WARPS = BFS_THREADS / 32;
 constexpr int QBUF = 512;           // per-warp buffer of discovered vertices (shared memory)
 constexpr int BBUF = 32;            // per-warp buffer of discovered big-degree vertices
+// Narrow top-down levels are run by one block (solo_levels): frontiers of at
+// most SOLO_Q vertices with at most SOLO_E edges, or SOLO_E_SHORT edges if
+// the rows are short (at most SOLO_ROW entries each, one vertex per thread).
+// At 4,000 edges of long rows the one block took 20 us longer than the grid.
+constexpr int SOLO_Q = 1024;
+constexpr int SOLO_E = 1024;
+constexpr int SOLO_E_SHORT = 4096;
 constexpr int SITE_BFS_BAR = 20;
 constexpr int SITE_BFS_LEVELS = 21;
 
@@ -80,11 +87,20 @@ struct BigEnt {
     uint32_t cbase;
 };
 
+// What the block that ran a stretch of narrow levels tells the others.
+struct SoloRec {
+    long long l;        // level of the frontier it left (in ctl)
+    long long qbase;    // start of that frontier in the queue
+    long long prev_qn;  // size of the frontier before it
+    double mu;          // edges of unvisited vertices, before that frontier's are taken off
+};
+
 struct WsHeader {
     GridBarrier bar;
     unsigned done;
     unsigned pad0;
     LevelCtl ctl[4];
+    SoloRec solo;
     unsigned long long acc[6];  // edges, touched, reached, nlevels, td, bu
     unsigned long long t0;      // global timer at the end of the init phase
 };
@@ -476,10 +492,310 @@ __device__ __noinline__ void canonical_rescan(const BfsArgs &a, const unsigned *
     }
 }
 
-// MINB = blocks of BFS_THREADS per SM the register budget is sized for:
-// 2 (64 registers, no spills) or 3 (40 registers, more warps to hide latency).
-template <int MINB>
-__global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
+// Shared memory of solo_levels (laid over the warp buffers, which are empty
+// between levels): the frontier being expanded and the one being filled, each
+// vertex with its row start and degree, the exclusive prefix of the degrees,
+// and a ring of counters (one record being filled, one read, one cleared).
+struct SoloBuf {
+    int64_t start[2][SOLO_Q];
+    int32_t v[2][SOLO_Q];
+    int32_t deg[2][SOLO_Q];
+    int32_t pre[SOLO_Q];
+    struct {
+        unsigned long long mf;
+        int cnt, dmax;
+    } c[3];
+    unsigned long long big;
+    int wsum[32];
+    int stop;
+};
+static_assert(sizeof(SoloBuf) <= sizeof(WarpBuf) * (BFS_THREADS / 32), "SoloBuf lies over the warp buffers");
+static_assert(SOLO_Q == 2 * BFS_THREADS, "two frontier vertices per thread in the prefix sum");
+
+// Block-collective part of a narrow level: TD_E edges per thread (src[t] ->
+// v[t], v[t] < 0: none).  An edge's target is claimed on the visited bitmap
+// while its offsets are loaded; the winners join the next frontier.
+__device__ __forceinline__ void solo_visit(const BfsArgs &a, SoloBuf &sb, int nx, int slot, int l, int64_t qnext,
+                                           const int32_t (&src)[TD_E], const int32_t (&v)[TD_E],
+                                           unsigned long long &mfs, int &dmax)
+{
+    unsigned old[TD_E];
+    int64_t s0[TD_E];
+    int32_t dg[TD_E];
+#pragma unroll
+    for (int t = 0; t < TD_E; ++t)
+        old[t] = v[t] >= 0 ? atomicOr(&a.vis[(unsigned)v[t] >> 5], 1u << (v[t] & 31)) : kFull;
+#pragma unroll
+    for (int t = 0; t < TD_E; ++t) {
+        s0[t] = v[t] >= 0 ? __ldg(&a.off[v[t]]) : 0;
+        dg[t] = v[t] >= 0 ? (int32_t)(__ldg(&a.off[v[t] + 1]) - s0[t]) : 0;
+    }
+    int c = 0;
+#pragma unroll
+    for (int t = 0; t < TD_E; ++t) c += !((old[t] >> (v[t] & 31)) & 1u);
+    const int ci = warp_inclusive_scan(c);
+    int pos = 0;
+    if (lane_id() == 31 && ci) pos = atomicAdd(&sb.c[slot].cnt, ci);
+    pos = __shfl_sync(kFull, pos, 31) + ci - c;
+#pragma unroll
+    for (int t = 0; t < TD_E; ++t) {
+        if ((old[t] >> (v[t] & 31)) & 1u) continue;
+        a.parent[v[t]] = src[t];
+        mark_reached(a, v[t], l + 1, false);
+        if (GB_OK_IDX(a.st, qnext + pos, a.n, 243)) __stcg(&a.queue[qnext + pos], v[t]);
+        if (pos < SOLO_Q) {
+            sb.v[nx][pos] = v[t];
+            sb.start[nx][pos] = s0[t];
+            sb.deg[nx][pos] = dg[t];
+        }
+        mfs += (unsigned long long)dg[t];
+        dmax = dg[t] > dmax ? dg[t] : dmax;
+        ++pos;
+    }
+}
+
+// The frontier vertex of edge k in the prefix of the degrees (the last one
+// whose prefix is <= k).
+__device__ __forceinline__ int solo_owner(const SoloBuf &sb, int k)
+{
+    int o = 0;
+#pragma unroll
+    for (int step = SOLO_Q / 2; step >= 1; step >>= 1)
+        if (sb.pre[o + step] <= k) o += step;
+    return o;
+}
+
+// Canonical mode, CSR entry j of frontier vertex u at level l: if its target
+// was claimed by this level, u is one of its possible parents.
+__device__ __forceinline__ void solo_min_parent(const BfsArgs &a, int64_t j, int32_t u, int l)
+{
+    const int32_t w = GB_OK_IDX(a.st, j, a.nnz, 244) ? __ldg(&a.col[j]) : -1;
+    if (w < 0 || !GB_OK_IDX(a.st, w, a.n, 245)) return;
+    const unsigned e = __ldcg(&a.st8[w]) & ST_ESC;
+    const int lw = e == ST_ESC ? ldcg_i32(&a.level[w]) : (int)e - 1;
+    if (lw == l + 1) atomicMin(&a.parent[w], u);
+}
+
+// A stretch of narrow top-down levels, run by block 0 alone while the others
+// wait at the level barrier.  A level of a few hundred vertices is a chain of
+// dependent L2 accesses, not work: with the grid barrier and the global queue
+// and counters in that chain it took 7.5-10 us, whatever the frontier's size.
+// Here the frontier stays in shared memory with its row starts and degrees (a
+// discovered vertex's offsets are loaded beside the atomic that claims it), so
+// a level is two round trips to L2 (column, claim) and one block barrier.  A
+// frontier of short rows is dealt one vertex per thread; any other one edge
+// by edge, each thread finding its edges' vertices in the prefix of the
+// degrees, so that a hub does not hold one warp.  A 997 x 601 mesh (1,233
+// levels, frontiers of up to 1,000 vertices): 12.3 -> 6.3 ms, 10.0 -> 5.1 us a
+// level; levels of three vertices 2.3 us.
+//
+// The frontier bitmaps are not kept during the stretch: nothing reads them
+// between top-down levels.  Its last frontier's bits are set at the end, in
+// the bitmap Fn that is clear now and becomes the next level's.  In canonical
+// mode every frontier vertex offers itself as parent of the vertices the
+// level claimed (a minimum), so no rescan follows.  The stretch ends when the
+// frontier is empty or too wide for it, when the rule asks for bottom-up, or
+// after a quarter of the wait limit, so that the waiting blocks stay within it.
+constexpr int SOLO_ROW = 2 * TD_E;
+template <int NT>
+__device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l, int64_t qbase, int64_t qn,
+                                            int64_t bnext_base, double mf, double mu, unsigned *Fn, LevelCtl *nxt)
+{
+    const int tid = threadIdx.x;
+    const int lane = (int)lane_id();
+    const int warp = tid >> 5;
+    WsHeader *h = a.hdr;
+    const uint64_t t_start = globaltimer_ns();
+    for (int i = tid; i < qn; i += NT) {
+        int32_t u = ldcg_i32(&a.queue[qbase + i]);
+        if (!GB_OK_IDX(a.st, u, a.n, 240)) u = 0;
+        const int64_t s0 = a.off[u];
+        sb.v[0][i] = u;
+        sb.start[0][i] = s0;
+        sb.deg[0][i] = (int32_t)(a.off[u + 1] - s0);
+    }
+    if (tid == 0) {
+        sb.c[0].cnt = sb.c[0].dmax = 0;
+        sb.c[0].mf = 0;
+        sb.big = 0;
+        sb.stop = 0;
+    }
+    __syncthreads();
+    unsigned long long edges = 0, touched = 0;
+    int64_t prev_qn = 0;
+    int x = 0;                            // levels of the stretch so far
+    int slot = 0;                         // x mod 3: the counters being filled
+    int dm = SOLO_ROW + 1;                // the frontier's largest degree (not known of the first)
+    for (;;) {
+        const int cur = x & 1;
+        const int q = (int)qn;
+        const int total = (int)mf;
+        const int64_t qnext = qbase + qn;
+        const int slot1 = slot == 2 ? 0 : slot + 1;
+        if (tid == 0) {  // its last readers passed the previous level's barrier
+            sb.c[slot1].cnt = sb.c[slot1].dmax = 0;
+            sb.c[slot1].mf = 0;
+        }
+        unsigned long long mfs = 0;
+        int dmx = 0;
+        const bool by_edge = dm > SOLO_ROW;
+        if (!by_edge) {
+            for (int i0 = 0; i0 < q; i0 += NT) {
+                const int i = i0 + tid;
+                const int32_t u = i < q ? sb.v[cur][i] : 0;
+                const int d = i < q ? sb.deg[cur][i] : 0;
+                const int64_t s0 = i < q ? sb.start[cur][i] : 0;
+                for (int b = 0; b < dm; b += TD_E) {
+                    int32_t src[TD_E], v[TD_E];
+#pragma unroll
+                    for (int t = 0; t < TD_E; ++t) {
+                        src[t] = u;
+                        v[t] = b + t < d && GB_OK_IDX(a.st, s0 + b + t, a.nnz, 241) ? __ldg(&a.col[s0 + b + t]) : -1;
+                        if (v[t] >= 0 && !GB_OK_IDX(a.st, v[t], a.n, 242)) v[t] = -1;
+                    }
+                    solo_visit(a, sb, cur ^ 1, slot, l, qnext, src, v, mfs, dmx);
+                }
+            }
+        } else {
+            // exclusive prefix of the frontier's degrees, two vertices per thread
+            // (of the first SOLO_Q / 2)
+            const int d0 = 2 * tid < q ? sb.deg[cur][2 * tid] : 0;
+            const int d1 = 2 * tid + 1 < q ? sb.deg[cur][2 * tid + 1] : 0;
+            const int incl = warp_inclusive_scan(d0 + d1);
+            if (lane == 31) sb.wsum[warp] = incl;
+            __syncthreads();
+            const int ws = lane < NT / 32 ? sb.wsum[lane] : 0;
+            const int wi = warp_inclusive_scan(ws);
+            const int ex = __shfl_sync(kFull, wi - ws, warp) + incl - d0 - d1;
+            if (2 * tid < SOLO_Q) {
+                sb.pre[2 * tid] = 2 * tid < q ? ex : 0x7fffffff;
+                sb.pre[2 * tid + 1] = 2 * tid + 1 < q ? ex + d0 : 0x7fffffff;
+            }
+            __syncthreads();
+            for (int k0 = 0; k0 < total; k0 += TD_E * NT) {
+                int32_t src[TD_E], v[TD_E];
+#pragma unroll
+                for (int t = 0; t < TD_E; ++t) {
+                    const int k = k0 + t * NT + tid;
+                    const int o = solo_owner(sb, k);
+                    src[t] = sb.v[cur][o];
+                    const int64_t j = sb.start[cur][o] + (k - sb.pre[o]);
+                    v[t] = k < total && GB_OK_IDX(a.st, j, a.nnz, 241) ? __ldg(&a.col[j]) : -1;
+                    if (v[t] >= 0 && !GB_OK_IDX(a.st, v[t], a.n, 242)) v[t] = -1;
+                }
+                solo_visit(a, sb, cur ^ 1, slot, l, qnext, src, v, mfs, dmx);
+            }
+        }
+        if (__any_sync(kFull, mfs != 0)) {
+            // 64-bit degree sum from two 32-bit reductions (each half's sum fits)
+            const unsigned lo = __reduce_add_sync(kFull, (unsigned)(mfs & 0x3ffffffu));
+            const unsigned hi = __reduce_add_sync(kFull, (unsigned)(mfs >> 26));
+            dmx = __reduce_max_sync(kFull, dmx);
+            if (lane == 0) {
+                atomicAdd(&sb.c[slot].mf, ((unsigned long long)hi << 26) + lo);
+                atomicMax(&sb.c[slot].dmax, dmx);
+            }
+        }
+        if (tid == 0) {
+            edges += (unsigned long long)total;
+            touched += (unsigned long long)q;
+            if (l < kStatLevels || (x & 15) == 15) {
+                const uint64_t now = globaltimer_ns();
+                if (now - t_start > a.timeout_ns / 4) sb.stop = 1;
+                if (l < kStatLevels) {
+                    a.stats->level_ns[l] = now - h->t0;
+                    a.stats->level_frontier[l] = qn;
+                    a.stats->level_dir[l] = 1;
+                    h->t0 = now;
+                }
+            }
+        }
+        __syncthreads();
+        if (a.canonical) {
+            // smallest-id parents: every edge of the level once more, to the
+            // vertices the level claimed (parent writes above are complete)
+            for (int k = tid; by_edge && k < total; k += NT) {
+                const int o = solo_owner(sb, k);
+                solo_min_parent(a, sb.start[cur][o] + (k - sb.pre[o]), sb.v[cur][o], l);
+            }
+            for (int i = tid; !by_edge && i < q; i += NT)
+                for (int t = 0; t < sb.deg[cur][i]; ++t) solo_min_parent(a, sb.start[cur][i] + t, sb.v[cur][i], l);
+            __syncthreads();
+        }
+        const int64_t cnt = sb.c[slot].cnt;
+        const unsigned long long nmf = sb.c[slot].mf;
+        dm = sb.c[slot].dmax;
+        const bool stop = sb.stop != 0;
+        prev_qn = qn;
+        qbase = qnext;
+        qn = cnt;
+        mf = (double)nmf;
+        ++l;
+        ++x;
+        slot = slot1;
+        if (qn == 0 || qn > SOLO_Q || nmf > (unsigned long long)(dm > SOLO_ROW ? SOLO_E : SOLO_E_SHORT) || stop ||
+            l > a.n)
+            break;
+        if (qn > prev_qn && mf > (mu - mf) / a.alpha) break;  // the bottom-up rule, applied by the grid
+        mu -= mf;
+    }
+    // the frontier left: its bits, its big vertices, its counters (the first
+    // SOLO_Q vertices are in shared memory)
+    const int cur = x & 1;
+    for (int64_t i0 = 0; i0 < qn; i0 += TD_E * NT) {
+        int32_t u[TD_E];
+        int64_t d[TD_E];
+#pragma unroll
+        for (int t = 0; t < TD_E; ++t) {
+            const int64_t i = i0 + t * NT + tid;
+            u[t] = i >= qn ? -1 : i < SOLO_Q ? sb.v[cur][i] : ldcg_i32(&a.queue[qbase + i]);
+            if (u[t] >= 0 && !GB_OK_IDX(a.st, u[t], a.n, 246)) u[t] = -1;
+            if (u[t] >= 0) atomicOr(&Fn[(unsigned)u[t] >> 5], 1u << (u[t] & 31));
+        }
+        if (dm <= a.big_deg) continue;
+#pragma unroll
+        for (int t = 0; t < TD_E; ++t) {
+            const int64_t i = i0 + t * NT + tid;
+            d[t] = u[t] < 0 ? 0 : i < SOLO_Q ? (int64_t)sb.deg[cur][i] : a.off[u[t] + 1] - a.off[u[t]];
+        }
+#pragma unroll
+        for (int t = 0; t < TD_E; ++t) {
+            const bool big = d[t] > a.big_deg;
+            const unsigned bm = __ballot_sync(kFull, big);
+            if (!bm) continue;
+            const unsigned nch = big ? nchunks(d[t]) : 0u;
+            const unsigned incl = warp_inclusive_scan(nch);
+            unsigned long long b = 0;
+            if (lane == 31) b = atomicAdd(&sb.big, ((unsigned long long)__popc(bm) << 32) | incl);
+            b = __shfl_sync(kFull, b, 31);
+            const int64_t at = bnext_base + (int64_t)(b >> 32) + __popc(bm & lanemask_lt());
+            if (big && GB_OK_IDX(a.st, at, a.bigcap, 247))
+                __stcg(reinterpret_cast<unsigned long long *>(a.bigq) + at,
+                       (unsigned long long)(uint32_t)u[t] | (((b & 0xffffffffull) + incl - nch) << 32));
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        nxt->qcnt = (unsigned long long)qn;
+        nxt->mf = (unsigned long long)mf;
+        nxt->big = sb.big;
+        h->solo.l = l;
+        h->solo.qbase = qbase;
+        h->solo.prev_qn = prev_qn;
+        h->solo.mu = mu;
+        atomicAdd(&h->acc[0], edges);
+        atomicAdd(&h->acc[1], touched);
+        atomicAdd(&h->acc[4], (unsigned long long)x);
+    }
+    // the barrier that follows returns the buffers to the warps
+}
+
+// NT threads per block, MINB blocks per SM the register budget is sized for:
+// 2 x 512 or 1 x 1024 (64 registers, no spills), or 3 x 512 (40 registers,
+// more warps to hide latency).  One block of 1024 threads per SM keeps as many
+// warps as two of 512 but halves the arrivals at every level barrier.
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
 {
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
@@ -490,7 +806,7 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
     WsHeader *h = a.hdr;
     const int32_t root = a.root;
     unsigned bar_target = grid_barrier_base(&h->bar);
-    __shared__ WarpBuf s_wb[BFS_WARPS];
+    __shared__ WarpBuf s_wb[NT / 32];
     __shared__ unsigned long long s_mf;
     WarpBuf &wb = s_wb[threadIdx.x >> 5];
     int qn_buf = 0, bn_buf = 0;  // warp-uniform fill levels of wb
@@ -534,10 +850,13 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
     int64_t qbase = 0, bbase = 0, prev_qn = 0;
     double mu = (double)a.nnz;
     bool td = true, prev_td = true;
+    bool rescan = false;  // canonical mode: the frontier was claimed by a grid-wide top-down level
     unsigned long long my_edges = 0, my_touched = 0;
     int l = 0;
-    for (;; ++l) {
-        LevelCtl *cur = &h->ctl[l & 3];
+    // ring position of the level's bitmaps and control record: one step per
+    // grid-wide level and per stretch of narrow levels
+    for (int p = 0;; ++p, ++l) {
+        LevelCtl *cur = &h->ctl[p & 3];
         const int64_t qn = (int64_t)ldcg_u64(&cur->qcnt);
         if (qn == 0) break;
         if (l > n) {
@@ -551,28 +870,46 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
         mu -= mf;
         if (l > 0) {
             if (td) {
-                if (mf > mu / a.alpha) td = false;
+                // bottom-up pays while the frontier grows: after its peak, few
+                // vertices are unvisited and the ratio alone would send a
+                // search of thin last levels over every vertex again
+                if (mf > mu / a.alpha && qn > prev_qn) td = false;
             } else if (qn < prev_qn && (double)qn < (double)n / a.beta) {
                 td = true;
             }
         }
-        unsigned *F = a.fb + (size_t)(l & 3) * nw;
-        unsigned *Fn = a.fb + (size_t)((l + 1) & 3) * nw;
-        unsigned *Fz = a.fb + (size_t)((l + 2) & 3) * nw;
-        unsigned *Fp = a.fb + (size_t)((l + 3) & 3) * nw;
-        LevelCtl *nxt = &h->ctl[(l + 1) & 3];
+        unsigned *F = a.fb + (size_t)(p & 3) * nw;
+        unsigned *Fn = a.fb + (size_t)((p + 1) & 3) * nw;
+        unsigned *Fz = a.fb + (size_t)((p + 2) & 3) * nw;
+        unsigned *Fp = a.fb + (size_t)((p + 3) & 3) * nw;
+        LevelCtl *nxt = &h->ctl[(p + 1) & 3];
         const int64_t qnext_base = qbase + qn;
         const int64_t bnext_base = bbase + nb;
 
-        // Clear the bitmap and control record that level l+1 will fill.
+        // Clear the bitmap and control record that the next step will fill.
         for (int64_t w = gtid; w < nw; w += gthreads) Fz[w] = 0;
         if (gtid == 0) {
             LevelCtl z = {0, 0, 0, 0};
-            h->ctl[(l + 2) & 3] = z;
+            h->ctl[(p + 2) & 3] = z;
         }
 
         // Canonical parents of vertices claimed top-down at level l-1.
-        if (a.canonical && l > 0 && prev_td) canonical_rescan(a, Fp, qbase, qn, gwarp, nwarps);
+        if (rescan) canonical_rescan(a, Fp, qbase, qn, gwarp, nwarps);
+
+        // Narrow levels: block 0 runs them alone, the others wait.
+        if (td && qn <= SOLO_Q && (mf <= (double)SOLO_E || (mf <= (double)SOLO_E_SHORT && mf <= 4.0 * (double)qn))) {
+            if (blockIdx.x == 0)
+                solo_levels<NT>(a, reinterpret_cast<SoloBuf &>(s_wb), l, qbase, qn, bnext_base, mf, mu, Fn, nxt);
+            if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_BFS_BAR)) return;
+            l = (int)__ldcg(&h->solo.l) - 1;  // the loop adds one
+            qbase = __ldcg(&h->solo.qbase);
+            prev_qn = __ldcg(&h->solo.prev_qn);
+            mu = __ldcg(&h->solo.mu);
+            bbase += nb;
+            prev_td = true;
+            rescan = false;
+            continue;
+        }
 
         if (td) {
             // (a) chunks of big frontier vertices, a contiguous range per warp
@@ -834,6 +1171,7 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
             }
         }
         prev_td = td;
+        rescan = td && a.canonical;
         prev_qn = qn;
         qbase += qn;
         bbase += nb;
@@ -950,12 +1288,46 @@ static int vec_ok(const BfsArgs &a)
 int bfs_pick_blocks(int num_sms, int minb)
 {
     int per_sm = 0;
-    const void *k = minb == 2 ? (const void *)bfs_kernel<2> : (const void *)bfs_kernel<3>;
+    const void *k = minb == 2 ? (const void *)bfs_kernel<BFS_THREADS, 2> : (const void *)bfs_kernel<BFS_THREADS, 3>;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, BFS_THREADS, 0) != cudaSuccess ||
         per_sm < 1)
         per_sm = 1;
     return num_sms * std::min(per_sm, minb);
 }
+
+namespace {
+// How a search is launched: the kernel, its threads per block and its grid.
+struct BfsLaunch {
+    const void *kern;
+    int threads;
+    int blocks;
+};
+
+// `cap`: the most blocks the caller grants (0: the whole GPU).  The grid
+// follows the graph: every level passes a barrier of all its blocks, which
+// costs more than a small graph's work.  us per search of Kronecker graphs
+// (edgefactor 16) on 1 / 16 / 64 / 152 / 304 blocks of 512 threads: SCALE 10
+// 41 / 42 / 45 / 49 / 63; SCALE 14 92 / 59 / 61 / 67 / 82; SCALE 17 401 / 86 /
+// 72 / 77 / 97; SCALE 20 - / 240 / 122 / 107 / 132; SCALE 21 - / 486 / 212 /
+// 164 / 174; SCALE 22 - / 936 / 304 / 193 / 184.  Above kWideNnz two blocks'
+// worth of warps per SM are needed, as one block of 1024 threads.
+BfsLaunch pick_launch(int64_t nnz, const gb_bfs_options &o, int num_sms, int blocks2, int blocks3, int cap)
+{
+    constexpr int64_t kPerBlock = int64_t(1) << 15;  // CSR entries per block of a small graph
+    constexpr int64_t kWideNnz = int64_t(100) << 20;
+    const int one = std::max(1, std::min(blocks2, num_sms));
+    if (o.blocks_per_sm == 3) {
+        const int b = cap > 0 ? std::min(cap, blocks3) : blocks3;
+        return {(const void *)bfs_kernel<BFS_THREADS, 3>, BFS_THREADS, b};
+    }
+    if (o.blocks_per_sm == 2 && nnz >= kWideNnz && cap <= 0 && blocks2 >= 2 * num_sms)
+        return {(const void *)bfs_kernel<BFS_WIDE, 1>, BFS_WIDE, num_sms};
+    int b = o.blocks_per_sm == 1 || nnz < kWideNnz ? one : blocks2;
+    if (cap > 0) b = std::min(b, cap);
+    b = (int)std::min<int64_t>(b, std::max<int64_t>(1, (nnz + kPerBlock - 1) / kPerBlock));
+    return {(const void *)bfs_kernel<BFS_THREADS, 2>, BFS_THREADS, b};
+}
+}  // namespace
 
 namespace {
 // Entries of the open list: every warp of the grid gets a segment for the
@@ -1051,16 +1423,10 @@ gb_status bfs_impl(const gb_graph *g, int64_t root, int32_t *parent, int32_t *le
     a.vec_col = (reinterpret_cast<uintptr_t>(a.col) & 15u) == 0;  // allocated with col_alloc_entries
     a.timeout_ns = timeout_ns();
     void *args[] = {&a};
-    // 1 block per SM runs the 2-per-SM kernel on half its grid
-    const int minb = o.blocks_per_sm == 3 ? 3 : 2;
-    const int full = minb == 3 ? ctx->bfs_blocks
-                               : (o.blocks_per_sm == 1 ? std::max(1, ctx->bfs_blocks2 / 2) : ctx->bfs_blocks2);
-    const int blocks = grid > 0 && grid < full ? grid : full;
-    a.useg = open_list_seg(n, (int64_t)blocks * (BFS_THREADS / 32));
+    const BfsLaunch L = pick_launch(g->nnz, o, ctx->num_sms, ctx->bfs_blocks2, ctx->bfs_blocks, grid);
+    a.useg = open_list_seg(n, (int64_t)L.blocks * (L.threads / 32));
     if (a.useg == 0 || !a.hd) a.ulist = nullptr;  // the list walks read hd
-    const void *kern = minb == 2 ? (const void *)bfs_kernel<2> : (const void *)bfs_kernel<3>;
-    GB_CUDA(cudaLaunchCooperativeKernel(kern, dim3(blocks),
-                                        dim3(BFS_THREADS), args, 0, s));
+    GB_CUDA(cudaLaunchCooperativeKernel(L.kern, dim3(L.blocks), dim3(L.threads), args, 0, s));
     note_launch();
     return GB_OK;
 }
@@ -1153,7 +1519,7 @@ gb_status bfs_noalloc_impl(const int64_t *off, const int32_t *col, int64_t n, in
             GB_CUDA(cudaGetSymbolAddress((void **)&nd.scratch, g_noalloc_scratch));
             GB_CUDA(cudaDeviceGetAttribute(&nd.num_sms, cudaDevAttrMultiProcessorCount, dev));
             int per_sm = 0;
-            GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bfs_kernel<2>,
+            GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bfs_kernel<BFS_THREADS, 2>,
                                                                   BFS_THREADS, 0));
             nd.blocks = nd.num_sms * std::max(1, std::min(per_sm, 2));
             nd.ready = true;
@@ -1203,8 +1569,11 @@ gb_status bfs_noalloc_impl(const int64_t *off, const int32_t *col, int64_t n, in
     a.vec_col = 0;  // a caller's columns: neither alignment nor padding is known
     a.timeout_ns = timeout_ns();
     void *args[] = {&a};
-    GB_CUDA(cudaLaunchCooperativeKernel((const void *)bfs_kernel<2>, dim3(d.blocks),
-                                        dim3(BFS_THREADS), args, 0, s));
+    // the scratch holds no open list, so any grid will do; one block per SM at most
+    gb_bfs_options one = o;
+    one.blocks_per_sm = 1;
+    const BfsLaunch L = pick_launch(nnz, one, d.num_sms, d.blocks, d.blocks, 0);
+    GB_CUDA(cudaLaunchCooperativeKernel(L.kern, dim3(L.blocks), dim3(L.threads), args, 0, s));
     note_launch();
     DevStatus hst;
     GB_CUDA(cudaMemcpyAsync(&hst, ws + kNaStatus, sizeof(hst), cudaMemcpyDeviceToHost, s));
