@@ -134,7 +134,7 @@ struct MsArgs {
     unsigned long long active;  // serving: bits in use; ignored when do_init
     const MsSlots *slots;   // serving: per-bit outputs; nullptr = graph outputs [k][n]
     int vec_col;            // 1: every graph's column array is 16-byte aligned and padded
-    int32_t *huge;          // single-graph batch calls: vertices of degree > MS_HUGE (else null)
+    int32_t *huge;          // batch calls: vertices of degree > MS_HUGE (serving: null)
 };
 
 template <typename T>
@@ -572,38 +572,42 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
             a.mbuf[i] = 0;
             a.mbuf[a.mstride + i] = 0;
             a.mbuf[2 * a.mstride + i] = 0;
-            if (a.huge && i < ntot && s_g[0].off[i + 1] - s_g[0].off[i] > MS_HUGE)
-                a.huge[atomicAdd(&h->nhuge, 1ull)] = (int32_t)i;
+            if (i < ntot) {
+                const MsGraph &G = s_g[find_graph(s_voff, a.ng, i)];
+                if (G.off[i - G.voff + 1] - G.off[i - G.voff] > MS_HUGE)
+                    a.huge[atomicAdd(&h->nhuge, 1ull)] = (int32_t)i;
+            }
         }
         if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_MS_BAR)) return;
-        // roots: bit b of graph g at its root; roots that coincide share one entry
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            unsigned long long na = 0, mf = 0;
-            for (int g = 0; g < a.ng; ++g) {
-                const MsGraph G = s_g[g];
-                for (int b = 0; b < a.k; ++b) {
-                    const int64_t r0 = a.roots[(int64_t)g * a.k + b];
-                    const int64_t r = G.inv ? (int64_t)G.inv[r0] : r0;
-                    const int64_t gid = G.voff + r;
-                    if (a.mbuf[gid] == 0) {
-                        a.act[na++] = (int32_t)gid;
-                        const int64_t deg = G.off[r + 1] - G.off[r];
-                        mf += deg;
-                        if (deg > MS_BIG_DEG) {
-                            const unsigned long long p = h->ctl[0].big;
-                            a.bigq[p >> 32] = (unsigned long long)(uint32_t)gid | ((p & 0xffffffffull) << 32);
-                            h->ctl[0].big = p + ((1ull << 32) | (unsigned long long)((deg + MS_BIG_CHUNK - 1) / MS_BIG_CHUNK));
-                        }
+        // roots: bit b of graph g at its root, one thread each; roots that
+        // coincide share one entry (the first to set a bit makes it).  One
+        // thread placing them all, a chain of some ten memory accesses each,
+        // held 32 graphs x 8 roots for 0.4 ms of a 1.39 ms call, and 64 roots
+        // of one graph for 0.15 ms.
+        if (blockIdx.x == 0) {
+            for (int i = threadIdx.x; i < a.ng * a.k; i += MS_THREADS) {
+                const int b = i % a.k;
+                const MsGraph &G = s_g[i / a.k];
+                const int64_t r0 = a.roots[i];
+                const int64_t r = G.inv ? (int64_t)G.inv[r0] : r0;
+                const int64_t gid = G.voff + r;
+                const int64_t deg = G.off[r + 1] - G.off[r];
+                const T bit = (T)((T)1 << b);
+                if (atomic_or_mask(&a.mbuf[gid], bit) == 0) {
+                    a.act[atomicAdd(&h->ctl[0].na, 1ull)] = (int32_t)gid;
+                    atomicAdd(&h->ctl[0].mf, (unsigned long long)deg);
+                    if (deg > MS_BIG_DEG) {
+                        const unsigned long long nch = (unsigned long long)((deg + MS_BIG_CHUNK - 1) / MS_BIG_CHUNK);
+                        const unsigned long long p = atomicAdd(&h->ctl[0].big, (1ull << 32) | nch);
+                        a.bigq[p >> 32] = (unsigned long long)(uint32_t)gid | ((p & 0xffffffffull) << 32);
                     }
-                    a.mbuf[gid] |= (T)((T)1 << b);
-                    a.seen[gid] |= (T)((T)1 << b);
-                    a.hist[G.voff + r0] |= (T)((T)1 << b);  // level 0 (staging: original ids)
-                    G.pst[r0 * G.kst + b] = (int32_t)r0;
                 }
+                atomic_or_mask(&a.seen[gid], bit);
+                atomic_or_mask(&a.hist[G.voff + r0], bit);  // level 0 (staging: original ids)
+                G.pst[r0 * G.kst + b] = (int32_t)r0;
             }
-            h->ctl[0].na = na;
-            h->ctl[0].mf = mf;
-            h->acc[2] = (unsigned long long)a.ng * (unsigned long long)a.k;  // the roots themselves
+            if (threadIdx.x == 0)
+                h->acc[2] = (unsigned long long)a.ng * (unsigned long long)a.k;  // the roots themselves
         }
         if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_MS_BAR)) return;
     }
@@ -760,26 +764,29 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
             }
         } else {
             // bottom-up over all vertices with unseen bits.  First the huge
-            // rows (single-graph batches), one per warp, so that the longest
+            // rows (batch calls), one per warp, so that the longest
             // scans start at once; then groups of 32 consecutive vertices,
             // handed out by a counter (the next index fetched one group ahead)
             const int64_t nh = a.huge ? (int64_t)ldcg_u64(&h->nhuge) : 0;
             for (int64_t hi = gwarp; hi < nh; hi += nwarps) {
                 const int64_t gu = ldcg_i32(&a.huge[hi]);
+                const int g = find_graph(s_voff, a.ng, gu);
+                const MsGraph &G = s_g[g];
+                const int64_t lu = gu - G.voff;
                 const T sn = ld_mask(&a.seen[gu]);
                 const T need = all & (T)~sn;
-                const int64_t rs = s_g[0].off[gu], re = s_g[0].off[gu + 1];
+                const int64_t rs = G.off[lu], re = G.off[lu + 1];
                 T found = 0;
                 if (need) {
                     my_touched += (lane == 0);
-                    found = ms_row_warp(s_g, S, M, 0, orig_id(s_g[0], gu), rs, re, need, a.vec_col != 0,
-                                        my_edges);
+                    found = ms_row_warp(s_g, S, M, g, orig_id(G, lu), rs, re, need, a.vec_col != 0, my_edges);
                 }
                 if (found && lane == 0) {
-                    write_levels(s_g[0], S, gu, found, l + 1);
+                    write_levels(G, S, lu, found, l + 1);
                     st_mask(&a.seen[gu], (T)(sn | found));
                     st_mask(&Mn[gu], found);
-                    if (a.hist && l + 1 < MS_HIST) a.hist[(size_t)(l + 1) * a.mstride + orig_id(s_g[0], gu)] = found;
+                    if (a.hist && l + 1 < MS_HIST)
+                        a.hist[(size_t)(l + 1) * a.mstride + G.voff + orig_id(G, lu)] = found;
                     reached_new += __popcll((unsigned long long)found);
                     my_any |= found;
                 }
@@ -984,7 +991,7 @@ gb_status ms_launch(std::vector<MsGraph> gs, int k, const std::vector<int64_t> &
     const size_t o_act = o_m + up(3 * np * sizeof(T));
     const size_t o_big = o_act + up(3 * (size_t)ntot * sizeof(int32_t));
     const size_t o_huge = o_big + up(2 * bigcap * sizeof(unsigned long long));
-    const int64_t hugecap = ng == 1 ? nnz_tot / (MS_HUGE + 1) + 1 : 0;
+    const int64_t hugecap = nnz_tot / (MS_HUGE + 1) + 1;
     const size_t total = o_huge + hugecap * sizeof(int32_t);
     unsigned char *ws = nullptr;
     Scratch tmp(s);
@@ -1030,7 +1037,7 @@ gb_status ms_launch(std::vector<MsGraph> gs, int k, const std::vector<int64_t> &
     a.do_init = 1;
     a.active = 0;
     a.slots = nullptr;
-    a.huge = hugecap ? reinterpret_cast<int32_t *>(ws + o_huge) : nullptr;
+    a.huge = reinterpret_cast<int32_t *>(ws + o_huge);
     a.vec_col = 1;
     for (int i = 0; i < ng; ++i)
         if (reinterpret_cast<uintptr_t>(gs[i].col) & 15u) a.vec_col = 0;
