@@ -1,5 +1,9 @@
 // Kernel 1 (Sec. 2.2): the undirected CSR graph from the Kronecker tuples.
 //
+// Tuples in memory are sorted by buckets (bucket.cu).  The steps below serve
+// the inputs that it does not take (SCALE 27 and more, 2^31 tuples and more,
+// buckets that stay too long), a caller's own sort portions, and the generator fused with kernel 1:
+//
 //   1. symmetrise: tuple (u,v) becomes keys (u << S | v) and (v << S | u),
 //      S = scale, so one key holds an ordered pair in 2*S contiguous bits;
 //   2. radix sort of the keys (ceil(2S/8) passes): the CSR of Sec. 2.2 is
@@ -16,6 +20,7 @@
 // degree (the "hub" that the bottom-up step tests first: a neighbour with many
 // edges is the likeliest to sit in the frontier; rows longer than HUB_SCAN
 // are sampled by their first HUB_SCAN entries).
+#include "bucket.h"
 #include "common.cuh"
 #include "internal.h"
 
@@ -699,6 +704,13 @@ gb_status build_csr(const int64_t *edges, int64_t m, int scale, gb_graph *g, cud
     g->device = ctx->device;
     GB_CUDA(cudaMemsetAsync(ctx->status, 0, sizeof(DevStatus), s));
     if (nk == 0) return empty_csr(g, s);
+    // a caller that set a portion size asks for the LSD sort in portions
+    BucketPlan bp;
+    if (sort_portion() == SORT_PORTION_DEFAULT && bucket_plan(m, scale, false, &bp)) {
+        bool overflow = false;
+        const gb_status rc = bucket_build(edges, nullptr, m, scale, bp, g, &overflow, s);
+        if (rc != GB_OK || !overflow) return rc;
+    }
     uint64_t *k0 = nullptr, *k1 = nullptr;
     unsigned long long *hist = nullptr;
     SortPlan plan = sort_plan(0, 2 * scale);

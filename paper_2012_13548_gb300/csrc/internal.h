@@ -141,6 +141,7 @@ struct SortPlan {
 };
 SortPlan sort_plan(int begin_bit, int end_bit);
 // Keys per portion of radix_sort (process-wide; 0 restores the default 2^28).
+constexpr int64_t SORT_PORTION_DEFAULT = int64_t(1) << 28;  // also the largest
 gb_status set_sort_portion(int64_t keys);
 int64_t sort_portion();
 

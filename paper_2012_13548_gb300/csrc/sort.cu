@@ -30,7 +30,7 @@ constexpr int RS_ITEMS = 16;
 constexpr int RS_TILE = RS_THREADS * RS_ITEMS;  // keys per tile
 #define RS_MINB(vals) ((vals) ? 3 * 256 / RS_THREADS : 4 * 256 / RS_THREADS)
 static_assert(RS_THREADS % 256 == 0, "threads 0..255 own one digit each");
-constexpr int64_t RS_PORTION = int64_t(1) << 28;  // default and largest portion
+constexpr int64_t RS_PORTION = SORT_PORTION_DEFAULT;
 constexpr unsigned FLAG_AGG = 1u << 30;
 constexpr unsigned FLAG_INCL = 2u << 30;
 constexpr unsigned VAL_MASK = FLAG_AGG - 1u;

@@ -44,6 +44,7 @@
 // (each tuple finds its two entries by bisection of the sorted rows); the
 // weight-sorted rows come from one radix sort of (row << 25 | weight) keys
 // carrying the columns (stable, so equal weights keep ascending columns).
+#include "bucket.h"
 #include "common.cuh"
 #include "internal.h"
 
@@ -864,8 +865,10 @@ int sssp_pick_blocks(int num_sms)
 
 }  // namespace
 
-gb_status build_csr_weighted(const int64_t *edges, const float *w, int64_t m, int scale, gb_graph *g,
-                             cudaStream_t s)
+namespace {
+
+// Kernel 1 by the LSD sort, then each entry's least weight.
+gb_status attach_weights(const int64_t *edges, const float *w, int64_t m, int scale, gb_graph *g, cudaStream_t s)
 {
     gb_status rc = build_csr(edges, m, scale, g, s);
     if (rc != GB_OK) return rc;
@@ -888,10 +891,40 @@ gb_status build_csr_weighted(const int64_t *edges, const float *w, int64_t m, in
                                          : "graph_build_csr_weighted: device error while attaching weights");
         return (gb_status)hst.code;
     }
-    // the rows by ascending weight: one sort of (row << 25 | weight) keys with the columns
+    return GB_OK;
+}
+
+}  // namespace
+
+gb_status build_csr_weighted(const int64_t *edges, const float *w, int64_t m, int scale, gb_graph *g,
+                             cudaStream_t s)
+{
+    Context *ctx = context();
+    if (!ctx) return GB_ERR_CUDA;
+    BucketPlan bp;
+    bool overflow = true;
+    const bool buckets = sort_portion() == SORT_PORTION_DEFAULT;
+    if (buckets && bucket_plan(m, scale, true, &bp)) {
+        g->n = int64_t(1) << scale;
+        g->scale = scale;
+        g->device = ctx->device;
+        GB_CUDA(cudaMemsetAsync(ctx->status, 0, sizeof(DevStatus), s));
+        const gb_status rc = bucket_build(edges, w, m, scale, bp, g, &overflow, s);
+        if (rc != GB_OK) return rc;
+    }
+    if (overflow) {
+        const gb_status rc = attach_weights(edges, w, m, scale, g, s);
+        if (rc != GB_OK) return rc;
+    }
     const int64_t nnz = g->nnz;
     GB_CUDA(gb::dmalloc(&g->wadj, std::max<int64_t>(nnz, 4) * sizeof(uint2)));
-    if (nnz > 0) {
+    overflow = true;
+    if (buckets && nnz > 0) {
+        const gb_status rc = bucket_weight_order(g, g->wadj, &overflow, s);
+        if (rc != GB_OK) return rc;
+    }
+    if (overflow && nnz > 0) {
+        // the rows by ascending weight: one sort of (row << 25 | weight) keys with the columns
         uint64_t *k0 = nullptr, *k1 = nullptr, *ks = nullptr;
         uint32_t *v0 = nullptr, *v1 = nullptr, *vs = nullptr;
         Scratch tmp(s);
@@ -911,7 +944,6 @@ gb_status build_csr_weighted(const int64_t *edges, const float *w, int64_t m, in
     GB_CUDA(cudaStreamSynchronize(s));
     return GB_OK;
 }
-
 gb_status sssp_impl(const gb_graph *g, int64_t root, double delta, double *dist, int32_t *parent,
                     SsspDevStats *stats, cudaStream_t s)
 {
