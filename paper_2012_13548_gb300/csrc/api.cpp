@@ -75,12 +75,24 @@ SsspDevStats *sssp_stats_buffer()
     return t_sssp.dev;
 }
 
-// Free every device array of a graph (any may be null) and the graph.
+// Free every device array of a graph (any may be null) and the graph.  The
+// caller has waited for the work that uses them.
 void destroy_graph(gb_graph *g)
 {
+    int dev = -1;
+    cudaGetDevice(&dev);
+    const bool other = g->device >= 0 && g->device != dev;
+    if (other) cudaSetDevice(g->device);
     void *arrays[] = {g->off, g->col, g->nz, g->hub, g->nzl, g->hd, g->rl_off, g->rl_col, g->rl_perm, g->rl_inv, g->wgt, g->wadj};
     for (void *p : arrays)
-        if (p) gb::dfree(p);
+        if (p) gb::dfree_async(p, nullptr);
+    cudaMemPool_t pool;
+    uint64_t held = 0;
+    if (cudaDeviceGetDefaultMemPool(&pool, other ? g->device : dev) == cudaSuccess &&
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+        held > gb::kPoolKeep && cudaStreamSynchronize(nullptr) == cudaSuccess)
+        cudaMemPoolTrimTo(pool, gb::kPoolKeep);
+    if (other) cudaSetDevice(dev);
     delete g;
 }
 
@@ -323,6 +335,7 @@ gb_status graph_build_csr(const int64_t *edges, int64_t m, int scale, gb_graph *
         gb_graph *g = new gb_graph();
         gb_status rc = build_csr(edges, m, scale, g, as_stream(s));
         if (rc != GB_OK) {
+            cudaStreamSynchronize(as_stream(s));
             destroy_graph(g);
             return rc;
         }
@@ -343,6 +356,7 @@ gb_status graph_build_csr_counting(const int64_t *edges, int64_t m, int scale, g
         gb_graph *g = new gb_graph();
         gb_status rc = build_csr_counting(edges, m, scale, g, as_stream(s));
         if (rc != GB_OK) {
+            cudaStreamSynchronize(as_stream(s));
             destroy_graph(g);
             return rc;
         }
@@ -477,6 +491,7 @@ gb_status graph_generate_csr(int scale, int edgefactor, double a, double b, doub
         gb_graph *g = new gb_graph();
         gb_status rc = kron_csr(scale, edgefactor, a, b, c, seed_gen, seed_perm, g, as_stream(s));
         if (rc != GB_OK) {
+            cudaStreamSynchronize(as_stream(s));
             destroy_graph(g);
             return rc;
         }
@@ -522,19 +537,19 @@ gb_status graph_from_csr(const int64_t *off, const int32_t *col, int64_t n, int6
         g->scale = -1;
         g->device = ctx->device;
         cudaError_t e;
-        if ((e = gb::dmalloc(&g->off, (n + 1) * sizeof(int64_t))) != cudaSuccess ||
-            (e = gb::dmalloc(&g->col, col_alloc_entries(nnz) * sizeof(int32_t))) != cudaSuccess ||
+        if ((e = gb::dmalloc_async(&g->off, (n + 1) * sizeof(int64_t), st)) != cudaSuccess ||
+            (e = gb::dmalloc_async(&g->col, col_alloc_entries(nnz) * sizeof(int32_t), st)) != cudaSuccess ||
             (e = cudaMemcpyAsync(g->off, off, (n + 1) * sizeof(int64_t), cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
             (nnz && (e = cudaMemcpyAsync(g->col, col, nnz * sizeof(int32_t), cudaMemcpyDeviceToDevice, st)) != cudaSuccess) ||
             (e = cudaStreamSynchronize(st)) != cudaSuccess) {
-            gb::dfree(g->off);
-            gb::dfree(g->col);
-            delete g;
+            cudaStreamSynchronize(st);
+            destroy_graph(g);
             return cuda_fail(e, "graph_from_csr");
         }
         gb_status rc = build_graph_aux(g, st);
         if (rc == GB_OK && (e = cudaStreamSynchronize(st)) != cudaSuccess) rc = cuda_fail(e, "graph_from_csr");
         if (rc != GB_OK) {
+            cudaStreamSynchronize(st);
             destroy_graph(g);
             return rc;
         }
@@ -547,7 +562,11 @@ gb_status graph_free(gb_graph *g)
 {
     return guarded([&]() -> gb_status {
         if (!g) return GB_OK;
+        int dev = -1;
+        cudaGetDevice(&dev);
+        if (g->device >= 0 && g->device != dev) cudaSetDevice(g->device);
         cudaDeviceSynchronize();
+        if (g->device >= 0 && g->device != dev) cudaSetDevice(dev);
         destroy_graph(g);
         return GB_OK;
     });

@@ -94,11 +94,6 @@ struct BkCtl {
     unsigned nseg, ntile, npiece, ndesc, overflow, pad[3];
 };
 
-template <typename K>
-struct KeyBits {
-    static constexpr int value = 8 * (int)sizeof(K);
-};
-
 __device__ __forceinline__ uint64_t low_mask(int bits)
 {
     return bits >= 64 ? ~uint64_t(0) : (uint64_t(1) << bits) - 1;
@@ -629,7 +624,7 @@ constexpr int LF_CROWD = 64;
 constexpr int LF_PLACES = BK_CAP + BK_CAP / 32;
 
 struct LeafShared {
-    unsigned bins[LF_BINS + LF_ROWS + 2];
+    alignas(16) unsigned bins[LF_BINS + LF_ROWS + 4];
     unsigned row[LF_ROWS];  // entries, then first place | places << 16
     unsigned w[LF_WARPS];
     unsigned crowd;  // keys that the ranks will read
@@ -714,7 +709,7 @@ __device__ __forceinline__ bool count_sort(const LeafArgs &a, const Leaf<K> &lf,
     const K fmask = (K)low_mask(lf.fbits);
     const bool rows = lf.nrows > 1;
     const int total_max = nb + (rows ? lf.nrows : 0);
-    for (int i = tid; i <= total_max; i += LF_THREADS) sh.bins[i] = 0;
+    for (int i = tid; i <= total_max >> 2; i += LF_THREADS) reinterpret_cast<uint4 *>(sh.bins)[i] = make_uint4(0, 0, 0, 0);
     if (rows)
         for (int i = tid; i < lf.nrows; i += LF_THREADS) sh.row[i] = 0;
     if (tid == 0) sh.crowd = 0;
@@ -762,7 +757,7 @@ __device__ __forceinline__ bool count_sort(const LeafArgs &a, const Leaf<K> &lf,
     for (int i = tid; i < n; i += LF_THREADS) atomicAdd(&sh.bins[place(load(i)) + 1], 1u);
     __syncthreads();
     {  // exclusive scan of the places, each thread a run of them
-        const int per = (total + LF_THREADS - 1) / LF_THREADS;
+        const int per = ((total + LF_THREADS - 1) / LF_THREADS) | 1;  // odd: a warp's runs start in 32 banks
         const int i0 = 1 + tid * per, i1 = min(total + 1, i0 + per);
         unsigned t = 0, reads = 0;
         for (int i = i0; i < i1; ++i) {
@@ -1325,9 +1320,9 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     *overflow = ovf != 0;
     if (ovf) return GB_OK;
     g->nnz = (int64_t)nnz;
-    GB_CUDA(gb::dmalloc(&g->off, (n + 1) * sizeof(int64_t)));
-    GB_CUDA(gb::dmalloc(&g->col, col_alloc_entries(g->nnz) * sizeof(int32_t)));
-    if (WEIGHTED) GB_CUDA(gb::dmalloc(&g->wgt, std::max<int64_t>(g->nnz, 4) * sizeof(uint32_t)));
+    GB_CUDA(gb::dmalloc_async(&g->off, (n + 1) * sizeof(int64_t), s));
+    GB_CUDA(gb::dmalloc_async(&g->col, col_alloc_entries(g->nnz) * sizeof(int32_t), s));
+    if (WEIGHTED) GB_CUDA(gb::dmalloc_async(&g->wgt, std::max<int64_t>(g->nnz, 4) * sizeof(uint32_t), s));
     uint2 *kept = reinterpret_cast<uint2 *>(ws + o_kept);
     bk_compact_kernel<K><<<(unsigned)npos, CP_THREADS, 0, s>>>(kb, total, base, g->col, g->wgt, kept, nnz, ctx->status);
     bk_off_kernel<<<(int)std::min<int64_t>((n + 256) / 256, sms * 16), 256, 0, s>>>(la.rawoff, kept, total, n, g->nnz,

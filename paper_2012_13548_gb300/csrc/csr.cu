@@ -544,14 +544,14 @@ gb_status build_batched_layout(gb_graph *g, cudaStream_t s)
     auto fail = [&](cudaError_t e) {
         void *arrays[] = {tmpg.rl_off, tmpg.rl_col, tmpg.rl_perm, tmpg.rl_inv};
         for (void *p : arrays)
-            if (p) gb::dfree(p);
+            if (p) gb::dfree_async(p, s);
         return cuda_fail(e, "batched layout");
     };
     cudaError_t e;
-    if ((e = gb::dmalloc(&tmpg.rl_perm, (size_t)n * sizeof(int32_t))) != cudaSuccess ||
-        (e = gb::dmalloc(&tmpg.rl_inv, (size_t)n * sizeof(int32_t))) != cudaSuccess ||
-        (e = gb::dmalloc(&tmpg.rl_off, (size_t)(n + 1) * sizeof(int64_t))) != cudaSuccess ||
-        (e = gb::dmalloc(&tmpg.rl_col, (size_t)col_alloc_entries(g->nnz) * sizeof(int32_t))) != cudaSuccess)
+    if ((e = gb::dmalloc_async(&tmpg.rl_perm, (size_t)n * sizeof(int32_t), s)) != cudaSuccess ||
+        (e = gb::dmalloc_async(&tmpg.rl_inv, (size_t)n * sizeof(int32_t), s)) != cudaSuccess ||
+        (e = gb::dmalloc_async(&tmpg.rl_off, (size_t)(n + 1) * sizeof(int64_t), s)) != cudaSuccess ||
+        (e = gb::dmalloc_async(&tmpg.rl_col, (size_t)col_alloc_entries(g->nnz) * sizeof(int32_t), s)) != cudaSuccess)
         return fail(e);
     rl_perm_kernel<<<ctx->num_sms * 8, 256, 0, s>>>(vs, g->off, n, tmpg.rl_perm, tmpg.rl_inv, dnew);
     note_launch();
@@ -594,7 +594,7 @@ gb_status build_graph_aux(gb_graph *g, cudaStream_t s)
     Context *ctx = context();
     if (!ctx) return GB_ERR_CUDA;
     const int64_t nw = (g->n + 31) / 32;
-    GB_CUDA(gb::dmalloc(&g->nz, nw * sizeof(uint32_t)));
+    GB_CUDA(gb::dmalloc_async(&g->nz, nw * sizeof(uint32_t), s));
     nz_bitmap_kernel<<<ctx->num_sms * 4, 256, 0, s>>>(g->off, g->n, g->nz, nw);
     note_launch();
     GB_CUDA(cudaGetLastError());
@@ -614,12 +614,12 @@ gb_status build_graph_aux(gb_graph *g, cudaStream_t s)
         GB_CUDA(cudaMemcpyAsync(&nnzv, base + nb, sizeof(nnzv), cudaMemcpyDeviceToHost, s));
         GB_CUDA(cudaStreamSynchronize(s));
         g->nnzv = (int64_t)nnzv;
-        GB_CUDA(gb::dmalloc(&g->nzl, std::max<int64_t>(g->nnzv, 4) * sizeof(int32_t)));
+        GB_CUDA(gb::dmalloc_async(&g->nzl, std::max<int64_t>(g->nnzv, 4) * sizeof(int32_t), s));
         nzl_write_kernel<<<(unsigned)nb, NZL_WORDS, 0, s>>>(g->nz, nw, base, g->nzl);
         note_launch();
         GB_CUDA(cudaGetLastError());
     }
-    GB_CUDA(gb::dmalloc(&g->hub, std::max<int64_t>(g->n, 1) * sizeof(int32_t)));
+    GB_CUDA(gb::dmalloc_async(&g->hub, std::max<int64_t>(g->n, 1) * sizeof(int32_t), s));
     uint8_t *key = nullptr;
     GB_CUDA(tmp.alloc(&key, (size_t)g->n));
     deg_key_kernel<<<ctx->num_sms * 4, 256, 0, s>>>(g->off, g->n, key);
@@ -627,7 +627,7 @@ gb_status build_graph_aux(gb_graph *g, cudaStream_t s)
     hub_kernel<<<ctx->num_sms * 8, HUB_THREADS, 0, s>>>(g->off, g->col, key, g->n, g->nnz, g->hub,
                                                         ctx->status);
     note_launch();
-    GB_CUDA(gb::dmalloc(&g->hd, std::max<int64_t>(g->n, 1) * sizeof(int2)));
+    GB_CUDA(gb::dmalloc_async(&g->hd, std::max<int64_t>(g->n, 1) * sizeof(int2), s));
     hd_kernel<<<ctx->num_sms * 8, 256, 0, s>>>(g->off, g->hub, g->n, g->hd);
     note_launch();
     GB_CUDA(cudaGetLastError());
@@ -670,8 +670,8 @@ gb_status csr_from_keys(uint64_t *k0, uint64_t *k1, int64_t nk, int scale, gb_gr
         return (gb_status)hst.code;
     }
     g->nnz = (int64_t)nnz;
-    GB_CUDA(gb::dmalloc(&g->off, (n + 1) * sizeof(int64_t)));
-    GB_CUDA(gb::dmalloc(&g->col, col_alloc_entries(g->nnz) * sizeof(int32_t)));
+    GB_CUDA(gb::dmalloc_async(&g->off, (n + 1) * sizeof(int64_t), s));
+    GB_CUDA(gb::dmalloc_async(&g->col, col_alloc_entries(g->nnz) * sizeof(int32_t), s));
     k1_write_kernel<<<(unsigned)ntiles, FIN_THREADS, 0, s>>>(ks, nk, scale, tbase, wcnt, n, g->off,
                                                              g->col, g->nnz, ctx->status);
     note_launch();
@@ -683,8 +683,8 @@ gb_status csr_from_keys(uint64_t *k0, uint64_t *k1, int64_t nk, int scale, gb_gr
 gb_status empty_csr(gb_graph *g, cudaStream_t s)
 {
     g->nnz = 0;
-    GB_CUDA(gb::dmalloc(&g->off, (g->n + 1) * sizeof(int64_t)));
-    GB_CUDA(gb::dmalloc(&g->col, 16));
+    GB_CUDA(gb::dmalloc_async(&g->off, (g->n + 1) * sizeof(int64_t), s));
+    GB_CUDA(gb::dmalloc_async(&g->col, 16, s));
     GB_CUDA(cudaMemsetAsync(g->off, 0, (g->n + 1) * sizeof(int64_t), s));
     gb_status r0 = build_graph_aux(g, s);
     if (r0 != GB_OK) return r0;
@@ -1161,14 +1161,14 @@ gb_status build_csr_counting(const int64_t *edges, int64_t m, int scale, gb_grap
         GB_CUDA(cudaGetLastError());
     }
     // 5: offsets from the distinct counts, then the columns
-    GB_CUDA(gb::dmalloc(&g->off, (n + 1) * sizeof(int64_t)));
+    GB_CUDA(gb::dmalloc_async(&g->off, (n + 1) * sizeof(int64_t), s));
     rc = cs_scan(dcnt, n, g->off, s);
     if (rc != GB_OK) return rc;
     int64_t nnz = 0;
     GB_CUDA(cudaMemcpyAsync(&nnz, g->off + n, sizeof(nnz), cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
     g->nnz = nnz;
-    GB_CUDA(gb::dmalloc(&g->col, col_alloc_entries(nnz) * sizeof(int32_t)));
+    GB_CUDA(gb::dmalloc_async(&g->col, col_alloc_entries(nnz) * sizeof(int32_t), s));
     cs_compact_kernel<<<grid, 256, 0, s>>>(s0, g->off, n, tmp, g->col, nnz, ctx->status);
     note_launch();
     GB_CUDA(cudaGetLastError());

@@ -72,6 +72,14 @@ inline cudaError_t dmalloc_async(T **p, size_t bytes, cudaStream_t s)
     return dmalloc_async_raw(reinterpret_cast<void **>(p), bytes, s);
 }
 
+// A graph's arrays come from the stream-ordered pool, in the order of the stream
+// that builds it, and go back to it when the graph is freed (graph_free waits
+// for the device first, so no stream still reads them).  cudaMalloc and
+// cudaFree map and unmap memory and wait for the device each time: a SCALE 16 build
+// took 554 us, of which its kernels 230.  What the pool keeps between graphs
+// is bounded: graph_free returns what exceeds kPoolKeep to the device.
+constexpr uint64_t kPoolKeep = uint64_t(48) << 30;  // a SCALE 26 build's temporaries and graph
+
 // Stream-ordered temporaries.
 template <typename T>
 inline cudaError_t alloc_async(T **p, size_t count, cudaStream_t s)

@@ -873,7 +873,7 @@ gb_status attach_weights(const int64_t *edges, const float *w, int64_t m, int sc
     gb_status rc = build_csr(edges, m, scale, g, s);
     if (rc != GB_OK) return rc;
     Context *ctx = context();
-    GB_CUDA(gb::dmalloc(&g->wgt, std::max<int64_t>(g->nnz, 4) * sizeof(uint32_t)));
+    GB_CUDA(gb::dmalloc_async(&g->wgt, std::max<int64_t>(g->nnz, 4) * sizeof(uint32_t), s));
     GB_CUDA(cudaMemsetAsync(g->wgt, 0xff, std::max<int64_t>(g->nnz, 4) * sizeof(uint32_t), s));
     if (m > 0) {
         wt_attach_kernel<<<ctx->num_sms * 8, 256, 0, s>>>(edges, w, m, g->off, g->col, g->n, g->wgt,
@@ -917,7 +917,7 @@ gb_status build_csr_weighted(const int64_t *edges, const float *w, int64_t m, in
         if (rc != GB_OK) return rc;
     }
     const int64_t nnz = g->nnz;
-    GB_CUDA(gb::dmalloc(&g->wadj, std::max<int64_t>(nnz, 4) * sizeof(uint2)));
+    GB_CUDA(gb::dmalloc_async(&g->wadj, std::max<int64_t>(nnz, 4) * sizeof(uint2), s));
     overflow = true;
     if (buckets && nnz > 0) {
         const gb_status rc = bucket_weight_order(g, g->wadj, &overflow, s);
