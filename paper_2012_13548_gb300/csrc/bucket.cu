@@ -51,6 +51,8 @@ constexpr int BK_SPLIT = 1024;                  // mean length aimed at by the e
 constexpr int BK_GROUP = 2048;                  // and how many keys' pieces are taken together
 static_assert(2 * BK_GROUP <= BK_CAP, "a group ends within BK_GROUP keys after the next border");
 constexpr int BK_ROWBITS = 9;                   // most rows of a bucket, as bits
+constexpr int SC_THREADS = 256;  // of the scans of a split's pieces
+constexpr int SC_WARPS = SC_THREADS / 32;
 constexpr int LF_THREADS = 256;
 constexpr int LF_WARPS = LF_THREADS / 32;
 constexpr int WBITS = 25;  // bits of a weight in units of 2^-24
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(BK_THREADS) bk_hist0_kernel(const int64_t *__r
         if (s_h[i]) atomicAdd(&cnt[i], s_h[i]);
 }
 
-// Exclusive scan of up to BK_BINS bin counts by one block of LF_THREADS.
+// Exclusive scan of up to BK_BINS bin counts by one block of SC_THREADS.
 __device__ __forceinline__ void scan_bins(const unsigned *cnt, int nb, unsigned *excl4, unsigned *s_w)
 {
     const int i0 = threadIdx.x * 4;
@@ -170,19 +172,19 @@ __device__ __forceinline__ void scan_bins(const unsigned *cnt, int nb, unsigned 
     }
     __syncthreads();
 }
-static_assert(LF_THREADS * 4 == BK_BINS, "scan_bins: four bins a thread");
+static_assert(SC_THREADS * 4 == BK_BINS, "scan_bins: four bins a thread");
 
 // The pieces of every listed bucket: places, cursors, descriptors.  One block a
 // bucket.  grouped: neighbouring pieces are taken together, those that start in
 // the same BK_GROUP keys, so that the next sort gets buckets of a useful length
 // (a piece longer than BK_GROUP stays alone); a group's keys count from the split
 // bucket's prefix, whose bits they still hold.
-__global__ void __launch_bounds__(LF_THREADS) bk_scan_kernel(const BkSeg *__restrict__ segs, BkCtl *__restrict__ ctl,
+__global__ void __launch_bounds__(SC_THREADS) bk_scan_kernel(const BkSeg *__restrict__ segs, BkCtl *__restrict__ ctl,
                                                              int grouped, const unsigned *__restrict__ cnt,
                                                              unsigned *__restrict__ cursor,
                                                              BkDesc *__restrict__ desc)
 {
-    __shared__ unsigned s_w[LF_WARPS], s_ex[BK_BINS + 1], s_base;
+    __shared__ unsigned s_w[SC_WARPS], s_ex[BK_BINS + 1], s_base;
     __shared__ uint16_t s_first[BK_BINS];
     const unsigned nseg = ctl->nseg;
     for (unsigned q = blockIdx.x; q < nseg; q += gridDim.x) {
@@ -202,7 +204,7 @@ __global__ void __launch_bounds__(LF_THREADS) bk_scan_kernel(const BkSeg *__rest
         if (threadIdx.x == 0) s_ex[nb] = sg.count;
         __syncthreads();
         if (!grouped) {
-            for (int i = threadIdx.x; i < nb; i += LF_THREADS)
+            for (int i = threadIdx.x; i < nb; i += SC_THREADS)
                 desc[sg.gbase + i] = whole_desc(sg.start + s_ex[i], s_ex[i + 1] - s_ex[i], pre | (uint64_t)i, rem);
         } else {
             unsigned first = 0, nf = 0;  // bit j: piece 4 t + j opens a group
@@ -220,7 +222,7 @@ __global__ void __launch_bounds__(LF_THREADS) bk_scan_kernel(const BkSeg *__rest
             if ((threadIdx.x & 31) == 31) s_w[threadIdx.x >> 5] = incl;
             __syncthreads();
             unsigned g = incl - nf, total = 0;
-            for (int w = 0; w < LF_WARPS; ++w) {
+            for (int w = 0; w < SC_WARPS; ++w) {
                 if (w < (int)(threadIdx.x >> 5)) g += s_w[w];
                 total += s_w[w];
             }
@@ -229,7 +231,7 @@ __global__ void __launch_bounds__(LF_THREADS) bk_scan_kernel(const BkSeg *__rest
                 if ((first >> j) & 1u) s_first[g++] = (uint16_t)(threadIdx.x * 4 + j);
             if (threadIdx.x == 0) s_base = atomicAdd(&ctl->ndesc, total);
             __syncthreads();
-            for (unsigned k = threadIdx.x; k < total; k += LF_THREADS) {
+            for (unsigned k = threadIdx.x; k < total; k += SC_THREADS) {
                 const int i = s_first[k], e = k + 1 < total ? (int)s_first[k + 1] : nb;
                 BkDesc d;
                 if (e == i + 1) {
@@ -250,11 +252,11 @@ __global__ void __launch_bounds__(LF_THREADS) bk_scan_kernel(const BkSeg *__rest
 }
 
 // Step 0's buckets: one segment over all keys, its total to *total.
-__global__ void __launch_bounds__(LF_THREADS) bk_scan0_kernel(const unsigned *__restrict__ cnt, int p0, int rem,
+__global__ void __launch_bounds__(SC_THREADS) bk_scan0_kernel(const unsigned *__restrict__ cnt, int p0, int rem,
                                                               unsigned *__restrict__ cursor,
                                                               BkDesc *__restrict__ desc, unsigned *__restrict__ total)
 {
-    __shared__ unsigned s_w[LF_WARPS];
+    __shared__ unsigned s_w[SC_WARPS];
     unsigned ex[4];
     const int nb = 1 << p0;
     scan_bins(cnt, nb, ex, s_w);
@@ -389,10 +391,10 @@ __global__ void __launch_bounds__(BK_THREADS, 2) bk_part0_kernel(const int64_t *
 
 // Lists the buckets to split and the tiles that cover them.  forced > 0: all of
 // them by that many bits, the pieces of bucket i at i << forced; else those
-// longer than BK_CAP, by as many bits as bring their pieces to BK_SPLIT keys on
-// average, and at least down to single rows (`field` bits hold what is not the
-// row): long buckets are long by one row as a rule, and bits of the row do not
-// split it.  low: bits that do not tell entries apart.
+// longer than BK_CAP, down to single rows (`field` bits hold what is not the
+// row) and from there by as many bits as bring a row of the bucket's length to
+// BK_SPLIT keys: long buckets are long by one row as a rule, and bits of the row
+// do not split it.  low: bits that do not tell entries apart.
 __global__ void bk_list_kernel(const BkDesc *__restrict__ desc, const unsigned *__restrict__ ndesc_dev, unsigned ndesc,
                                int forced, int field, int low, BkSeg *__restrict__ segs, uint2 *__restrict__ tiles,
                                BkCtl *__restrict__ ctl)
@@ -411,7 +413,7 @@ __global__ void bk_list_kernel(const BkDesc *__restrict__ desc, const unsigned *
         } else {
             if (d.count <= (unsigned)BK_CAP || rem <= low) continue;
             const unsigned want = (d.count + BK_SPLIT - 1) / BK_SPLIT;
-            bits = max(32 - __clz(want - 1), rem - field);
+            bits = 32 - __clz(want - 1) + max(0, rem - field);
             bits = min(min(bits, BK_BITS), rem - low);
             gbase = atomicAdd(&ctl->npiece, 1u << bits);
             q = atomicAdd(&ctl->nseg, 1u);
@@ -1106,14 +1108,14 @@ gb_status split(Context *ctx, const Level &lv, const BkDesc *desc, const unsigne
                 int field, int low, int64_t nk, const KIN *in, KOUT *out, cudaStream_t s)
 {
     const int sms = ctx->num_sms;
-    const int64_t most = ndesc_dev ? nk / 512 + 2 : (int64_t)ndesc;
+    const int64_t most = ndesc_dev ? nk / (BK_SPLIT / 2) + 2 : (int64_t)ndesc;
     const int lb = (int)std::max<int64_t>(1, std::min<int64_t>((most + 255) / 256, sms * 4));
     bk_list_kernel<<<lb, 256, 0, s>>>(desc, ndesc_dev, ndesc, forced, field, low, lv.segs, lv.tiles, lv.ctl);
     const int64_t tiles = nk / BK_TILE + 1 + (forced ? (int64_t)ndesc : nk / BK_CAP);
     const int hb = (int)std::min<int64_t>(tiles, sms * 4), pb = (int)std::min<int64_t>(tiles, sms * 2);
     const int64_t nseg = forced ? (int64_t)ndesc : nk / BK_CAP + 1;
     bk_hist_kernel<KIN><<<hb, BK_THREADS, 0, s>>>(in, lv.segs, lv.tiles, lv.ctl, lv.cnt);
-    bk_scan_kernel<<<(int)std::min<int64_t>(nseg, sms * 8), LF_THREADS, 0, s>>>(
+    bk_scan_kernel<<<(int)std::min<int64_t>(nseg, sms * 8), SC_THREADS, 0, s>>>(
         lv.segs, lv.ctl, forced == 0, lv.cnt, lv.cursor, lv.desc);
     constexpr int smem = PartShared<KOUT, sizeof(KIN) != sizeof(KOUT)>::bytes;
     GB_CUDA(smem_limit(bk_part_kernel<KIN, KOUT>, smem));
@@ -1148,10 +1150,11 @@ struct Arena {
 };
 
 // Most pieces of a split of buckets longer than BK_CAP among nk keys, the rows
-// of a bucket numbered by `rowbits` bits: two per BK_SPLIT keys, or a piece a row.
+// of a bucket numbered by `rowbits` bits: two per BK_SPLIT keys and row, BK_BINS a bucket.
 int64_t split_pieces(int64_t nk, int rowbits)
 {
-    return nk / 512 + 2 + ((nk / BK_CAP + 1) << std::max(0, std::min(rowbits, BK_BITS)));
+    const int64_t by_rows = (nk / (BK_SPLIT / 2) + 2) << std::max(0, std::min(rowbits, BK_BITS));
+    return std::min(by_rows, (nk / BK_CAP + 1) * BK_BINS);
 }
 
 struct LevelPlan {
@@ -1201,7 +1204,7 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     const int64_t npos = (nk + POS_TILE - 1) / POS_TILE;
     const int64_t n0 = int64_t(1) << bp.p0, n1 = int64_t(1) << total_bits;
     const int rowbits = std::max(0, scale - total_bits);  // of a bucket after step 1
-    const int64_t seg_x = nk / BK_CAP + 1, desc_x = nk / 512 + 2, tile_x = nk / BK_TILE + 1 + seg_x;
+    const int64_t seg_x = nk / BK_CAP + 1, desc_x = nk / (BK_SPLIT / 2) + 2, tile_x = nk / BK_TILE + 1 + seg_x;
     const int64_t piece2 = split_pieces(nk, rowbits), piece3 = split_pieces(nk, rowbits - BK_BITS);
 
     Arena ar;
@@ -1244,7 +1247,7 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     bk_hist0_kernel<<<(int)std::max<int64_t>(1, std::min<int64_t>(hthreads, sms * 4)), BK_THREADS, 0, s>>>(
         edges, m, scale, bp.p0, cnt0, ctx->status);
     const int rem0 = 2 * scale + LOW - bp.p0;
-    bk_scan0_kernel<<<1, LF_THREADS, 0, s>>>(cnt0, bp.p0, rem0, cur0, desc0, total);
+    bk_scan0_kernel<<<1, SC_THREADS, 0, s>>>(cnt0, bp.p0, rem0, cur0, desc0, total);
     const int64_t tiles0 = (nk + BK_TILE - 1) / BK_TILE;
     const int pb = (int)std::min<int64_t>(tiles0, sms * 2);
     const unsigned limit = (unsigned)nk;
@@ -1381,7 +1384,7 @@ gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, bool *overflow, cu
     const int field = WBITS + g->scale, rem = q + field;
     if (rem > 64) return GB_OK;
     const unsigned nd = (unsigned)((n + (int64_t(1) << q) - 1) >> q);
-    const int64_t seg_x = nnz / BK_CAP + 1, desc_x = nnz / 512 + 2, tile_x = nnz / BK_TILE + 1 + seg_x;
+    const int64_t seg_x = nnz / BK_CAP + 1, desc_x = nnz / (BK_SPLIT / 2) + 2, tile_x = nnz / BK_TILE + 1 + seg_x;
     const int64_t piece2 = split_pieces(nnz, q), piece3 = split_pieces(nnz, q - BK_BITS);
     Arena ar;
     LevelPlan l2 = plan_zeroed(ar, piece2), l3 = plan_zeroed(ar, piece3);
