@@ -87,11 +87,12 @@ void destroy_graph(gb_graph *g)
     for (void *p : arrays)
         if (p) gb::dfree_async(p, nullptr);
     cudaMemPool_t pool;
-    uint64_t held = 0;
+    uint64_t held = 0, used = 0;
     if (cudaDeviceGetDefaultMemPool(&pool, other ? g->device : dev) == cudaSuccess &&
         cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
-        held > gb::kPoolKeep && cudaStreamSynchronize(nullptr) == cudaSuccess)
-        cudaMemPoolTrimTo(pool, gb::kPoolKeep);
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+        held > used + gb::kPoolKeep && cudaStreamSynchronize(nullptr) == cudaSuccess)
+        cudaMemPoolTrimTo(pool, used + gb::kPoolKeep);
     if (other) cudaSetDevice(dev);
     delete g;
 }

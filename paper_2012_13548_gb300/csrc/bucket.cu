@@ -928,10 +928,19 @@ __global__ void __launch_bounds__(PS_THREADS) bk_possum_kernel(const unsigned *_
     }
 }
 
-// base[i] = kept entries before tile i; the total to base[nt].
+// What the host reads once the entries are sorted.
+struct BkResult {
+    unsigned nnz, overflow;
+    DevStatus status;
+};
+
+// base[i] = kept entries before tile i; their total, the last split's overflow flag and
+// the device status to *res.
 __global__ void __launch_bounds__(PS_THREADS) bk_posscan_kernel(const unsigned *__restrict__ cnt, unsigned nt,
                                                                 const unsigned *__restrict__ sums,
-                                                                unsigned *__restrict__ base)
+                                                                unsigned *__restrict__ base,
+                                                                const BkCtl *__restrict__ ctl, const DevStatus *st,
+                                                                BkResult *__restrict__ res)
 {
     __shared__ unsigned s_w[PS_THREADS / 32], s_b[PS_THREADS / 32];
     unsigned before = 0;
@@ -957,7 +966,11 @@ __global__ void __launch_bounds__(PS_THREADS) bk_posscan_kernel(const unsigned *
     for (int j = 0; j < PS_ITEMS; ++j) {
         if (i0 + j < nt) base[i0 + j] = run;
         run += c[j];
-        if (i0 + j + 1 == nt) base[nt] = run;
+        if (i0 + j + 1 == nt) {
+            res->nnz = run;
+            res->overflow = ctl->overflow;
+            res->status = *st;
+        }
     }
 }
 
@@ -1217,7 +1230,8 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     const size_t zeroed = ar.used;
     const size_t o_cur0 = ar.take(BK_BINS * 4);
     const size_t o_desc0 = ar.take(BK_BINS * sizeof(BkDesc));
-    const size_t o_base = ar.take((size_t)npos * 4 + 4);
+    const size_t o_base = ar.take((size_t)npos * 4);
+    const size_t o_res = ar.take(sizeof(BkResult));
     const size_t o_sums = ar.take((size_t)(npos / PS_CHUNK + 1) * 4);
     const size_t o_raw = ar.take((size_t)(n + 1) * 4);
     const size_t o_kept = ar.take((size_t)npos * (POS_TILE / 32) * sizeof(uint2));
@@ -1303,15 +1317,15 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     unsigned *sums = reinterpret_cast<unsigned *>(ws + o_sums), *base = reinterpret_cast<unsigned *>(ws + o_base);
     const unsigned psb = (unsigned)((npos + PS_CHUNK - 1) / PS_CHUNK);
     bk_possum_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums);
-    bk_posscan_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums, base);
+    BkResult *res = reinterpret_cast<BkResult *>(ws + o_res);
+    bk_posscan_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums, base, lv3.ctl, ctx->status, res);
     note_launch(2);
     GB_CUDA(cudaGetLastError());
-    unsigned nnz = 0, ovf = 0;
-    DevStatus hst;
-    GB_CUDA(cudaMemcpyAsync(&nnz, base + npos, sizeof(nnz), cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(&ovf, &lv3.ctl->overflow, sizeof(ovf), cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaMemcpyAsync(&hst, ctx->status, sizeof(hst), cudaMemcpyDeviceToHost, s));
+    BkResult hr;
+    GB_CUDA(cudaMemcpyAsync(&hr, res, sizeof(hr), cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
+    const DevStatus &hst = hr.status;
+    const unsigned nnz = hr.nnz;
     if (hst.code != 0) {
         GB_CUDA(cudaMemsetAsync(ctx->status, 0, sizeof(DevStatus), s));
         set_error(hst.code != GB_ERR_RANGE      ? "graph_build_csr: device error during the build"
@@ -1320,8 +1334,8 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
                                                 : "graph_build_csr: device error during the build");
         return (gb_status)hst.code;
     }
-    *overflow = ovf != 0;
-    if (ovf) return GB_OK;
+    *overflow = hr.overflow != 0;
+    if (hr.overflow) return GB_OK;
     g->nnz = (int64_t)nnz;
     GB_CUDA(gb::dmalloc_async(&g->off, (n + 1) * sizeof(int64_t), s));
     GB_CUDA(gb::dmalloc_async(&g->col, col_alloc_entries(g->nnz) * sizeof(int32_t), s));

@@ -199,152 +199,156 @@ __global__ void __launch_bounds__(FIN_THREADS) k1_write_kernel(
     }
 }
 
-// Bit v of word v/32: row v is not empty.  One warp per word.
-__global__ void nz_bitmap_kernel(const int64_t *__restrict__ off, int64_t n,
-                                 uint32_t *__restrict__ nz, int64_t nw)
-{
-    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const unsigned lane = threadIdx.x & 31u;
-    for (int64_t w = gw; w < nw; w += stride) {
-        const int64_t v = w * 32 + lane;
-        const bool has = v < n && off[v + 1] > off[v];
-        const unsigned b = __ballot_sync(kFull, has);
-        if (lane == 0) nz[w] = b;
-    }
-}
-
 // The list of vertices of degree >= 1 in ascending order (the first
-// bottom-up level of a search walks it instead of the whole visited bitmap):
-// per block of NZL_WORDS bitmap words a count, a scan of the counts, then
-// each block writes its vertices.
-constexpr int NZL_WORDS = 1024;
+// bottom-up level of a search walks it instead of the whole visited bitmap)
+// is written by blocks of NZL_THREADS bitmap words: their counts, a scan
+// of the counts, then the vertices.
+constexpr int NZL_THREADS = 256;
+constexpr int NZL_WARPS = NZL_THREADS / 32;
 
-__global__ void __launch_bounds__(NZL_WORDS) nzl_count_kernel(const uint32_t *__restrict__ nz, int64_t nw,
-                                                             unsigned *__restrict__ cnt)
+// An 8-bit increasing key of the degree: 8 * floor(log2 d) + the next three
+// bits of d, plus one (0 for an empty row).
+__device__ __forceinline__ uint8_t degree_key(int64_t d)
 {
-    __shared__ unsigned s_w[NZL_WORDS / 32];
-    const int64_t w = (int64_t)blockIdx.x * NZL_WORDS + threadIdx.x;
-    const unsigned c = warp_sum(w < nw ? (unsigned)__popc(nz[w]) : 0u);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = c;
+    if (d <= 0) return 0;
+    const int e = 63 - __clzll(d);
+    const unsigned m = e >= 3 ? (unsigned)(d >> (e - 3)) & 7u : (unsigned)(d << (3 - e)) & 7u;
+    return (uint8_t)min((unsigned)e * 8u + m + 1u, 255u);
+}
+
+// One read of the offsets: the degree >= 1 bitmap, the degree keys and, per
+// NZL_THREADS words, the number of vertices of degree >= 1.  A warp per word.
+__global__ void __launch_bounds__(NZL_THREADS) degrees_kernel(const int64_t *__restrict__ off, int64_t n,
+                                                             uint32_t *__restrict__ nz, int64_t nw,
+                                                             uint8_t *__restrict__ key, unsigned *__restrict__ cnt)
+{
+    __shared__ unsigned s_w[NZL_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w0 = (int64_t)blockIdx.x * NZL_THREADS;
+    unsigned c = 0;
+#pragma unroll 4
+    for (int j = 0; j < NZL_THREADS / NZL_WARPS; ++j) {
+        const int64_t w = w0 + warp + (int64_t)j * NZL_WARPS, v = w * 32 + lane;
+        if (w >= nw) break;
+        const int64_t d = v < n ? off[v + 1] - off[v] : 0;
+        const unsigned b = __ballot_sync(kFull, d > 0);
+        if (v < n) key[v] = degree_key(d);
+        if (lane == 0) nz[w] = b;
+        c += __popc(b);
+    }
+    if (lane == 0) s_w[warp] = c;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        const unsigned t = warp_sum(s_w[threadIdx.x]);
-        if (threadIdx.x == 0) cnt[blockIdx.x] = t;
+    if (threadIdx.x == 0) {
+        unsigned t = 0;
+        for (int w = 0; w < NZL_WARPS; ++w) t += s_w[w];
+        cnt[blockIdx.x] = t;
     }
 }
 
-__global__ void __launch_bounds__(NZL_WORDS) nzl_write_kernel(const uint32_t *__restrict__ nz, int64_t nw,
-                                                             const unsigned long long *__restrict__ base,
-                                                             int32_t *__restrict__ list)
+// A warp writes its 32 words' vertices word by word, a lane per bit: whole lines.
+__global__ void __launch_bounds__(NZL_THREADS) nzl_write_kernel(const uint32_t *__restrict__ nz, int64_t nw,
+                                                               const unsigned long long *__restrict__ base,
+                                                               int32_t *__restrict__ list)
 {
-    __shared__ unsigned s_w[NZL_WORDS / 32];
-    const int64_t w = (int64_t)blockIdx.x * NZL_WORDS + threadIdx.x;
-    unsigned bits = w < nw ? nz[w] : 0u;
+    __shared__ unsigned s_w[NZL_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w = (int64_t)blockIdx.x * NZL_THREADS + threadIdx.x;
+    const unsigned bits = w < nw ? nz[w] : 0u;
     const unsigned c = (unsigned)__popc(bits);
     const unsigned incl = warp_inclusive_scan(c);
-    if ((threadIdx.x & 31) == 31) s_w[threadIdx.x >> 5] = incl;
+    if (lane == 31) s_w[warp] = incl;
     __syncthreads();
-    unsigned long long pos = base[blockIdx.x] + incl - c;
-    for (int k = 0; k < (int)(threadIdx.x >> 5); ++k) pos += s_w[k];
-    while (bits) {
-        const int b = __ffs(bits) - 1;
-        bits &= bits - 1;
-        list[pos++] = (int32_t)(w * 32 + b);
-    }
-}
-
-// hd[v] = (hub[v], min(degree(v), 65535)): the bottom-up list walks read both
-// with one 8-byte load instead of a hub load and two 8-byte offsets from
-// other sectors.
-__global__ void hd_kernel(const int64_t *__restrict__ off, const int32_t *__restrict__ hub, int64_t n,
-                          int2 *__restrict__ hd)
-{
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const int64_t d = off[v + 1] - off[v];
-        hd[v] = make_int2(hub[v], (int)(d < 65535 ? d : 65535));
+    unsigned long long pos = base[blockIdx.x];
+    for (int k = 0; k < warp; ++k) pos += s_w[k];
+    const int32_t v0 = (int32_t)((w - lane) * 32) + lane;
+#pragma unroll 4
+    for (int j = 0; j < 32; ++j) {
+        const unsigned bj = __shfl_sync(kFull, bits, j);
+        const unsigned before = __shfl_sync(kFull, incl - c, j);
+        if ((bj >> lane) & 1u) list[pos + before + __popc(bj & lanemask_lt())] = v0 + 32 * j;
     }
 }
 
 constexpr int HUB_THREADS = 256;
-constexpr int64_t HUB_SCAN = 128;  // entries of a row examined for its hub
-
-// An 8-bit increasing key of the degree: 8 * floor(log2 d) + the next three
-// bits of d, plus one (0 for an empty row).
-__global__ void deg_key_kernel(const int64_t *__restrict__ off, int64_t n, uint8_t *__restrict__ key)
-{
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const int64_t d = off[v + 1] - off[v];
-        unsigned k = 0;
-        if (d > 0) {
-            const int e = 63 - __clzll(d);
-            const unsigned m = e >= 3 ? (unsigned)(d >> (e - 3)) & 7u : (unsigned)(d << (3 - e)) & 7u;
-            k = (unsigned)e * 8u + m + 1u;
-            if (k > 255u) k = 255u;
-        }
-        key[v] = (uint8_t)k;
-    }
-}
+constexpr int HUB_SCAN = 128;  // entries of a row examined for its hub
+constexpr int HUB_ROUNDS = 4;  // rounds whose loads are in flight together
 
 // hub[u] = among the first HUB_SCAN neighbours of u (all of them for a shorter
 // row) the one with the largest degree key, the smallest id among equals; -1
 // for an empty row.  The hub is a heuristic (the bottom-up step tests it
 // first), so long rows, whose vertices are reached early anyway, are only
-// sampled: every row costs at most HUB_SCAN entries.  A warp
-// takes 32 rows and streams their edges as one sequence (lane k of a round
-// reads entry k), each edge folded into its row's slot with a shared-memory
-// atomic max of (key << 32 | ~v).
+// sampled: every row costs at most HUB_SCAN entries.  hd[u] = (hub[u], min(degree(u), 65535)): the bottom-up list walks read both with one
+// 8-byte load instead of a hub load and two 8-byte offsets from other sectors.
+// A warp takes 32 rows and streams their edges as one sequence (lane k of a
+// round reads entry k).  Rows ascend, so the smallest id among equal keys is the
+// first of them: (key, 255 - place in the row) fits 16 bits, and a row's
+// greatest is one warp reduction where a round lies in one row, a native
+// 32-bit shared-memory maximum where it does not.
 __global__ void __launch_bounds__(HUB_THREADS) hub_kernel(const int64_t *__restrict__ off,
                                                           const int32_t *__restrict__ col,
                                                           const uint8_t *__restrict__ key, int64_t n,
                                                           int64_t nnz, int32_t *__restrict__ hub,
-                                                          DevStatus *st)
+                                                          int2 *__restrict__ hd, DevStatus *st)
 {
-    __shared__ unsigned long long s_best[HUB_THREADS];
+    __shared__ unsigned s_best[HUB_THREADS];
     const unsigned lane = threadIdx.x & 31u;
     const int wbase = threadIdx.x & ~31;
     const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t r0 = gwarp * 32; r0 < n; r0 += nwarps * 32) {
         const int64_t r = r0 + lane;
-        int64_t s0 = 0, d = 0;
+        int64_t s0 = 0, deg = 0;
         if (r < n) {
             s0 = off[r];
-            d = off[r + 1] - s0;
-            if (d < 0 || s0 < 0 || s0 + d > nnz) d = 0;
-            if (d > HUB_SCAN) d = HUB_SCAN;
+            deg = off[r + 1] - s0;
         }
+        const int d = deg < 0 || s0 < 0 || s0 + deg > nnz ? 0 : (int)(deg < HUB_SCAN ? deg : HUB_SCAN);
         s_best[threadIdx.x] = 0;
         __syncwarp();
-        const int64_t incl = warp_inclusive_scan(d);
-        const int64_t total = __shfl_sync(kFull, incl, 31);
-        const int64_t excl = incl - d;
-        for (int64_t b = 0; b < total; b += 32) {
-            const int64_t k = b + lane;
-            int owner = 0;
+        const int incl = warp_inclusive_scan(d);
+        const int total = __shfl_sync(kFull, incl, 31);
+        const int excl = incl - d;
+        const int64_t at = s0 - excl;  // entry k of the sequence, in this row, is col[at + k]
+        for (int b = 0; b < total; b += 32 * HUB_ROUNDS) {
+            int owner[HUB_ROUNDS], eo[HUB_ROUNDS];
+            int32_t v[HUB_ROUNDS];
 #pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const int cand = owner + step;
-                if (__shfl_sync(kFull, excl, cand) <= k) owner = cand;
+            for (int j = 0; j < HUB_ROUNDS; ++j) {
+                const int k = b + 32 * j + (int)lane;
+                int o = 0;
+#pragma unroll
+                for (int step = 16; step >= 1; step >>= 1)
+                    if (__shfl_sync(kFull, excl, o + step) <= k) o += step;
+                owner[j] = o;
+                const int64_t ao = __shfl_sync(kFull, at, o);
+                eo[j] = __shfl_sync(kFull, excl, o);
+                v[j] = k < total ? col[ao + k] : -1;
             }
-            const int64_t so = __shfl_sync(kFull, s0, owner);
-            const int64_t eo = __shfl_sync(kFull, excl, owner);
-            if (k < total) {
-                const int32_t v = col[so + (k - eo)];
-                if (v >= 0 && v < n) {
-                    const unsigned long long kv = ((unsigned long long)key[v] << 32) |
-                                                  (unsigned long long)(0xffffffffu - (uint32_t)v);
-                    atomicMax(&s_best[wbase + owner], kv);
-                } else {
-                    record_error(st, GB_ERR_RANGE, 12, v);
+            unsigned val[HUB_ROUNDS];
+#pragma unroll
+            for (int j = 0; j < HUB_ROUNDS; ++j) {
+                const int k = b + 32 * j + (int)lane;
+                val[j] = v[j] >= 0 && v[j] < n ? ((unsigned)key[v[j]] << 8) | (unsigned)(255 - (k - eo[j])) : 0u;
+                if (k < total && val[j] == 0) record_error(st, GB_ERR_RANGE, 12, v[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < HUB_ROUNDS; ++j) {
+                if (b + 32 * j >= total) break;
+                if (__shfl_sync(kFull, owner[j], 0) == __shfl_sync(kFull, owner[j], 31)) {
+                    const unsigned m = __reduce_max_sync(kFull, val[j]);
+                    if (lane == 0) s_best[wbase + owner[j]] = max(s_best[wbase + owner[j]], m);
+                } else if (val[j]) {
+                    atomicMax(&s_best[wbase + owner[j]], val[j]);
                 }
+                __syncwarp();
             }
         }
-        __syncwarp();
-        const unsigned long long best = s_best[threadIdx.x];
-        if (r < n) hub[r] = best ? (int32_t)(0xffffffffu - (uint32_t)(best & 0xffffffffull)) : -1;
+        const unsigned best = s_best[threadIdx.x];
+        if (r < n) {
+            const int32_t h = best ? col[s0 + (255 - (int)(best & 255u))] : -1;
+            hub[r] = h;
+            hd[r] = make_int2(h, (int)(deg < 65535 ? deg : 65535));
+        }
         __syncwarp();
     }
 }
@@ -593,42 +597,30 @@ gb_status build_graph_aux(gb_graph *g, cudaStream_t s)
 {
     Context *ctx = context();
     if (!ctx) return GB_ERR_CUDA;
-    const int64_t nw = (g->n + 31) / 32;
-    GB_CUDA(gb::dmalloc_async(&g->nz, nw * sizeof(uint32_t), s));
-    nz_bitmap_kernel<<<ctx->num_sms * 4, 256, 0, s>>>(g->off, g->n, g->nz, nw);
-    note_launch();
-    GB_CUDA(cudaGetLastError());
+    const int64_t n = g->n, nw = (n + 31) / 32, nb = (nw + NZL_THREADS - 1) / NZL_THREADS;
     Scratch tmp(s);
-    {
-        const int64_t nb = (nw + NZL_WORDS - 1) / NZL_WORDS;
-        unsigned *cnt = nullptr;
-        unsigned long long *base = nullptr;
-        GB_CUDA(tmp.alloc(&cnt, (size_t)nb));
-        GB_CUDA(tmp.alloc(&base, (size_t)nb + 1));
-        nzl_count_kernel<<<(unsigned)nb, NZL_WORDS, 0, s>>>(g->nz, nw, cnt);
-        note_launch();
-        k1_scan_tiles_kernel<<<1, 1024, 0, s>>>(cnt, nb, base);
-        note_launch();
-        GB_CUDA(cudaGetLastError());
-        unsigned long long nnzv = 0;
-        GB_CUDA(cudaMemcpyAsync(&nnzv, base + nb, sizeof(nnzv), cudaMemcpyDeviceToHost, s));
-        GB_CUDA(cudaStreamSynchronize(s));
-        g->nnzv = (int64_t)nnzv;
-        GB_CUDA(gb::dmalloc_async(&g->nzl, std::max<int64_t>(g->nnzv, 4) * sizeof(int32_t), s));
-        nzl_write_kernel<<<(unsigned)nb, NZL_WORDS, 0, s>>>(g->nz, nw, base, g->nzl);
-        note_launch();
-        GB_CUDA(cudaGetLastError());
-    }
-    GB_CUDA(gb::dmalloc_async(&g->hub, std::max<int64_t>(g->n, 1) * sizeof(int32_t), s));
+    unsigned *cnt = nullptr;
+    unsigned long long *base = nullptr;
     uint8_t *key = nullptr;
-    GB_CUDA(tmp.alloc(&key, (size_t)g->n));
-    deg_key_kernel<<<ctx->num_sms * 4, 256, 0, s>>>(g->off, g->n, key);
-    note_launch();
-    hub_kernel<<<ctx->num_sms * 8, HUB_THREADS, 0, s>>>(g->off, g->col, key, g->n, g->nnz, g->hub,
-                                                        ctx->status);
-    note_launch();
-    GB_CUDA(gb::dmalloc_async(&g->hd, std::max<int64_t>(g->n, 1) * sizeof(int2), s));
-    hd_kernel<<<ctx->num_sms * 8, 256, 0, s>>>(g->off, g->hub, g->n, g->hd);
+    GB_CUDA(gb::dmalloc_async(&g->nz, nw * sizeof(uint32_t), s));
+    GB_CUDA(gb::dmalloc_async(&g->hub, std::max<int64_t>(n, 1) * sizeof(int32_t), s));
+    GB_CUDA(gb::dmalloc_async(&g->hd, std::max<int64_t>(n, 1) * sizeof(int2), s));
+    GB_CUDA(tmp.alloc(&cnt, (size_t)nb));
+    GB_CUDA(tmp.alloc(&base, (size_t)nb + 1));
+    GB_CUDA(tmp.alloc(&key, (size_t)n));
+    degrees_kernel<<<(unsigned)nb, NZL_THREADS, 0, s>>>(g->off, n, g->nz, nw, key, cnt);
+    k1_scan_tiles_kernel<<<1, 1024, 0, s>>>(cnt, nb, base);
+    // several waves of blocks: rows differ in length
+    const unsigned hb = (unsigned)std::min<int64_t>((n + HUB_THREADS - 1) / HUB_THREADS, (int64_t)ctx->num_sms * 64);
+    hub_kernel<<<hb, HUB_THREADS, 0, s>>>(g->off, g->col, key, n, g->nnz, g->hub, g->hd, ctx->status);
+    note_launch(3);
+    GB_CUDA(cudaGetLastError());
+    unsigned long long nnzv = 0;
+    GB_CUDA(cudaMemcpyAsync(&nnzv, base + nb, sizeof(nnzv), cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaStreamSynchronize(s));
+    g->nnzv = (int64_t)nnzv;
+    GB_CUDA(gb::dmalloc_async(&g->nzl, std::max<int64_t>(g->nnzv, 4) * sizeof(int32_t), s));
+    nzl_write_kernel<<<(unsigned)nb, NZL_THREADS, 0, s>>>(g->nz, nw, base, g->nzl);
     note_launch();
     GB_CUDA(cudaGetLastError());
     return GB_OK;

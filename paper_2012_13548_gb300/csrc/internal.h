@@ -78,7 +78,7 @@ inline cudaError_t dmalloc_async(T **p, size_t bytes, cudaStream_t s)
 // cudaFree map and unmap memory and wait for the device each time: a SCALE 16 build
 // took 554 us, of which its kernels 230.  What the pool keeps between graphs
 // is bounded: graph_free returns what exceeds kPoolKeep to the device.
-constexpr uint64_t kPoolKeep = uint64_t(48) << 30;  // a SCALE 26 build's temporaries and graph
+constexpr uint64_t kPoolKeep = uint64_t(48) << 30;  // unused bytes: a SCALE 26 build and its graph take 40 GB
 
 // Stream-ordered temporaries.
 template <typename T>
