@@ -210,10 +210,14 @@ gb_status graph_prepare_batched(gb_graph *g, gb_stream s);
  *   alpha, beta        direction switch: top-down -> bottom-up when the
  *                      frontier's edges exceed (unexplored edges)/alpha;
  *                      bottom-up -> top-down when the frontier shrinks below
- *                      n/beta vertices (Beamer et al., SC 2012).
+ *                      n/beta vertices (Beamer et al., SC 2012).  A
+ *                      frontier of hubs (16 times the mean degree) switches
+ *                      at up to four times that ratio, at most 64.
  *   big_degree         frontier vertices of larger degree are split over the
  *                      whole grid in top-down steps.
- *   ms_alpha, ms_beta  the same switch for the multi-source BFS.
+ *   ms_alpha, ms_beta  the same switch for the multi-source BFS, on all edges
+ *                      of the graph; where its masks fit the L2 it stays
+ *                      top-down up to four times as many edges (to a ratio of 4).
  *   timeout_ms         limit of every device-side wait (grid barriers, the
  *                      radix-sort look-back); on expiry the kernel records
  *                      GB_ERR_TIMEOUT and returns.

@@ -99,7 +99,9 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned &target, DevS
                 ok = 0;
                 break;
             }
-            if ((++spins & 31u) == 0) {
+            // the clock from the first poll on, every eighth: a poll is an L2 round
+            // trip, so a limit below a few microseconds runs out within them
+            if ((++spins & 7u) == 1) {
                 const uint64_t now = globaltimer_ns();
                 if (t0 == 0) {
                     t0 = now;
