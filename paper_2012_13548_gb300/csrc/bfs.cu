@@ -515,6 +515,68 @@ __device__ __noinline__ void canonical_rescan(const BfsArgs &a, const unsigned *
     }
 }
 
+// The same by the other end of the edges: every edge of the previous level's frontier
+// (queue entries [qb, qb + qn), big vertices bb.. in nc chunks) once more, each
+// neighbour that the level claimed (a bit of F) keeping the least of the frontier
+// vertices that reach it.  The choice is by edges: a few vertices next to
+// the root claim the hubs, whose rows hold a thousand times as many entries
+// (SCALE 26: 7 vertices claimed 159,420 with 1.3 G entries; scanned row by
+// row, the longest by one warp, the search took 9.1 ms, by the frontier's edges 1.8), while
+// a wide frontier's last claims have short rows.
+__device__ __noinline__ void canonical_edges(const BfsArgs &a, const unsigned *F, int64_t qb, int64_t qn, int64_t bb,
+                                             int64_t nb, int64_t nc, int64_t gwarp, int64_t nwarps)
+{
+    const int lane = (int)lane_id();
+    const auto edge = [&](int64_t j, int32_t u) {
+        if (!GB_OK_IDX(a.st, j, a.nnz, 228)) return;
+        const int32_t v = __ldg(&a.col[j]);
+        if (!GB_OK_IDX(a.st, v, a.n, 229)) return;
+        if (((__ldcg(&F[(unsigned)v >> 5]) >> (v & 31)) & 1u) && ldcg_i32(&a.parent[v]) > u) atomicMin(&a.parent[v], u);
+    };
+    for (int64_t c = gwarp; c < nc; c += nwarps) {
+        int64_t lo = 0, hi = nb;  // largest i with cbase(i) <= c
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) >> 1;
+            if ((int64_t)load_big(a.bigq, bb + mid).cbase <= c) lo = mid;
+            else hi = mid;
+        }
+        const BigEnt be = load_big(a.bigq, bb + lo);
+        if (!GB_OK_IDX(a.st, be.u, a.n, 230)) continue;
+        const int64_t su = a.off[be.u], eu = a.off[be.u + 1];
+        const int64_t cs = (su & ~int64_t(3)) + (c - (int64_t)be.cbase) * BIG_CHUNK;
+        const int64_t e = cs + BIG_CHUNK < eu ? cs + BIG_CHUNK : eu;
+        for (int64_t j = cs + lane; j < e; j += 32)
+            if (j >= su) edge(j, be.u);
+    }
+    for (int64_t i0 = gwarp * 32; i0 < qn; i0 += nwarps * 32) {
+        const int64_t i = i0 + lane;
+        int32_t u = 0;
+        int64_t s = 0, d = 0;
+        if (i < qn && GB_OK_IDX(a.st, qb + i, a.n, 231)) {
+            u = ldcg_i32(&a.queue[qb + i]);
+            if (!GB_OK_IDX(a.st, u, a.n, 232)) u = 0;
+            s = a.off[u];
+            d = a.off[u + 1] - s;
+            if (d > a.big_deg) d = 0;
+        }
+        const int64_t incl = warp_inclusive_scan(d);
+        const int64_t total = __shfl_sync(kFull, incl, 31);
+        const int64_t excl = incl - d;
+        for (int64_t b = 0; b < total; b += 32) {
+            const int64_t k = b + lane;
+            int owner = 0;
+#pragma unroll
+            for (int step = 16; step >= 1; step >>= 1) {
+                const int64_t ex = __shfl_sync(kFull, excl, owner + step);
+                if (ex <= k) owner += step;
+            }
+            const int32_t su = __shfl_sync(kFull, u, owner);
+            const int64_t so = __shfl_sync(kFull, s, owner), eo = __shfl_sync(kFull, excl, owner);
+            if (k < total) edge(so + (k - eo), su);
+        }
+    }
+}
+
 // Shared memory of solo_levels (laid over the warp buffers, which are empty
 // between levels): the frontier being expanded and the one being filled, each
 // vertex with its row start and degree, the exclusive prefix of the degrees,
@@ -874,6 +936,8 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
     double mu = (double)a.nnz;
     bool td = true, prev_td = true;
     bool rescan = false;  // canonical mode: the frontier was claimed by a grid-wide top-down level
+    double prev_mf = 0;   // that level's edges and big vertices
+    int64_t prev_nb = 0, prev_nc = 0;
     unsigned long long my_edges = 0, my_touched = 0;
     int l = 0;
     // ring position of the level's bitmaps and control record: one step per
@@ -917,7 +981,10 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
         }
 
         // Canonical parents of vertices claimed top-down at level l-1.
-        if (rescan) canonical_rescan(a, Fp, qbase, qn, gwarp, nwarps);
+        if (rescan) {
+            if (prev_mf < mf) canonical_edges(a, F, qbase - prev_qn, prev_qn, bbase - prev_nb, prev_nb, prev_nc, gwarp, nwarps);
+            else canonical_rescan(a, Fp, qbase, qn, gwarp, nwarps);
+        }
 
         // Narrow levels: block 0 runs them alone, the others wait.
         if (td && qn <= SOLO_Q && (mf <= (double)SOLO_E || (mf <= (double)SOLO_E_SHORT && mf <= 4.0 * (double)qn))) {
@@ -1195,6 +1262,9 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
         }
         prev_td = td;
         rescan = td && a.canonical;
+        prev_mf = mf;
+        prev_nb = nb;
+        prev_nc = nc;
         prev_qn = qn;
         qbase += qn;
         bbase += nb;
