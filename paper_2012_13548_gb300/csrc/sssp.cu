@@ -27,10 +27,11 @@
 //     edges, which can only produce distances >= T) is relaxed once, with
 //     the final dist(u).  A vertex expanded again after its distance dropped
 //     re-reads only its light prefix;
-//   * rows longer than SP_BIG are cut into SP_CHUNK-edge chunks that all warps
-//     share (a chunk tests each edge against the split itself); shorter rows
-//     find their split by bisection and are expanded 32 per warp as one
-//     stream of edges;
+//   * rows longer than SP_BIG are cut into chunks that all warps share (their light
+//     prefix by SP_LIGHT edges, whole rows by SP_CHUNK); shorter rows find
+//     their split and are expanded up to 32 per warp as one stream of edges;
+//   * a settle step reads the heavy edges from whichever end has fewer: the
+//     settled rows, or the rows of what is still unsettled (pull_settle);
 //   * a relaxation that lowers dist(v) also writes u as v's parent (a plain
 //     store: racing winners may leave a parent that is no longer tight);
 //   * after the last bucket the kernel writes the distances as doubles and the
@@ -41,9 +42,10 @@
 //
 // Kernel 1's weights: graph_build_csr_weighted builds the CSR as kernel 1 does
 // and then gives each entry the least weight among the tuples joining its pair
-// (each tuple finds its two entries by bisection of the sorted rows); the
-// weight-sorted rows come from one radix sort of (row << 25 | weight) keys
-// carrying the columns (stable, so equal weights keep ascending columns).
+// (the bucket sort of bucket.cu carries the weight below the key, and sorts the rows
+// once more by weight; where it does not serve, each tuple finds its two entries by
+// bisection of the sorted rows and the weight-sorted rows come from one radix sort of
+// (row << 25 | weight) keys carrying the columns).
 #include "bucket.h"
 #include "common.cuh"
 #include "internal.h"
@@ -59,6 +61,7 @@ constexpr int SP_THREADS = 512;
 constexpr int SP_MINB = 2;
 constexpr int64_t SP_BIG = 1024;   // longer rows are expanded in chunks by all warps
 constexpr int64_t SP_CHUNK = 256;  // edges per chunk
+constexpr int64_t SP_LIGHT = 128;  // edges per chunk of a light prefix
 constexpr unsigned long long SP_INF = ~0ull;
 constexpr double kUnit = 5.9604644775390625e-8;  // 2^-24: one weight unit
 constexpr int SITE_SP_BAR = 40, SITE_SP_NEAR = 41, SITE_SP_FAR = 42, SITE_SP_BIGQ = 43,
@@ -160,6 +163,9 @@ struct SpHeader {
     unsigned long long farcnt[2];  // far list sizes, by epoch parity
     SpQueueCtl q[4];               // near queue counters, by queue id mod 4
     SpQueueCtl settle;             // vertices expanded in the current bucket
+    unsigned long long light[2];   // (big rows << 32) | chunks of their light prefixes, by queue parity
+    unsigned long long sdeg;       // degrees of all vertices settled so far, this bucket's included
+    unsigned long long open[2];    // lengths of the pull steps' lists, by parity
     unsigned long long acc[4];     // processed, scanned, won, reached
 };
 
@@ -177,7 +183,9 @@ struct SpArgs {
     int32_t *nq;               // 2 near queues of n
     int32_t *fq;               // 2 far lists of n
     int32_t *sq;               // the settle list of n
-    SpBig *bq;                 // 2 big-row lists of bigcap, then the settle list's
+    int32_t *open;             // 2 lists of n: the vertices that pull steps left unsettled
+    int64_t nnz;
+    SpBig *bq;                 // 2 big-row lists of bigcap, the settle list's, the light prefixes'
     int64_t bigcap;
     SpHeader *hdr;
     DevStatus *st;
@@ -200,61 +208,115 @@ __device__ __forceinline__ SpBig load_spbig(const SpBig *q, int64_t i)
     return b;
 }
 
-// Warp-collective: the lanes with `want` append v to near queue `qid`; a row
-// longer than SP_BIG is also listed with its chunks.
-__device__ __forceinline__ void push_near(const SpArgs &a, unsigned qid, bool want, int32_t v)
+// What a warp lists (near, far, settled vertices) is staged in shared memory
+// and moved to the lists SP_STAGE entries at a time: the lists' counters are
+// three addresses, and with an atomic per step of 64 edges they were what the large
+// rounds waited for (SCALE 22, delta 0.05: rounds 2.9 -> 2.5 ms, settle steps
+// 1.1 -> 0.8, far splits 0.73 -> 0.43).
+constexpr int SP_STAGE = 96;
+struct SpWarp {
+    int32_t near[SP_STAGE], far[SP_STAGE], settle[SP_STAGE];
+};
+struct SpFill {  // warp-uniform fill levels, and the degrees of the lane's staged settled vertices
+    int near = 0, far = 0, settle = 0;
+    unsigned long long deg = 0;
+};
+
+// Warp-collective: list `n` staged vertices at *cnt of `list`.
+__device__ __forceinline__ int64_t stage_base(unsigned long long *cnt, int n)
 {
-    const unsigned m = __ballot_sync(kFull, want);
-    if (!m) return;
-    const unsigned lane = lane_id();
-    const int leader = __ffs(m) - 1;
     unsigned long long base = 0;
-    if ((int)lane == leader) base = atomicAdd(&a.hdr->q[qid & 3].cnt, (unsigned long long)__popc(m));
-    base = __shfl_sync(kFull, base, leader);
-    if (!want) return;
-    const int64_t pos = (int64_t)base + __popc(m & lanemask_lt());
-    if (pos < a.n) a.nq[(int64_t)(qid & 1) * a.n + pos] = v;
-    else record_error(a.st, GB_ERR_RANGE, SITE_SP_NEAR, pos);
-    const int64_t d = a.off[v + 1] - a.off[v];
-    if (d > SP_BIG) {
-        const unsigned nch = (unsigned)((d + SP_CHUNK - 1) / SP_CHUNK);
-        const unsigned long long old = atomicAdd(&a.hdr->q[qid & 3].big, (1ull << 32) | nch);
-        const int64_t bi = (int64_t)(old >> 32);
-        if (bi < a.bigcap) {
-            const unsigned long long r = (unsigned long long)(uint32_t)v | ((old & 0xffffffffull) << 32);
-            reinterpret_cast<unsigned long long *>(a.bq)[(int64_t)(qid & 1) * a.bigcap + bi] = r;
-        } else {
-            record_error(a.st, GB_ERR_RANGE, SITE_SP_BIGQ, bi);
-        }
-    }
+    __syncwarp();
+    if (lane_id() == 0) base = atomicAdd(cnt, (unsigned long long)n);
+    return (int64_t)__shfl_sync(kFull, base, 0);
 }
 
-// Warp-collective: the lanes with `want` append v to the settle list of the
-// current bucket (a row longer than SP_BIG also with its chunks).
-__device__ __forceinline__ void push_settle(const SpArgs &a, bool want, int32_t v, int64_t d)
+// A row longer than SP_BIG is also listed with its chunks.
+__device__ __forceinline__ void list_big(const SpArgs &a, SpQueueCtl *q, SpBig *bq, int32_t v, int64_t d)
+{
+    if (d <= SP_BIG) return;
+    const unsigned nch = (unsigned)((d + SP_CHUNK - 1) / SP_CHUNK);
+    const unsigned long long old = atomicAdd(&q->big, (1ull << 32) | nch);
+    const int64_t bi = (int64_t)(old >> 32);
+    if (bi < a.bigcap)
+        reinterpret_cast<unsigned long long *>(bq)[bi] = (unsigned long long)(uint32_t)v | ((old & 0xffffffffull) << 32);
+    else record_error(a.st, GB_ERR_RANGE, SITE_SP_BIGQ, bi);
+}
+
+__device__ __forceinline__ void flush_near(const SpArgs &a, SpWarp &wb, SpFill &f, unsigned qid)
+{
+    if (f.near == 0) return;
+    SpQueueCtl *q = &a.hdr->q[qid & 3];
+    const int64_t base = stage_base(&q->cnt, f.near);
+    for (int i = lane_id(); i < f.near; i += 32) {
+        const int32_t v = wb.near[i];
+        if (base + i < a.n) a.nq[(int64_t)(qid & 1) * a.n + base + i] = v;
+        else record_error(a.st, GB_ERR_RANGE, SITE_SP_NEAR, base + i);
+        list_big(a, q, a.bq + (int64_t)(qid & 1) * a.bigcap, v, a.off[v + 1] - a.off[v]);
+    }
+    __syncwarp();
+    f.near = 0;
+}
+
+__device__ __forceinline__ void flush_far(const SpArgs &a, SpWarp &wb, SpFill &f, unsigned epoch)
+{
+    if (f.far == 0) return;
+    const int64_t base = stage_base(&a.hdr->farcnt[epoch & 1], f.far);
+    for (int i = lane_id(); i < f.far; i += 32) {
+        if (base + i < a.n) a.fq[(int64_t)(epoch & 1) * a.n + base + i] = wb.far[i];
+        else record_error(a.st, GB_ERR_RANGE, SITE_SP_FAR, base + i);
+    }
+    __syncwarp();
+    f.far = 0;
+}
+
+__device__ __forceinline__ void flush_settle(const SpArgs &a, SpWarp &wb, SpFill &f)
+{
+    if (f.settle == 0) return;
+    const unsigned long long d = warp_sum(f.deg);
+    if (lane_id() == 0) atomicAdd(&a.hdr->sdeg, d);
+    const int64_t base = stage_base(&a.hdr->settle.cnt, f.settle);
+    for (int i = lane_id(); i < f.settle; i += 32) {
+        const int32_t v = wb.settle[i];
+        if (base + i < a.n) a.sq[base + i] = v;
+        else record_error(a.st, GB_ERR_RANGE, SITE_SP_NEAR, base + i);
+        list_big(a, &a.hdr->settle, a.bq + 2 * a.bigcap, v, a.off[v + 1] - a.off[v]);
+    }
+    __syncwarp();
+    f.settle = 0;
+    f.deg = 0;
+}
+
+// Warp-collective: the lanes with `want` list v in near queue `qid`, in the far
+// list of `epoch`, or in the settle list of the current bucket.
+__device__ __forceinline__ void push_near(const SpArgs &a, SpWarp &wb, SpFill &f, unsigned qid, bool want, int32_t v)
 {
     const unsigned m = __ballot_sync(kFull, want);
     if (!m) return;
-    const unsigned lane = lane_id();
-    const int leader = __ffs(m) - 1;
-    unsigned long long base = 0;
-    if ((int)lane == leader) base = atomicAdd(&a.hdr->settle.cnt, (unsigned long long)__popc(m));
-    base = __shfl_sync(kFull, base, leader);
-    if (!want) return;
-    const int64_t pos = (int64_t)base + __popc(m & lanemask_lt());
-    if (pos < a.n) a.sq[pos] = v;
-    else record_error(a.st, GB_ERR_RANGE, SITE_SP_NEAR, pos);
-    if (d > SP_BIG) {
-        const unsigned nch = (unsigned)((d + SP_CHUNK - 1) / SP_CHUNK);
-        const unsigned long long old = atomicAdd(&a.hdr->settle.big, (1ull << 32) | nch);
-        const int64_t bi = (int64_t)(old >> 32);
-        if (bi < a.bigcap) {
-            const unsigned long long r = (unsigned long long)(uint32_t)v | ((old & 0xffffffffull) << 32);
-            reinterpret_cast<unsigned long long *>(a.bq)[2 * a.bigcap + bi] = r;
-        } else {
-            record_error(a.st, GB_ERR_RANGE, SITE_SP_BIGQ, bi);
-        }
+    if (f.near + __popc(m) > SP_STAGE) flush_near(a, wb, f, qid);
+    if (want) wb.near[f.near + __popc(m & lanemask_lt())] = v;
+    f.near += __popc(m);
+}
+
+__device__ __forceinline__ void push_far(const SpArgs &a, SpWarp &wb, SpFill &f, unsigned epoch, bool want, int32_t v)
+{
+    const unsigned m = __ballot_sync(kFull, want);
+    if (!m) return;
+    if (f.far + __popc(m) > SP_STAGE) flush_far(a, wb, f, epoch);
+    if (want) wb.far[f.far + __popc(m & lanemask_lt())] = v;
+    f.far += __popc(m);
+}
+
+__device__ __forceinline__ void push_settle(const SpArgs &a, SpWarp &wb, SpFill &f, bool want, int32_t v, int64_t d)
+{
+    const unsigned m = __ballot_sync(kFull, want);
+    if (!m) return;
+    if (f.settle + __popc(m) > SP_STAGE) flush_settle(a, wb, f);
+    if (want) {
+        wb.settle[f.settle + __popc(m & lanemask_lt())] = v;
+        f.deg += (unsigned long long)d;
     }
+    f.settle += __popc(m);
 }
 
 // The weight-sorted rows are a stream (each entry read about once by a light
@@ -277,10 +339,29 @@ __device__ __forceinline__ uint2 ld_stream(const uint2 *p, uint64_t pol)
     return r;
 }
 
-// First index j in [lo, hi) of a weight-sorted row with weight >= lim (hi if none).
+// First index j in [lo, hi) of a weight-sorted row with weight >= lim (hi if
+// none).  A light prefix is short (delta of a row's entries), so the first four
+// entries are read together and only a longer prefix is searched, in doubling steps
+// from there: one memory latency for most rows, where bisecting
+// the row took six, each in a sector of its own.
 __device__ __forceinline__ int64_t weight_split(const uint2 *__restrict__ wadj, int64_t lo, int64_t hi,
                                                 unsigned long long lim)
 {
+    unsigned y[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) y[t] = lo + t < hi ? wadj[lo + t].y : 0xffffffffu;
+    int c = 0;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) c += (unsigned long long)y[t] < lim && lo + t < hi;
+    lo += c;
+    if (c < 4) return lo;
+    for (int64_t step = 4; lo + step < hi; step *= 2) {
+        if ((unsigned long long)wadj[lo + step].y >= lim) {
+            hi = lo + step;
+            break;
+        }
+        lo += step + 1;
+    }
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
         if ((unsigned long long)wadj[mid].y < lim) lo = mid + 1;
@@ -301,28 +382,12 @@ __device__ __forceinline__ SpBig find_chunk(const SpBig *B, int64_t nb, int64_t 
     return load_spbig(B, lo);
 }
 
-// Warp-collective: the lanes with `want` append v to the far list of `epoch`.
-__device__ __forceinline__ void push_far(const SpArgs &a, unsigned epoch, bool want, int32_t v)
-{
-    const unsigned m = __ballot_sync(kFull, want);
-    if (!m) return;
-    const unsigned lane = lane_id();
-    const int leader = __ffs(m) - 1;
-    unsigned long long base = 0;
-    if ((int)lane == leader) base = atomicAdd(&a.hdr->farcnt[epoch & 1], (unsigned long long)__popc(m));
-    base = __shfl_sync(kFull, base, leader);
-    if (!want) return;
-    const int64_t pos = (int64_t)base + __popc(m & lanemask_lt());
-    if (pos < a.n) a.fq[(int64_t)(epoch & 1) * a.n + pos] = v;
-    else record_error(a.st, GB_ERR_RANGE, SITE_SP_FAR, pos);
-}
-
 // Warp-collective relaxation of one edge per lane whose distance test has
 // been made: dist(v) lowered to nd if still smaller; a lowered v is queued
 // near (nd < T) or listed far.
 __device__ __forceinline__ void relax_tail(const SpArgs &a, bool cand, int32_t u, int32_t v,
                                            unsigned long long nd, unsigned long long T, unsigned qnext,
-                                           unsigned epoch, unsigned long long &won)
+                                           unsigned epoch, unsigned long long &won, SpWarp &wb, SpFill &f)
 {
     bool to_near = false, to_far = false;
     if (cand) {
@@ -334,8 +399,8 @@ __device__ __forceinline__ void relax_tail(const SpArgs &a, bool cand, int32_t u
             else to_far = atomicExch(&a.fstamp[v], epoch) != epoch;
         }
     }
-    push_near(a, qnext, to_near, v);
-    push_far(a, epoch, to_far, v);
+    push_near(a, wb, f, qnext, to_near, v);
+    push_far(a, wb, f, epoch, to_far, v);
 }
 
 // Two edges per lane: both endpoint distances are read before either atomic,
@@ -343,13 +408,13 @@ __device__ __forceinline__ void relax_tail(const SpArgs &a, bool cand, int32_t u
 __device__ __forceinline__ void relax2(const SpArgs &a, bool ok0, int32_t u0, uint2 c0,
                                        unsigned long long d0, bool ok1, int32_t u1, uint2 c1,
                                        unsigned long long d1, unsigned long long T, unsigned qnext,
-                                       unsigned epoch, unsigned long long &won)
+                                       unsigned epoch, unsigned long long &won, SpWarp &wb, SpFill &f)
 {
     const unsigned long long nd0 = d0 + c0.y, nd1 = d1 + c1.y;
     const unsigned long long cur0 = ok0 ? __ldcg(&a.dist[c0.x]) : 0ull;
     const unsigned long long cur1 = ok1 ? __ldcg(&a.dist[c1.x]) : 0ull;
-    relax_tail(a, ok0 && nd0 < cur0, u0, (int32_t)c0.x, nd0, T, qnext, epoch, won);
-    relax_tail(a, ok1 && nd1 < cur1, u1, (int32_t)c1.x, nd1, T, qnext, epoch, won);
+    relax_tail(a, ok0 && nd0 < cur0, u0, (int32_t)c0.x, nd0, T, qnext, epoch, won, wb, f);
+    relax_tail(a, ok1 && nd1 < cur1, u1, (int32_t)c1.x, nd1, T, qnext, epoch, won, wb, f);
 }
 
 // The row of stream slot k of a warp's 32-row edge stream (the lane whose
@@ -365,13 +430,24 @@ __device__ __forceinline__ int stream_owner(int64_t excl, int64_t k)
     return owner;
 }
 
+// How many of `cnt` rows a warp takes at a time: 32 if there are enough for every
+// warp, else fewer, so that all warps take part.  A step of a stream is a chain of
+// five memory latencies (entry, distance, minimum, stamp, queue), and a
+// round lasts as long as its longest warp: 32 rows of up to 1024 entries in
+// one warp while most had none took most of a round's time.
+__device__ __forceinline__ int rows_per_warp(int64_t cnt, int64_t nwarps)
+{
+    const int64_t r = (cnt + nwarps - 1) / nwarps;
+    return r > 32 ? 32 : (int)r;
+}
+
 // Warp-collective: relax the edges [so + (k - eo)] of a 32-row stream of
 // `total` slots (row starts s0, exclusive prefixes excl, distances du, ids u),
 // two slots per lane per step.
 __device__ __forceinline__ void relax_stream(const SpArgs &a, uint64_t pol, int64_t total, int64_t s0,
                                              int64_t excl, unsigned long long du, int32_t u,
                                              unsigned long long T, unsigned qnext, unsigned epoch,
-                                             unsigned long long &won)
+                                             unsigned long long &won, SpWarp &wb, SpFill &f)
 {
     const unsigned lane = lane_id();
     for (int64_t b = 0; b < total; b += 64) {
@@ -385,8 +461,133 @@ __device__ __forceinline__ void relax_stream(const SpArgs &a, uint64_t pol, int6
         uint2 c0 = make_uint2(0u, 0u), c1 = make_uint2(0u, 0u);
         if (ok0) c0 = ld_stream(a.wadj + so0 + (k0 - eo0), pol);
         if (ok1) c1 = ld_stream(a.wadj + so1 + (k1 - eo1), pol);
-        relax2(a, ok0, u0, c0, du0, ok1, u1, c1, du1, T, qnext, epoch, won);
+        relax2(a, ok0, u0, c0, du0, ok1, u1, c1, du1, T, qnext, epoch, won, wb, f);
     }
+}
+
+// A settle step from the other end of the heavy edges: every vertex v that is
+// still unsettled looks among its neighbours for the ones below T.  Rows are
+// weight-sorted and weights symmetric, the vertices settled before this bucket have reached v
+// already, and those of this bucket have dist >= L, so only the prefix of v's row
+// with w < dist(v) - L can lower it, and the bound shrinks with every hit.  Once the hubs
+// are settled what is left unsettled has short rows, while the settled rows
+// hold nearly all edges and nearly none of them lowers anything: SCALE 22,
+// delta 0.05, settle steps by rows of the settled vertices only 3.3 ms of
+// 7.9, with this choice 0.8 of 4.1.
+// ids: the list of `cnt` vertices, or null for all of them; what stays
+// unsettled goes to `out`.  Only this warp's lane touches dist(v) here, and
+// settled distances are final: no atomics but the lists' counters.
+constexpr int SP_PULL_LANE = 64;  // entries that a lane reads by itself before its warp takes the rest over
+__device__ __noinline__ void pull_settle(const SpArgs &a, const int32_t *ids, int64_t cnt, int32_t *out,
+                                         unsigned long long *out_cnt, unsigned long long T, unsigned long long L,
+                                         unsigned epoch, int64_t gwarp, int64_t nwarps, unsigned long long &scanned,
+                                         unsigned long long &won, SpWarp &wb)
+{
+    const unsigned lane = lane_id();
+    const int rw = rows_per_warp(cnt, nwarps);
+    SpFill f;  // far: lowered vertices; near: the next list's entries
+    const auto flush_open = [&]() {
+        if (f.near == 0) return;
+        const int64_t base = stage_base(out_cnt, f.near);
+        for (int i = lane; i < f.near; i += 32) {
+            if (base + i < a.n) __stcg(&out[base + i], wb.near[i]);
+            else record_error(a.st, GB_ERR_RANGE, SITE_SP_FAR, base + i);
+        }
+        __syncwarp();
+        f.near = 0;
+    };
+    for (int64_t i0 = gwarp * rw; i0 < cnt; i0 += nwarps * rw) {
+        const int64_t i = i0 + lane;
+        int32_t v = 0, par = 0;
+        unsigned long long best = 0, old = 0;
+        int64_t j = 0, re = 0;
+        bool open = false;
+        if ((int)lane < rw && i < cnt) {
+            v = ids ? __ldcg(&ids[i]) : (int32_t)i;
+            old = best = __ldcg(&a.dist[v]);
+            if (best >= T) {
+                j = a.off[v];
+                re = a.off[v + 1];
+                open = re > j;
+            }
+        }
+        const unsigned m = __ballot_sync(kFull, open);
+        if (!m) continue;
+        if (f.near + __popc(m) > SP_STAGE) flush_open();
+        if (open) wb.near[f.near + __popc(m & lanemask_lt())] = v;
+        f.near += __popc(m);
+        // four entries at a time: their weights, then the distances of those in reach
+        bool more = open;
+        const int64_t jl = j + SP_PULL_LANE < re ? j + SP_PULL_LANE : re;
+        while (more && j < jl) {
+            uint2 c[4];
+            unsigned long long du[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) c[t] = j + t < jl ? a.wadj[j + t] : make_uint2(0u, 0xffffffffu);
+            const unsigned long long lim = best - L;  // best >= T > L
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const bool in = c[t].y != 0xffffffffu && (unsigned long long)c[t].y < lim;
+                du[t] = in ? __ldcg(&a.dist[c[t].x]) : SP_INF;
+                scanned += in;
+                more = more && (in || c[t].y == 0xffffffffu);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                if (du[t] < T && du[t] + c[t].y < best) {
+                    best = du[t] + c[t].y;
+                    par = (int32_t)c[t].x;
+                }
+            }
+            j += 4;
+        }
+        // long rows: the warp in rounds of 32 entries
+        unsigned longm = __ballot_sync(kFull, more && j < re);
+        while (longm) {
+            const int src = __ffs(longm) - 1;
+            longm &= longm - 1;
+            int64_t k0 = __shfl_sync(kFull, j, src);
+            const int64_t e = __shfl_sync(kFull, re, src);
+            unsigned long long b = __shfl_sync(kFull, best, src);
+            int32_t bp = __shfl_sync(kFull, par, src);
+            for (; k0 < e; k0 += 32) {
+                const int64_t k = k0 + lane;
+                const uint2 c = k < e ? a.wadj[k] : make_uint2(0u, 0xffffffffu);
+                const bool in = k < e && (unsigned long long)c.y < b - L;
+                unsigned long long nd = SP_INF;
+                if (in) {
+                    const unsigned long long du = __ldcg(&a.dist[c.x]);
+                    if (du < T) nd = du + c.y;
+                    ++scanned;
+                }
+                unsigned long long mn = nd;
+                for (int o = 16; o >= 1; o >>= 1) {
+                    const unsigned long long x = __shfl_xor_sync(kFull, mn, o);
+                    mn = x < mn ? x : mn;
+                }
+                if (mn < b) {
+                    b = mn;
+                    bp = __shfl_sync(kFull, (int32_t)c.x, __ffs(__ballot_sync(kFull, nd == mn)) - 1);
+                }
+                if (!__all_sync(kFull, in)) break;
+            }
+            if ((int)lane == src) {
+                best = b;
+                par = bp;
+            }
+        }
+        bool to_far = false;
+        if (open && best < old) {
+            ++won;
+            a.dist[v] = best;
+            a.parent[v] = par;
+            to_far = a.fstamp[v] != epoch;
+            if (to_far) a.fstamp[v] = epoch;
+        }
+        push_far(a, wb, f, epoch, to_far, v);
+    }
+    flush_open();
+    flush_far(a, wb, f, epoch);
 }
 
 __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
@@ -398,6 +599,9 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
     const int64_t nwarps = gthreads >> 5;
     const int64_t n = a.n;
     SpHeader *h = a.hdr;
+    __shared__ SpWarp s_wb[SP_THREADS / 32];
+    SpWarp &wb = s_wb[threadIdx.x >> 5];
+    SpFill f;
     unsigned bar = grid_barrier_base(&h->bar);
     unsigned long long processed = 0, scanned = 0, won = 0, reached = 0;
     const uint64_t t_start = globaltimer_ns();
@@ -426,6 +630,8 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
     unsigned qcur = 1, epoch = 1;
     unsigned long long T = a.delta;
     long long rounds = 0, buckets = 0;
+    unsigned pulls = 0;            // pull steps so far
+    unsigned long long sdeg = 0;   // degrees of the vertices settled before this bucket
     // device time per phase, as thread 0 sees it from barrier to barrier
     unsigned long long ph[4] = {0, 0, 0, 0};
     uint64_t t_ph = globaltimer_ns();
@@ -453,40 +659,59 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
         const int64_t ncur = (int64_t)__ldcg(&h->q[qcur & 3].cnt);
         const unsigned long long bigc = __ldcg(&h->q[qcur & 3].big);
         const int32_t *Q = a.nq + (int64_t)(qcur & 1) * n;
-        // ---- light edges of big rows: chunk c of the queue's numbering, one per warp;
-        // an edge is light while w < T - dist(u), a prefix of the weight-sorted row
+        // ---- light edges of big rows: an edge is light while w < T - dist(u), a prefix of the
+        // weight-sorted row.  One lane a row finds the prefix and lists its chunks; after a
+        // barrier (in the few rounds that hold big rows) the warps take one chunk each.  By
+        // the chunks of whole rows, nine tenths of them heavy and each found by a bisection of its own, the rounds
+        // of a SCALE 22 search took 2.5 ms, so 2.1.
         const int64_t nb = (int64_t)(bigc >> 32) < a.bigcap ? (int64_t)(bigc >> 32) : a.bigcap;
-        const int64_t nch = nb > 0 ? (int64_t)(bigc & 0xffffffffull) : 0;
         const SpBig *B = a.bq + (int64_t)(qcur & 1) * a.bigcap;
-        for (int64_t c = gwarp; c < nch; c += nwarps) {
-            const SpBig be = find_chunk(B, nb, c);
-            const int64_t rs = a.off[be.u], re = a.off[be.u + 1];
-            const int64_t s0 = rs + (c - (int64_t)be.cbase) * SP_CHUNK;
-            const int64_t e0 = s0 + SP_CHUNK < re ? s0 + SP_CHUNK : re;
-            const unsigned long long du = __ldcg(&a.dist[be.u]);
-            const unsigned long long lim = T - du;
-            if ((unsigned long long)a.wadj[s0].y >= lim) continue;  // the chunk is all heavy
-            for (int64_t j0 = s0; j0 < e0; j0 += 64) {
-                const int64_t j = j0 + lane;
-                uint2 c0 = make_uint2(0u, 0u), c1 = make_uint2(0u, 0u);
-                if (j < e0) c0 = ld_stream(a.wadj + j, pol);
-                if (j + 32 < e0) c1 = ld_stream(a.wadj + j + 32, pol);
-                const bool ok0 = j < e0 && (unsigned long long)c0.y < lim;
-                const bool ok1 = j + 32 < e0 && (unsigned long long)c1.y < lim;
-                scanned += ok0 + ok1;
-                relax2(a, ok0, be.u, c0, du, ok1, be.u, c1, du, T, qnext, epoch, won);
-                if (!__any_sync(kFull, ok1)) break;  // past the split
+        SpBig *LB = a.bq + 3 * a.bigcap;
+        if (gtid == 0) h->light[qnext & 1] = 0;  // its last readers finished a barrier ago
+        if (nb > 0) {
+            for (int64_t i = gtid; i < nb; i += gthreads) {
+                const int32_t u = load_spbig(B, i).u;
+                const int64_t rs = a.off[u], re = a.off[u + 1];
+                const int64_t d = weight_split(a.wadj, rs, re, T - __ldcg(&a.dist[u])) - rs;
+                if (d == 0) continue;
+                const unsigned long long old =
+                    atomicAdd(&h->light[qcur & 1], (1ull << 32) | (unsigned long long)((d + SP_LIGHT - 1) / SP_LIGHT));
+                reinterpret_cast<unsigned long long *>(LB)[old >> 32] =
+                    (unsigned long long)(uint32_t)u | ((old & 0xffffffffull) << 32);
+            }
+            if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
+            const unsigned long long lc = __ldcg(&h->light[qcur & 1]);
+            const int64_t nlb = (int64_t)(lc >> 32), nch = nlb > 0 ? (int64_t)(lc & 0xffffffffull) : 0;
+            for (int64_t c = gwarp; c < nch; c += nwarps) {
+                const SpBig be = find_chunk(LB, nlb, c);
+                const int64_t rs = a.off[be.u], re = a.off[be.u + 1];
+                const int64_t s0 = rs + (c - (int64_t)be.cbase) * SP_LIGHT;
+                const int64_t e0 = s0 + SP_LIGHT < re ? s0 + SP_LIGHT : re;
+                const unsigned long long du = __ldcg(&a.dist[be.u]);
+                const unsigned long long lim = T - du;
+                for (int64_t j0 = s0; j0 < e0; j0 += 64) {
+                    const int64_t j = j0 + lane;
+                    uint2 c0 = make_uint2(0u, 0u), c1 = make_uint2(0u, 0u);
+                    if (j < e0) c0 = ld_stream(a.wadj + j, pol);
+                    if (j + 32 < e0) c1 = ld_stream(a.wadj + j + 32, pol);
+                    const bool ok0 = j < e0 && (unsigned long long)c0.y < lim;
+                    const bool ok1 = j + 32 < e0 && (unsigned long long)c1.y < lim;
+                    scanned += ok0 + ok1;
+                    relax2(a, ok0, be.u, c0, du, ok1, be.u, c1, du, T, qnext, epoch, won, wb, f);
+                    if (!__any_sync(kFull, ok1)) break;  // past the split
+                }
             }
         }
         // ---- every queue entry: listed for its bucket's settle step once; the
         // light prefix of a shorter row expanded, 32 rows per warp as one stream
-        for (int64_t i0 = gwarp * 32; i0 < ncur; i0 += nwarps * 32) {
+        const int rn = rows_per_warp(ncur, nwarps);
+        for (int64_t i0 = gwarp * rn; i0 < ncur; i0 += nwarps * rn) {
             const int64_t i = i0 + lane;
             int64_t s0 = 0, d = 0, deg = 0;
             unsigned long long du = 0;
             bool first = false;
             int32_t u = 0;
-            if (i < ncur) {
+            if ((int)lane < rn && i < ncur) {
                 u = __ldcg(&Q[i]);
                 s0 = a.off[u];
                 deg = a.off[u + 1] - s0;
@@ -496,11 +721,14 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
                 ++processed;
                 scanned += (unsigned long long)d;
             }
-            push_settle(a, first, u, deg);
+            push_settle(a, wb, f, first, u, deg);
             const int64_t incl = warp_inclusive_scan(d);
             const int64_t total = __shfl_sync(kFull, incl, 31);
-            relax_stream(a, pol, total, s0, incl - d, du, u, T, qnext, epoch, won);
+            relax_stream(a, pol, total, s0, incl - d, du, u, T, qnext, epoch, won, wb, f);
         }
+        flush_near(a, wb, f, qnext);
+        flush_far(a, wb, f, epoch);
+        flush_settle(a, wb, f);
         if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
         phase_end(0);
         if (__ldcg(&h->q[qnext & 3].cnt) > 0) {
@@ -511,7 +739,18 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
         // from their final distances (every candidate is >= T: far)
         const unsigned e = epoch;
         if (gtid == 0) h->farcnt[(e + 1) & 1] = 0;  // its last reader was the previous split
-        {
+        const unsigned long long sd = __ldcg(&h->sdeg);
+        // by the rows of the bucket's vertices, or from the unsettled ones: about a
+        // quarter of an unsettled row lies within reach, and the list itself is read
+        const int64_t nopen = pulls ? (int64_t)__ldcg(&h->open[pulls & 1]) : n;
+        const bool pull = (double)(sd - sdeg) > 0.25 * ((double)a.nnz - (double)sd + (double)nopen);
+        sdeg = sd;
+        if (pull) {
+            pull_settle(a, pulls ? a.open + (int64_t)(pulls & 1) * n : nullptr, nopen,
+                        a.open + (int64_t)((pulls + 1) & 1) * n, &h->open[(pulls + 1) & 1], T, T - a.delta, e, gwarp,
+                        nwarps, scanned, won, wb);
+            ++pulls;
+        } else {
             const int64_t ns = (int64_t)__ldcg(&h->settle.cnt);
             const unsigned long long sbig = __ldcg(&h->settle.big);
             const int64_t snb = (int64_t)(sbig >> 32) < a.bigcap ? (int64_t)(sbig >> 32) : a.bigcap;
@@ -533,15 +772,16 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
                     const bool ok0 = j < e0 && (unsigned long long)c0.y >= lim;
                     const bool ok1 = j + 32 < e0 && (unsigned long long)c1.y >= lim;
                     scanned += ok0 + ok1;
-                    relax2(a, ok0, be.u, c0, du, ok1, be.u, c1, du, T, qnext, e, won);
+                    relax2(a, ok0, be.u, c0, du, ok1, be.u, c1, du, T, qnext, e, won, wb, f);
                 }
             }
-            for (int64_t i0 = gwarp * 32; i0 < ns; i0 += nwarps * 32) {
+            const int rs_w = rows_per_warp(ns, nwarps);
+            for (int64_t i0 = gwarp * rs_w; i0 < ns; i0 += nwarps * rs_w) {
                 const int64_t i = i0 + lane;
                 int64_t s0 = 0, d = 0;
                 unsigned long long du = 0;
                 int32_t u = 0;
-                if (i < ns) {
+                if ((int)lane < rs_w && i < ns) {
                     u = __ldcg(&a.sq[i]);
                     const int64_t rs = a.off[u], deg = a.off[u + 1] - rs;
                     du = __ldcg(&a.dist[u]);
@@ -553,15 +793,17 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
                 }
                 const int64_t incl = warp_inclusive_scan(d);
                 const int64_t total = __shfl_sync(kFull, incl, 31);
-                relax_stream(a, pol, total, s0, incl - d, du, u, T, qnext, e, won);
+                relax_stream(a, pol, total, s0, incl - d, du, u, T, qnext, e, won, wb, f);
             }
         }
+        flush_far(a, wb, f, e);
         if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
         phase_end(1);
         // ---- the least far distance >= T
         if (gtid == 0) {  // every block read the settle list before the barrier above
             h->settle.cnt = 0;
             h->settle.big = 0;
+            if (pull) h->open[(pulls + 1) & 1] = 0;  // the list just read is the next one to fill
         }
         const int64_t nf = (int64_t)__ldcg(&h->farcnt[e & 1]);
         const int32_t *F = a.fq + (int64_t)(e & 1) * n;
@@ -597,9 +839,11 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
                     a.fstamp[v] = e + 1;
                 }
             }
-            push_near(a, qnext, to_near, v);
-            push_far(a, e + 1, to_far, v);
+            push_near(a, wb, f, qnext, to_near, v);
+            push_far(a, wb, f, e + 1, to_far, v);
         }
+        flush_near(a, wb, f, qnext);
+        flush_far(a, wb, f, e + 1);
         if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
         phase_end(3);
         if (gtid == 0) h->minfar = SP_INF;  // every block read it before the barrier above
@@ -957,8 +1201,8 @@ gb_status sssp_impl(const gb_graph *g, int64_t root, double delta, double *dist,
     const int64_t bigcap = g->nnz / SP_BIG + 2;
     auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
     // header | dist | near, far and settle stamps | near queues | far lists |
-    // settle list | big lists (2 near slots, then the settle list's); slot k of
-    // a region at base + k * size
+    // settle list | big lists (2 near slots, the settle list's, the light prefixes') | open lists;
+    // slot k of a region at base + k * size
     const size_t o_dist = al(sizeof(SpHeader));
     const size_t o_ns = o_dist + al(8 * (size_t)n);
     const size_t o_fs = o_ns + al(4 * (size_t)n);
@@ -967,7 +1211,8 @@ gb_status sssp_impl(const gb_graph *g, int64_t root, double delta, double *dist,
     const size_t o_fq = o_nq + al(8 * (size_t)n);
     const size_t o_sq = o_fq + al(8 * (size_t)n);
     const size_t o_bq = o_sq + al(4 * (size_t)n);
-    const size_t total = o_bq + al(24 * (size_t)bigcap);
+    const size_t o_op = o_bq + al(32 * (size_t)bigcap);
+    const size_t total = o_op + al(8 * (size_t)n);
     unsigned char *ws = nullptr;
     Scratch tmp(s);
     GB_CUDA(tmp.alloc(&ws, total));
@@ -987,6 +1232,8 @@ gb_status sssp_impl(const gb_graph *g, int64_t root, double delta, double *dist,
     a.fq = reinterpret_cast<int32_t *>(ws + o_fq);
     a.sq = reinterpret_cast<int32_t *>(ws + o_sq);
     a.bq = reinterpret_cast<SpBig *>(ws + o_bq);
+    a.open = reinterpret_cast<int32_t *>(ws + o_op);
+    a.nnz = g->nnz;
     a.bigcap = bigcap;
     a.hdr = reinterpret_cast<SpHeader *>(ws);
     a.st = ctx->status;
