@@ -970,11 +970,12 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
 // near 4, not ms_alpha's default of 16, whose place is graphs whose masks
 // do not fit.  SCALE 22, 64 roots, 4552 active vertices with 1/15 of
 // the edges: that level 1.80 ms bottom-up, 0.48 top-down (the call 5.29 -> 3.74 ms).
-// A lower ms_alpha is kept.
+// A lower ms_alpha is kept, and so is the line in canonical mode, where the rows
+// of what a top-down level reaches are scanned for the smallest parents.
 constexpr int64_t MS_L2_MASKS = int64_t(64) << 20;
 float switch_ratio(const gb_bfs_options &o, int64_t bytes)
 {
-    return (float)(bytes <= MS_L2_MASKS ? std::min(o.ms_alpha, std::max(4.0, o.ms_alpha / 4.0)) : o.ms_alpha);
+    return (float)(bytes <= MS_L2_MASKS && !o.canonical_parents ? std::min(o.ms_alpha, std::max(4.0, o.ms_alpha / 4.0)) : o.ms_alpha);
 }
 
 template <typename T>
