@@ -882,18 +882,25 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
                 }
             }
         }
-        // short rows: the lane scans its own row in order
+        // a tight neighbour u has w(u, v) = dist(v) - dist(u) <= dist(v): the smallest id among the
+        // tight entries of that prefix of the weight-sorted row, which for the long rows of
+        // hubs, close to the root, is a small part (SCALE 22, canonical: this pass 3.9 -> 1.2 ms).
+        // Short prefixes: the lane's own, four entries at a time
+        if (scan) d = weight_split(a.wadj, rs, rs + d, dv + 1) - rs;
         if (scan && d <= 32) {
-            for (int64_t j = rs; j < rs + d; ++j) {
-                const int32_t u = a.col[j];
-                const unsigned long long du = __ldcg(&a.dist[u]);
-                if (du != SP_INF && du + a.wgt[j] == dv) {
-                    p = u;
-                    break;
-                }
+            for (int64_t j = rs; j < rs + d; j += 4) {
+                uint2 c[4];
+                unsigned long long du[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) c[t] = a.wadj[j + t < rs + d ? j + t : j];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) du[t] = __ldcg(&a.dist[c[t].x]);
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (du[t] != SP_INF && du[t] + c[t].y == dv && (p < 0 || (int32_t)c[t].x < p)) p = (int32_t)c[t].x;
             }
         }
-        // long rows: the warp scans each in rounds of 32 entries
+        // long ones: the warp in rounds of 64 entries
         unsigned longm = __ballot_sync(kFull, scan && d > 32);
         while (longm) {
             const int src = __ffs(longm) - 1;
@@ -901,23 +908,23 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
             const int64_t lrs = __shfl_sync(kFull, rs, src);
             const int64_t ld = __shfl_sync(kFull, d, src);
             const unsigned long long ldv = __shfl_sync(kFull, dv, src);
-            int32_t found = -1;
-            for (int64_t j0 = lrs; j0 < lrs + ld; j0 += 32) {
-                const int64_t j = j0 + lane;
-                bool tight = false;
-                int32_t u = 0;
-                if (j < lrs + ld) {
-                    u = a.col[j];
-                    const unsigned long long du = __ldcg(&a.dist[u]);
-                    tight = du != SP_INF && du + a.wgt[j] == ldv;
+            unsigned found = 0xffffffffu;
+            for (int64_t j0 = lrs; j0 < lrs + ld; j0 += 64) {
+                uint2 c[2];
+                unsigned long long du[2];
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const int64_t j = j0 + 32 * t + lane;
+                    c[t] = a.wadj[j < lrs + ld ? j : lrs];
                 }
-                const unsigned tm = __ballot_sync(kFull, tight);
-                if (tm) {
-                    found = __shfl_sync(kFull, u, __ffs(tm) - 1);
-                    break;
-                }
+#pragma unroll
+                for (int t = 0; t < 2; ++t) du[t] = __ldcg(&a.dist[c[t].x]);
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+                    if (du[t] != SP_INF && du[t] + c[t].y == ldv) found = min(found, c[t].x);
             }
-            if ((int)lane == src) p = found;
+            found = __reduce_min_sync(kFull, found);
+            if ((int)lane == src) p = found == 0xffffffffu ? -1 : (int32_t)found;
         }
         if (v < n) a.parent[v] = p;
     }
