@@ -216,7 +216,7 @@ gb_status graph_prepare_batched(gb_graph *g, gb_stream s);
  *   big_degree         frontier vertices of larger degree are split over the
  *                      whole grid in top-down steps.
  *   ms_alpha, ms_beta  the same switch for the multi-source BFS, on all edges
- *                      of the graph; where its masks fit the L2 it stays (not in canonical mode)
+ *                      of the graph; where its masks fit the L2 it stays
  *                      top-down up to four times as many edges (to a ratio of 4).
  *   timeout_ms         limit of every device-side wait (grid barriers, the
  *                      radix-sort look-back); on expiry the kernel records

@@ -11,10 +11,11 @@
 //    M_{l+1}[u] for its neighbours u (one atomic per edge that adds bits);
 //    the first writer of a vertex appends it to the next active list, and
 //    the bits an atomic sets first have v as a valid parent, which is
-//    written there unless canonical parents are asked for; (2) after a grid
-//    barrier, in canonical mode, each new vertex scans its sorted adjacency
-//    list for, per new bit, the first neighbour carrying that bit in M_l --
-//    the smallest-id parent -- and writes levels and parents.
+//    written there, with the level; (2) after a grid barrier, in canonical
+//    mode, the smallest-id parents: on a level that grows the active vertices'
+//    edges are visited once more, each lowering the parents of the new bits
+//    that it carries; otherwise each new vertex scans its sorted adjacency
+//    list for, per new bit, the first neighbour carrying that bit in M_l.
 //  bottom-up level: every vertex with unseen bits scans its sorted adjacency
 //    list, collecting M_l bits until all its unseen bits are found; the first
 //    neighbour to supply a bit is its parent.  A warp takes 32 consecutive
@@ -348,11 +349,9 @@ __device__ __forceinline__ void ms_append(bool on, int64_t gid, int64_t deg, MsW
     }
 }
 
-// Top-down expansion of one edge (gv -> gu) carrying frontier bits f.
 // Top-down visit of edge (v, gu), v the frontier vertex (local id pv) with
 // mask f.  The bits this atomic sets first are gu's new bits with v as their
-// parent: outside canonical mode that parent and the level are written here,
-// once per bit, and gu's row is never scanned for them.
+// parent: that parent and the level are written here, once per bit.
 template <typename T>
 __device__ __forceinline__ void ms_td_edge(bool valid, T f, int64_t gu, int32_t pv, int l,
                                            const MsArgs<T> &a, const MsSlots *S, T *Mn,
@@ -368,13 +367,11 @@ __device__ __forceinline__ void ms_td_edge(bool valid, T f, int64_t gu, int32_t 
         if (m) {
             const T old = atomic_or_mask(&Mn[gu], m);
             const T newb = m & (T)~old;
-            if (old == 0 || (!a.canonical && newb)) {
+            if (newb) {  // always so for the first bits of gu
                 const int g = find_graph(s_voff, a.ng, gu);
                 const int64_t lu = gu - s_g[g].voff;
-                if (!a.canonical && newb) {
-                    write_parents(s_g[g], S, lu, newb, pv);
-                    write_levels(s_g[g], S, lu, newb, l + 1);
-                }
+                write_parents(s_g[g], S, lu, newb, pv);
+                write_levels(s_g[g], S, lu, newb, l + 1);
                 if (old == 0) {
                     first = true;
                     deg = s_g[g].off[lu + 1] - s_g[g].off[lu];
@@ -383,6 +380,29 @@ __device__ __forceinline__ void ms_td_edge(bool valid, T f, int64_t gu, int32_t 
         }
     }
     ms_append(first, gu, deg, wb, qn, bn, my_mf, nxt, act_next, bigq_next);
+}
+
+// Canonical mode, the same edge once more when the level is complete: of the
+// bits that gu gained at this level, those that v carries have v as a possible
+// parent.
+template <typename T>
+__device__ __forceinline__ void ms_min_edge(bool valid, T f, int64_t gu, int32_t pv, const MsArgs<T> &a,
+                                            const MsSlots *S, const T *Mn, const MsGraph *s_g, const int64_t *s_voff)
+{
+    unsigned long long m = valid ? (unsigned long long)(f & ld_mask(&Mn[gu])) : 0ull;
+    if (!m) return;
+    const int g = find_graph(s_voff, a.ng, gu);
+    const MsGraph &G = s_g[g];
+    int64_t lu = gu - G.voff;
+    if (!S && G.perm) {  // staged by original id, as an original id
+        lu = orig_id(G, lu);
+        pv = (int32_t)orig_id(G, pv);
+    }
+    while (m) {
+        const int b = __ffsll(m) - 1;
+        m &= m - 1;
+        atomicMin(S ? &S->par[b][lu] : &G.pst[lu * G.kst + b], pv);
+    }
 }
 
 // Rows of a warp (lane i owns one row: graph g, adjacency [s, e), missing
@@ -652,6 +672,12 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
         }
 
         if (td) {
+            // pass 0 visits the active vertices' edges; in canonical mode a level that
+            // grows visits them once more for the smallest parents (ms_min_edge):
+            // what it reached, hubs next to the roots, has far longer rows
+            int64_t nn = 0;
+            bool by_edges = false;
+            for (int pass = 0; pass < (by_edges ? 2 : 1); ++pass) {
             // (1a) big active vertices in 256-edge chunks
             if (nc > 0) {
                 const int64_t per = (nc + nwarps - 1) / nwarps;
@@ -684,8 +710,11 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                             const int64_t j = b + lane;
                             const bool valid = j < e;
                             const int64_t gu = valid ? G.voff + G.col[j] : 0;
-                            ms_td_edge(valid, f, gu, (int32_t)lv, l, a, S, Mn, s_g, s_voff, wb,
-                                       qn_buf, bn_buf, my_mf, nxt, act_next, bigq_next);
+                            if (pass == 0)
+                                ms_td_edge(valid, f, gu, (int32_t)lv, l, a, S, Mn, s_g, s_voff, wb,
+                                           qn_buf, bn_buf, my_mf, nxt, act_next, bigq_next);
+                            else
+                                ms_min_edge(valid, f, gu, (int32_t)lv, a, S, Mn, s_g, s_voff);
                         }
                     }
                 }
@@ -705,7 +734,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                     if (d > MS_BIG_DEG) d = 0;
                     f = ld_mask(&M[gv]);
                 }
-                my_touched += (i < na);
+                my_touched += (i < na && pass == 0);
                 my_edges += d;
                 const int64_t incl = warp_inclusive_scan(d);
                 const int64_t total = __shfl_sync(kFull, incl, 31);
@@ -726,17 +755,25 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                     const bool valid = kk < total;
                     const int64_t gu = valid ? vvo + s_g[og].col[so + (kk - eo)] : 0;
                     const int32_t pvo = (int32_t)(__shfl_sync(kFull, gv, owner) - vvo);
-                    ms_td_edge(valid, fo, gu, pvo, l, a, S, Mn, s_g, s_voff, wb, qn_buf, bn_buf,
-                               my_mf, nxt, act_next, bigq_next);
+                    if (pass == 0)
+                        ms_td_edge(valid, fo, gu, pvo, l, a, S, Mn, s_g, s_voff, wb, qn_buf, bn_buf,
+                                   my_mf, nxt, act_next, bigq_next);
+                    else
+                        ms_min_edge(valid, fo, gu, pvo, a, S, Mn, s_g, s_voff);
                 }
             }
-            ms_flush_q(wb, qn_buf, nxt, act_next);
-            ms_flush_b(wb, bn_buf, nxt, bigq_next);
-            if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_MS_BAR)) return;
-            // (2) the vertices that gained bits join `seen`; in canonical mode
-            // each also scans its row for its smallest-id parents and writes
-            // its levels (otherwise both were written in (1))
-            const int64_t nn = (int64_t)ldcg_u64(&nxt->na);
+            if (pass == 0) {
+                ms_flush_q(wb, qn_buf, nxt, act_next);
+                ms_flush_b(wb, bn_buf, nxt, bigq_next);
+                if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_MS_BAR)) return;
+                nn = (int64_t)ldcg_u64(&nxt->na);
+                by_edges = a.canonical && nn > na;
+            }
+            }
+            // (2) the vertices that gained bits join `seen`; in canonical mode, on
+            // a level that does not grow, each also scans its row for its
+            // smallest-id parents
+            const bool by_rows = a.canonical && !by_edges;
             for (int64_t i0 = gwarp * 32; i0 < nn; i0 += nwarps * 32) {
                 const int64_t i = i0 + lane;
                 int64_t gu = 0, lu = 0, rs = 0, re = 0;
@@ -747,14 +784,13 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                     g = find_graph(s_voff, a.ng, gu);
                     lu = gu - s_g[g].voff;
                     nw = ld_mask(&Mn[gu]);
-                    if (a.canonical) {
+                    if (by_rows) {
                         rs = s_g[g].off[lu];
                         re = s_g[g].off[lu + 1];
                     }
                 }
-                if (a.canonical) ms_rows(s_g, S, M, g, orig_id(s_g[g], lu), rs, re, nw, my_edges);
+                if (by_rows) ms_rows(s_g, S, M, g, orig_id(s_g[g], lu), rs, re, nw, my_edges);
                 if (i < nn) {
-                    if (a.canonical) write_levels(s_g[g], S, lu, nw, l + 1);
                     st_mask(&a.seen[gu], (T)(ld_mask(&a.seen[gu]) | nw));
                     if (a.hist && l + 1 < MS_HIST)
                         a.hist[(size_t)(l + 1) * a.mstride + s_g[g].voff + orig_id(s_g[g], lu)] = nw;
@@ -970,12 +1006,12 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
 // near 4, not ms_alpha's default of 16, whose place is graphs whose masks
 // do not fit.  SCALE 22, 64 roots, 4552 active vertices with 1/15 of
 // the edges: that level 1.80 ms bottom-up, 0.48 top-down (the call 5.29 -> 3.74 ms).
-// A lower ms_alpha is kept, and so is the line in canonical mode, where the rows
-// of what a top-down level reaches are scanned for the smallest parents.
+// A lower ms_alpha is kept.  (In canonical mode the level costs twice as much
+// top-down, 0.94 ms, and the call still gains: 5.34 -> 4.27 ms.)
 constexpr int64_t MS_L2_MASKS = int64_t(64) << 20;
 float switch_ratio(const gb_bfs_options &o, int64_t bytes)
 {
-    return (float)(bytes <= MS_L2_MASKS && !o.canonical_parents ? std::min(o.ms_alpha, std::max(4.0, o.ms_alpha / 4.0)) : o.ms_alpha);
+    return (float)(bytes <= MS_L2_MASKS ? std::min(o.ms_alpha, std::max(4.0, o.ms_alpha / 4.0)) : o.ms_alpha);
 }
 
 template <typename T>
