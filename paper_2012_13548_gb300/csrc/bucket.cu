@@ -633,14 +633,13 @@ struct LeafShared {
 };
 
 struct LeafArgs {
-    const BkDesc *desc;
-    const unsigned *ndesc_dev;  // or null: ndesc
+    const BkDesc *desc, *desc2;  // two lists of buckets: ndesc of them, read from src,
     unsigned ndesc;
+    const unsigned *ndesc2;      // and *ndesc2 pieces of the longer ones, read from src2
     int scale;
-    int last;              // no further split follows
+    BkCtl *ctl2;           // its overflow is set if a piece is too long for a sort here
     unsigned *tile_cnt;    // kept entries per POS_TILE positions
     unsigned *rawoff;      // [n + 1] first position of every row
-    BkCtl *ctl;
     uint2 *wadj;           // MODE 2
 };
 
@@ -665,14 +664,14 @@ template <typename K, int MODE>
 __device__ __forceinline__ void leaf_put(const LeafArgs &a, const Leaf<K> &lf, K *dst, uint32_t pos, K k, bool keep)
 {
     constexpr int LOW = MODE == 1 ? WBITS : 0;
-    const uint64_t uv = lf.uv0 + (uint64_t)(k >> LOW);
-    const uint32_t c = (uint32_t)(uv & low_mask(a.scale));
+    // the column lies in the low 32 bits of (u, v)
+    const uint32_t c = ((uint32_t)lf.uv0 + (uint32_t)(k >> LOW)) & (uint32_t)low_mask(a.scale);
     if (MODE == 0) {
         dst[pos] = (K)(c | (keep ? 0u : 0x80000000u));
     } else if (MODE == 1) {
         dst[pos] = (K)(((uint64_t)(c | (keep ? 0u : 0x80000000u)) << 32) | ((uint64_t)k & ((1u << WBITS) - 1)));
     } else {
-        a.wadj[pos] = make_uint2(c, (uint32_t)(uv >> a.scale) & ((1u << WBITS) - 1));
+        a.wadj[pos] = make_uint2(c, (uint32_t)((lf.uv0 + (uint64_t)k) >> a.scale) & ((1u << WBITS) - 1));
     }
 }
 
@@ -820,22 +819,24 @@ __device__ __forceinline__ bool count_sort(const LeafArgs &a, const Leaf<K> &lf,
 }
 
 template <typename K, int MODE>
-__global__ void __launch_bounds__(LF_THREADS, sizeof(K) == 4 ? 6 : 4) bk_leaf_kernel(LeafArgs a, const K *src, K *dst)
+__global__ void __launch_bounds__(LF_THREADS, sizeof(K) == 4 ? 6 : 4) bk_leaf_kernel(LeafArgs a, const K *src1, const K *src2, K *dst)
 {
     extern __shared__ __align__(16) unsigned char lf_dyn[];
     K *s = reinterpret_cast<K *>(lf_dyn);
     LeafShared &sh = *reinterpret_cast<LeafShared *>(lf_dyn + LF_PLACES * sizeof(K));
     __shared__ unsigned long long s_min;
-    const unsigned nd = a.ndesc_dev ? *a.ndesc_dev : a.ndesc;
+    const unsigned nd = a.ndesc + *a.ndesc2;
     constexpr int LOW = MODE == 1 ? WBITS : 0;  // bits that do not tell entries apart
     const uint64_t vmask = low_mask(a.scale);
     const int tid = threadIdx.x;
     for (unsigned q = blockIdx.x; q < nd; q += gridDim.x) {
-        const BkDesc d = a.desc[q];
+        const bool piece = q >= a.ndesc;
+        const BkDesc d = piece ? a.desc2[q - a.ndesc] : a.desc[q];
+        const K *src = piece ? src2 : src1;
         const int bits = desc_bits(d.pr), rem = d.rem;
         const bool big = d.count > (unsigned)BK_CAP;
         if (big && rem > LOW) {
-            if (a.last && tid == 0) a.ctl->overflow = 1;
+            if (piece && tid == 0) a.ctl2->overflow = 1;
             continue;
         }
         Leaf<K> lf;
@@ -934,8 +935,8 @@ struct BkResult {
     DevStatus status;
 };
 
-// base[i] = kept entries before tile i; their total, the last split's overflow flag and
-// the device status to *res.
+// base[i] = kept entries before tile i; their total, whether pieces are left that
+// need a further split, and the device status to *res.
 __global__ void __launch_bounds__(PS_THREADS) bk_posscan_kernel(const unsigned *__restrict__ cnt, unsigned nt,
                                                                 const unsigned *__restrict__ sums,
                                                                 unsigned *__restrict__ base,
@@ -1140,12 +1141,12 @@ gb_status split(Context *ctx, const Level &lv, const BkDesc *desc, const unsigne
 }
 
 template <typename K, int MODE>
-gb_status leaves(Context *ctx, const LeafArgs &a, int64_t most, const K *src, K *dst, cudaStream_t s)
+gb_status leaves(Context *ctx, const LeafArgs &a, int64_t most, const K *src, const K *src2, K *dst, cudaStream_t s)
 {
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(most, (int64_t)ctx->num_sms * 32));
     constexpr int smem = LF_PLACES * (int)sizeof(K) + (int)sizeof(LeafShared);
     GB_CUDA(smem_limit(bk_leaf_kernel<K, MODE>, smem));
-    bk_leaf_kernel<K, MODE><<<grid, LF_THREADS, smem, s>>>(a, src, dst);
+    bk_leaf_kernel<K, MODE><<<grid, LF_THREADS, smem, s>>>(a, src, src2, dst);
     note_launch();
     GB_CUDA(cudaGetLastError());
     return GB_OK;
@@ -1288,42 +1289,51 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
         if (rc != GB_OK) return rc;
         leaf_desc = lv.desc;
     }
-    // steps 2 and 3: the buckets of at most BK_CAP keys, then the pieces of the longer ones
+    // steps 2 and 3: the buckets of at most BK_CAP keys, and the pieces of the longer
+    // ones, moved to ka and sorted back into their places in kb
     const Level lv2 = level_at(ws, l2), lv3 = level_at(ws, l3);
     LeafArgs la{};
     la.desc = leaf_desc;
     la.ndesc = (unsigned)n1;
+    la.desc2 = lv2.desc;
+    la.ndesc2 = &lv2.ctl->ndesc;
+    la.ctl2 = lv2.ctl;
     la.scale = scale;
     la.tile_cnt = reinterpret_cast<unsigned *>(ws + o_pos);
     la.rawoff = reinterpret_cast<unsigned *>(ws + o_raw);
-    la.ctl = lv3.ctl;
     rc = split<K, K>(ctx, lv2, leaf_desc, nullptr, (unsigned)n1, 0, field, LOW, nk, kb, ka, s);
     if (rc != GB_OK) return rc;
-    rc = leaves<K, MODE>(ctx, la, n1, kb, kb, s);
-    if (rc != GB_OK) return rc;
-    // the longer ones' places in kb are free now: their pieces are sorted from ka into kb
-    rc = split<K, K>(ctx, lv3, lv2.desc, &lv2.ctl->ndesc, 0, 0, field, LOW, nk, ka, kb, s);
-    if (rc != GB_OK) return rc;
-    la.desc = lv2.desc;
-    la.ndesc_dev = &lv2.ctl->ndesc;
-    rc = leaves<K, MODE>(ctx, la, desc_x, ka, kb, s);
-    if (rc != GB_OK) return rc;
-    la.desc = lv3.desc;
-    la.ndesc_dev = &lv3.ctl->ndesc;
-    la.last = 1;
-    rc = leaves<K, MODE>(ctx, la, desc_x, kb, kb, s);
+    rc = leaves<K, MODE>(ctx, la, n1 + desc_x, kb, ka, kb, s);
     if (rc != GB_OK) return rc;
     // step 4
     unsigned *sums = reinterpret_cast<unsigned *>(ws + o_sums), *base = reinterpret_cast<unsigned *>(ws + o_base);
-    const unsigned psb = (unsigned)((npos + PS_CHUNK - 1) / PS_CHUNK);
-    bk_possum_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums);
     BkResult *res = reinterpret_cast<BkResult *>(ws + o_res);
-    bk_posscan_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums, base, lv3.ctl, ctx->status, res);
-    note_launch(2);
-    GB_CUDA(cudaGetLastError());
+    const unsigned psb = (unsigned)((npos + PS_CHUNK - 1) / PS_CHUNK);
     BkResult hr;
-    GB_CUDA(cudaMemcpyAsync(&hr, res, sizeof(hr), cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaStreamSynchronize(s));
+    const auto positions = [&]() -> gb_status {
+        bk_possum_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums);
+        bk_posscan_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums, base, la.ctl2, ctx->status, res);
+        note_launch(2);
+        GB_CUDA(cudaGetLastError());
+        GB_CUDA(cudaMemcpyAsync(&hr, res, sizeof(hr), cudaMemcpyDeviceToHost, s));
+        GB_CUDA(cudaStreamSynchronize(s));
+        return GB_OK;
+    };
+    rc = positions();
+    if (rc != GB_OK) return rc;
+    if (hr.overflow) {
+        // rows of 64 K entries and more in one bucket: their pieces are split once more
+        rc = split<K, K>(ctx, lv3, lv2.desc, &lv2.ctl->ndesc, 0, 0, field, LOW, nk, ka, kb, s);
+        if (rc != GB_OK) return rc;
+        la.ndesc = 0;
+        la.desc2 = lv3.desc;
+        la.ndesc2 = &lv3.ctl->ndesc;
+        la.ctl2 = lv3.ctl;
+        rc = leaves<K, MODE>(ctx, la, desc_x, kb, kb, kb, s);
+        if (rc != GB_OK) return rc;
+        rc = positions();
+        if (rc != GB_OK) return rc;
+    }
     const DevStatus &hst = hr.status;
     const unsigned nnz = hr.nnz;
     if (hst.code != 0) {
@@ -1422,27 +1432,30 @@ gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, bool *overflow, cu
     LeafArgs la{};
     la.desc = desc;
     la.ndesc = nd;
+    la.desc2 = lv2.desc;
+    la.ndesc2 = &lv2.ctl->ndesc;
+    la.ctl2 = lv2.ctl;
     la.scale = g->scale;
-    la.ctl = lv3.ctl;
     la.wadj = wadj;
     gb_status rc = split<uint64_t, uint64_t>(ctx, lv2, desc, nullptr, nd, 0, field, 0, nnz, kb, ka, s);
     if (rc != GB_OK) return rc;
-    rc = leaves<uint64_t, 2>(ctx, la, nd, kb, kb, s);
-    if (rc != GB_OK) return rc;
-    rc = split<uint64_t, uint64_t>(ctx, lv3, lv2.desc, &lv2.ctl->ndesc, 0, 0, field, 0, nnz, ka, kb, s);
-    if (rc != GB_OK) return rc;
-    la.desc = lv2.desc;
-    la.ndesc_dev = &lv2.ctl->ndesc;
-    rc = leaves<uint64_t, 2>(ctx, la, desc_x, ka, kb, s);
-    if (rc != GB_OK) return rc;
-    la.desc = lv3.desc;
-    la.ndesc_dev = &lv3.ctl->ndesc;
-    la.last = 1;
-    rc = leaves<uint64_t, 2>(ctx, la, desc_x, kb, kb, s);
+    rc = leaves<uint64_t, 2>(ctx, la, nd + desc_x, kb, ka, kb, s);
     if (rc != GB_OK) return rc;
     unsigned ovf = 0;
-    GB_CUDA(cudaMemcpyAsync(&ovf, &lv3.ctl->overflow, sizeof(ovf), cudaMemcpyDeviceToHost, s));
+    GB_CUDA(cudaMemcpyAsync(&ovf, &lv2.ctl->overflow, sizeof(ovf), cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
+    if (ovf) {
+        rc = split<uint64_t, uint64_t>(ctx, lv3, lv2.desc, &lv2.ctl->ndesc, 0, 0, field, 0, nnz, ka, kb, s);
+        if (rc != GB_OK) return rc;
+        la.ndesc = 0;
+        la.desc2 = lv3.desc;
+        la.ndesc2 = &lv3.ctl->ndesc;
+        la.ctl2 = lv3.ctl;
+        rc = leaves<uint64_t, 2>(ctx, la, desc_x, kb, kb, kb, s);
+        if (rc != GB_OK) return rc;
+        GB_CUDA(cudaMemcpyAsync(&ovf, &lv3.ctl->overflow, sizeof(ovf), cudaMemcpyDeviceToHost, s));
+        GB_CUDA(cudaStreamSynchronize(s));
+    }
     *overflow = ovf != 0;
     return GB_OK;
 }

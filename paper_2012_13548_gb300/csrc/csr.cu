@@ -279,8 +279,8 @@ constexpr int HUB_ROUNDS = 4;  // rounds whose loads are in flight together
 // first), so long rows, whose vertices are reached early anyway, are only
 // sampled: every row costs at most HUB_SCAN entries.  hd[u] = (hub[u], min(degree(u), 65535)): the bottom-up list walks read both with one
 // 8-byte load instead of a hub load and two 8-byte offsets from other sectors.
-// A warp takes 32 rows and streams their edges as one sequence (lane k of a
-// round reads entry k).  Rows ascend, so the smallest id among equal keys is the
+// A warp takes `rows` rows (32; fewer on a small graph, whose rows then reach more
+// warps) and streams their edges as one sequence (lane k of a round reads entry k).  Rows ascend, so the smallest id among equal keys is the
 // first of them: (key, 255 - place in the row) fits 16 bits, and a row's
 // greatest is one warp reduction where a round lies in one row, a native
 // 32-bit shared-memory maximum where it does not.
@@ -288,15 +288,15 @@ __global__ void __launch_bounds__(HUB_THREADS) hub_kernel(const int64_t *__restr
                                                           const int32_t *__restrict__ col,
                                                           const uint8_t *__restrict__ key, int64_t n,
                                                           int64_t nnz, int32_t *__restrict__ hub,
-                                                          int2 *__restrict__ hd, DevStatus *st)
+                                                          int2 *__restrict__ hd, int rows, DevStatus *st)
 {
     __shared__ unsigned s_best[HUB_THREADS];
     const unsigned lane = threadIdx.x & 31u;
     const int wbase = threadIdx.x & ~31;
     const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t r0 = gwarp * 32; r0 < n; r0 += nwarps * 32) {
-        const int64_t r = r0 + lane;
+    for (int64_t r0 = gwarp * rows; r0 < n; r0 += nwarps * rows) {
+        const int64_t r = (int)lane < rows ? r0 + lane : n;
         int64_t s0 = 0, deg = 0;
         if (r < n) {
             s0 = off[r];
@@ -611,8 +611,10 @@ gb_status build_graph_aux(gb_graph *g, cudaStream_t s)
     degrees_kernel<<<(unsigned)nb, NZL_THREADS, 0, s>>>(g->off, n, g->nz, nw, key, cnt);
     k1_scan_tiles_kernel<<<1, 1024, 0, s>>>(cnt, nb, base);
     // several waves of blocks: rows differ in length
-    const unsigned hb = (unsigned)std::min<int64_t>((n + HUB_THREADS - 1) / HUB_THREADS, (int64_t)ctx->num_sms * 64);
-    hub_kernel<<<hb, HUB_THREADS, 0, s>>>(g->off, g->col, key, n, g->nnz, g->hub, g->hd, ctx->status);
+    const int rows = n <= (int64_t)ctx->num_sms * 1024 ? 8 : 32;
+    const int64_t per = (int64_t)rows * (HUB_THREADS / 32);  // rows a block takes at a time
+    const unsigned hb = (unsigned)std::min<int64_t>((n + per - 1) / per, (int64_t)ctx->num_sms * 64);
+    hub_kernel<<<hb, HUB_THREADS, 0, s>>>(g->off, g->col, key, n, g->nnz, g->hub, g->hd, rows, ctx->status);
     note_launch(3);
     GB_CUDA(cudaGetLastError());
     unsigned long long nnzv = 0;
