@@ -149,9 +149,9 @@ struct BfsArgs {
 // level 1.68 ms top-down, the search 2.32 ms; bottom-up 1.50 ms in all. At a ratio
 // of 128 another root's search went from 1.31 to 2.77 ms, so the line is 64.
 constexpr float HUB_MEAN = 16.0f;
-__device__ __forceinline__ bool go_bottom_up(double mf, double mu, double qn, const BfsArgs &a)
+__device__ __forceinline__ bool go_bottom_up(float mf, float mu, float qn, const BfsArgs &a)
 {
-    return mf > mu / a.alpha || (mf > mu / a.alpha_hub && mf > qn * a.hub_deg);
+    return mf * a.alpha > mu || (mf * a.alpha_hub > mu && mf > qn * a.hub_deg);
 }
 
 void set_switch(BfsArgs &a, const gb_bfs_options &o)
@@ -253,6 +253,57 @@ __device__ __forceinline__ void flush_big(WarpBuf &wb, int &bn, const BfsArgs &a
                (e & 0xffffffffull) | (cb << 32));
     }
     __syncwarp();
+    bn = 0;
+}
+
+// Block-collective, at the end of a level: what the warps still hold staged, with
+// one atomic per block and list.  Each of up to 9728 warps took one for
+// itself, 1.6 ns apiece on the same address: 8 us a list and level.
+struct LevelFlush {
+    unsigned q[32];              // staged vertices of every warp, then where they go
+    unsigned long long b[32];    // (big vertices << 32) | their chunks, likewise
+};
+__device__ __forceinline__ void flush_level(LevelFlush &lf, WarpBuf &wb, int &qn, int &bn, int nwarps, const BfsArgs &a,
+                                            LevelCtl *nxt, int64_t qnext_base, int64_t bnext_base)
+{
+    const unsigned lane = lane_id();
+    const int warp = threadIdx.x >> 5;
+    __syncwarp();
+    const unsigned long long e = (int)lane < bn ? wb.b[lane] : 0ull;
+    const unsigned nch = (unsigned)(e >> 32);
+    const unsigned incl = warp_inclusive_scan(nch);
+    if (lane == 31) {
+        lf.q[warp] = (unsigned)qn;
+        lf.b[warp] = ((unsigned long long)bn << 32) | incl;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned q = (int)lane < nwarps ? lf.q[lane] : 0u;
+        const unsigned long long b = (int)lane < nwarps ? lf.b[lane] : 0ull;
+        const unsigned qi = warp_inclusive_scan(q);
+        const unsigned long long bi = warp_inclusive_scan(b);
+        unsigned long long q0 = 0, b0 = 0;
+        if (lane == 31) {
+            if (qi) q0 = atomicAdd(&nxt->qcnt, (unsigned long long)qi);
+            if (bi) b0 = atomicAdd(&nxt->big, bi);
+        }
+        q0 = __shfl_sync(kFull, q0, 31);
+        b0 = __shfl_sync(kFull, b0, 31);
+        lf.q[lane] = (unsigned)q0 + qi - q;  // a level holds at most n < 2^31 vertices
+        lf.b[lane] = b0 + bi - b;
+    }
+    __syncthreads();
+    const int64_t q0 = qnext_base + (int64_t)lf.q[warp];
+    const unsigned long long p = lf.b[warp];
+    for (int i = lane; i < qn; i += 32)
+        if (GB_OK_IDX(a.st, q0 + i, a.n, 200)) __stcg(&a.queue[q0 + i], wb.q[i]);
+    if ((int)lane < bn && GB_OK_IDX(a.st, bnext_base + (int64_t)(p >> 32) + lane, a.bigcap, 202)) {
+        const unsigned long long cb = (p & 0xffffffffull) + incl - nch;
+        __stcg(reinterpret_cast<unsigned long long *>(a.bigq) + bnext_base + (int64_t)(p >> 32) + lane,
+               (e & 0xffffffffull) | (cb << 32));
+    }
+    __syncwarp();
+    qn = 0;
     bn = 0;
 }
 
@@ -821,7 +872,7 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
         if (qn == 0 || qn > SOLO_Q || nmf > (unsigned long long)(dm > SOLO_ROW ? SOLO_E : SOLO_E_SHORT) || stop ||
             l > a.n)
             break;
-        if (qn > prev_qn && go_bottom_up(mf, mu - mf, (double)qn, a)) break;  // the bottom-up rule, applied by the grid
+        if (qn > prev_qn && go_bottom_up((float)mf, (float)(mu - mf), (float)qn, a)) break;  // the bottom-up rule, applied by the grid
         mu -= mf;
     }
     // the frontier left: its bits, its big vertices, its counters (the first
@@ -893,6 +944,7 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
     unsigned bar_target = grid_barrier_base(&h->bar);
     __shared__ WarpBuf s_wb[NT / 32];
     __shared__ unsigned long long s_mf;
+    __shared__ LevelFlush s_lf;
     WarpBuf &wb = s_wb[threadIdx.x >> 5];
     int qn_buf = 0, bn_buf = 0;  // warp-uniform fill levels of wb
     int un_open = 0;             // warp-uniform: vertices in this warp's open-list segment
@@ -960,7 +1012,7 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
                 // bottom-up pays while the frontier grows: after its peak, few
                 // vertices are unvisited and the ratio alone would send a
                 // search of thin last levels over every vertex again
-                if (go_bottom_up(mf, mu, (double)qn, a) && qn > prev_qn) td = false;
+                if (go_bottom_up((float)mf, (float)mu, (float)qn, a) && qn > prev_qn) td = false;
             } else if (qn < prev_qn && (double)qn < (double)n / a.beta) {
                 td = true;
             }
@@ -1248,8 +1300,7 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
                             nxt, qnext_base, bnext_base);
         }
         // end of level: flush the staged vertices and add the block's degree sum
-        flush_queue(wb, qn_buf, a, nxt, qnext_base);
-        flush_big(wb, bn_buf, a, nxt, bnext_base);
+        flush_level(s_lf, wb, qn_buf, bn_buf, NT / 32, a, nxt, qnext_base, bnext_base);
         {
             const unsigned long long t = warp_sum(my_mf);
             my_mf = 0;
