@@ -650,7 +650,11 @@ static_assert(SOLO_Q == 2 * BFS_THREADS, "two frontier vertices per thread in th
 
 // Block-collective part of a narrow level: TD_E edges per thread (src[t] ->
 // v[t], v[t] < 0: none).  An edge's target is claimed on the visited bitmap
-// while its offsets are loaded; the winners join the next frontier.
+// while its offsets are loaded; the winners join the next frontier.  TEST: only
+// targets that a plain load shows unvisited are claimed (a line of the L1 may be old,
+// which costs an atomic, not a wrong answer): one more memory latency, but one
+// SM's loads of scattered words are what a level of some hundred vertices waits for.
+template <bool TEST>
 __device__ __forceinline__ void solo_visit(const BfsArgs &a, SoloBuf &sb, int nx, int slot, int l, int64_t qnext,
                                            const int32_t (&src)[TD_E], const int32_t (&v)[TD_E],
                                            unsigned long long &mfs, int &dmax)
@@ -659,12 +663,17 @@ __device__ __forceinline__ void solo_visit(const BfsArgs &a, SoloBuf &sb, int nx
     int64_t s0[TD_E];
     int32_t dg[TD_E];
 #pragma unroll
-    for (int t = 0; t < TD_E; ++t)
-        old[t] = v[t] >= 0 ? atomicOr(&a.vis[(unsigned)v[t] >> 5], 1u << (v[t] & 31)) : kFull;
+    for (int t = 0; t < TD_E; ++t) old[t] = v[t] < 0 ? kFull : TEST ? a.vis[(unsigned)v[t] >> 5] : 0u;
+    bool cand[TD_E];
 #pragma unroll
     for (int t = 0; t < TD_E; ++t) {
-        s0[t] = v[t] >= 0 ? __ldg(&a.off[v[t]]) : 0;
-        dg[t] = v[t] >= 0 ? (int32_t)(__ldg(&a.off[v[t] + 1]) - s0[t]) : 0;
+        cand[t] = !((old[t] >> (v[t] & 31)) & 1u);
+        if (cand[t]) old[t] = atomicOr(&a.vis[(unsigned)v[t] >> 5], 1u << (v[t] & 31));
+    }
+#pragma unroll
+    for (int t = 0; t < TD_E; ++t) {
+        s0[t] = cand[t] ? __ldg(&a.off[v[t]]) : 0;
+        dg[t] = cand[t] ? (int32_t)(__ldg(&a.off[v[t] + 1]) - s0[t]) : 0;
     }
     int c = 0;
 #pragma unroll
@@ -776,21 +785,22 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
         int dmx = 0;
         const bool by_edge = dm > SOLO_ROW;
         if (!by_edge) {
-            for (int i0 = 0; i0 < q; i0 += NT) {
-                const int i = i0 + tid;
-                const int32_t u = i < q ? sb.v[cur][i] : 0;
-                const int d = i < q ? sb.deg[cur][i] : 0;
-                const int64_t s0 = i < q ? sb.start[cur][i] : 0;
-                for (int b = 0; b < dm; b += TD_E) {
-                    int32_t src[TD_E], v[TD_E];
+            // four or eight lanes a row, a lane an entry: a load of the columns touches 8
+            // or 4 rows' lines, not 32
+            const int gs = dm <= 4 ? 2 : 3;
+            const int e = tid & ((1 << gs) - 1), rows = NT >> gs;
+            for (int i0 = tid >> gs; i0 - (tid >> gs) < q; i0 += TD_E * rows) {
+                int32_t src[TD_E], v[TD_E];
 #pragma unroll
-                    for (int t = 0; t < TD_E; ++t) {
-                        src[t] = u;
-                        v[t] = b + t < d && GB_OK_IDX(a.st, s0 + b + t, a.nnz, 241) ? __ldg(&a.col[s0 + b + t]) : -1;
-                        if (v[t] >= 0 && !GB_OK_IDX(a.st, v[t], a.n, 242)) v[t] = -1;
-                    }
-                    solo_visit(a, sb, cur ^ 1, slot, l, qnext, src, v, mfs, dmx);
+                for (int t = 0; t < TD_E; ++t) {
+                    const int i = i0 + t * rows;
+                    src[t] = i < q ? sb.v[cur][i] : 0;
+                    const int d = i < q ? sb.deg[cur][i] : 0;
+                    const int64_t j = (i < q ? sb.start[cur][i] : 0) + e;
+                    v[t] = e < d && GB_OK_IDX(a.st, j, a.nnz, 241) ? __ldg(&a.col[j]) : -1;
+                    if (v[t] >= 0 && !GB_OK_IDX(a.st, v[t], a.n, 242)) v[t] = -1;
                 }
+                solo_visit<true>(a, sb, cur ^ 1, slot, l, qnext, src, v, mfs, dmx);
             }
         } else {
             // exclusive prefix of the frontier's degrees, two vertices per thread
@@ -819,7 +829,7 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
                     v[t] = k < total && GB_OK_IDX(a.st, j, a.nnz, 241) ? __ldg(&a.col[j]) : -1;
                     if (v[t] >= 0 && !GB_OK_IDX(a.st, v[t], a.n, 242)) v[t] = -1;
                 }
-                solo_visit(a, sb, cur ^ 1, slot, l, qnext, src, v, mfs, dmx);
+                solo_visit<false>(a, sb, cur ^ 1, slot, l, qnext, src, v, mfs, dmx);
             }
         }
         if (__any_sync(kFull, mfs != 0)) {
