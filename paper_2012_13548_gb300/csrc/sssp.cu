@@ -1260,6 +1260,15 @@ gb_status sssp_impl(const gb_graph *g, int64_t root, double delta, double *dist,
         blocks = sssp_pick_blocks(ctx->num_sms);
         if (dev < 64) blocks_cache[dev] = blocks;
     }
+    // The grid follows the graph, as the BFS's does: a search passes a few hundred
+    // barriers of all blocks.  us per search (edgefactor 16, delta 0.1) on 304 / 152 blocks and on one per
+    // 2^14 entries, at most 304: SCALE 10 425 / 324 / 316, SCALE 14 761 / 584 / 552, SCALE 16
+    // 928 / 728 / 717, SCALE 18 1155 / 908 / 1151, SCALE 20 1702 / 1475 / 1701, SCALE 22
+    // 3171 / 3204 / 3138.
+    constexpr int64_t kPerBlock = int64_t(1) << 14;
+    constexpr int64_t kWideNnz = int64_t(100) << 20;
+    if (g->nnz < kWideNnz) blocks = std::min(blocks, ctx->num_sms);
+    blocks = (int)std::min<int64_t>(blocks, std::max<int64_t>(1, (g->nnz + kPerBlock - 1) / kPerBlock));
     void *args[] = {&a};
     GB_CUDA(cudaLaunchCooperativeKernel((const void *)sssp_kernel, dim3(blocks), dim3(SP_THREADS), args,
                                         0, s));
