@@ -1092,8 +1092,14 @@ gb_status ms_launch(std::vector<MsGraph> gs, int k, const std::vector<int64_t> &
     a.vec_col = 1;
     for (int i = 0; i < ng; ++i)
         if (reinterpret_cast<uintptr_t>(gs[i].col) & 15u) a.vec_col = 0;
+    // Small graphs run on one block per SM: half the arrivals at every level's barriers.
+    // us per call on 304 / 152 blocks, 8 roots: SCALE 12 232 / 200, 14 199 / 167, 16 329 / 306,
+    // 18 324 / 309, 20 490 / 585; 64 roots: SCALE 14 358 / 292, 18 730 / 724, 20 1261 / 1510;
+    // 32 graphs of SCALE 8-12 (1.2 M entries) 435 / 408, of SCALE 12-18 (59 M) 1173 / 1411.
+    constexpr int64_t kNarrowNnz = int64_t(12) << 20;
+    const int blocks = nnz_tot < kNarrowNnz ? std::min(ctx->ms_blocks, ctx->num_sms) : ctx->ms_blocks;
     void *args[] = {&a};
-    GB_CUDA(cudaLaunchCooperativeKernel((const void *)ms_kernel<T>, dim3(ctx->ms_blocks),
+    GB_CUDA(cudaLaunchCooperativeKernel((const void *)ms_kernel<T>, dim3(blocks),
                                         dim3(MS_THREADS), args, 0, s));
     note_launch();
     return GB_OK;
