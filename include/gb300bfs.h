@@ -225,8 +225,8 @@ gb_status graph_prepare_batched(gb_graph *g, gb_stream s);
  *                      in units of 16 (3 trades register spills for more
  *                      warps; 1 makes the per-level grid barrier cheaper).
  *                      With 1 and 2 the grid also follows the graph: graphs
- *                      of up to 100 * 2^20 column entries run on at most one
- *                      block per SM, small ones on fewer. */
+ *                      of fewer than 2^22 vertices run on at most one block
+ *                      per SM, small ones on fewer. */
 typedef struct gb_bfs_options {
     int canonical_parents;
     double alpha;

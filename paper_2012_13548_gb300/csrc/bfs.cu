@@ -47,8 +47,7 @@
 namespace gb {
 namespace {
 
-constexpr int BFS_THREADS = 512;    // threads of a block; BFS_WIDE of one when it has an SM to itself
-constexpr int BFS_WIDE = 1024;
+constexpr int BFS_THREADS = 512;
 constexpr int BIG_CHUNK = 128;      // edges per chunk of a big frontier vertex (one round)
 constexpr int BU_LANE_FIRST = 8;    // bottom-up: each lane probes this many neighbours itself
 constexpr int BU_WORDS = 2;         // bottom-up hub pass: visited words (or 32-entry list groups) per warp step
@@ -742,10 +741,10 @@ __device__ __forceinline__ void solo_min_parent(const BfsArgs &a, int64_t j, int
 // frontier is empty or too wide for it, when the rule asks for bottom-up, or
 // after a quarter of the wait limit, so that the waiting blocks stay within it.
 constexpr int SOLO_ROW = 2 * TD_E;
-template <int NT>
 __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l, int64_t qbase, int64_t qn,
                                             int64_t bnext_base, double mf, double mu, unsigned *Fn, LevelCtl *nxt)
 {
+    constexpr int NT = BFS_THREADS;
     const int tid = threadIdx.x;
     const int lane = (int)lane_id();
     const int warp = tid >> 5;
@@ -936,12 +935,10 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
     // the barrier that follows returns the buffers to the warps
 }
 
-// NT threads per block, MINB blocks per SM the register budget is sized for:
-// 2 x 512 or 1 x 1024 (64 registers, no spills), or 3 x 512 (40 registers,
-// more warps to hide latency).  One block of 1024 threads per SM keeps as many
-// warps as two of 512 but halves the arrivals at every level barrier.
-template <int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
+// MINB: the blocks per SM that the register budget is sized for, 2 (64 registers) or 3
+// (40 registers, spills, more warps to hide latency).
+template <int MINB>
+__global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
 {
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
@@ -952,7 +949,7 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
     WsHeader *h = a.hdr;
     const int32_t root = a.root;
     unsigned bar_target = grid_barrier_base(&h->bar);
-    __shared__ WarpBuf s_wb[NT / 32];
+    __shared__ WarpBuf s_wb[BFS_THREADS / 32];
     __shared__ unsigned long long s_mf;
     __shared__ LevelFlush s_lf;
     WarpBuf &wb = s_wb[threadIdx.x >> 5];
@@ -1051,7 +1048,7 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
         // Narrow levels: block 0 runs them alone, the others wait.
         if (td && qn <= SOLO_Q && (mf <= (double)SOLO_E || (mf <= (double)SOLO_E_SHORT && mf <= 4.0 * (double)qn))) {
             if (blockIdx.x == 0)
-                solo_levels<NT>(a, reinterpret_cast<SoloBuf &>(s_wb), l, qbase, qn, bnext_base, mf, mu, Fn, nxt);
+                solo_levels(a, reinterpret_cast<SoloBuf &>(s_wb), l, qbase, qn, bnext_base, mf, mu, Fn, nxt);
             if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_BFS_BAR)) return;
             l = (int)__ldcg(&h->solo.l) - 1;  // the loop adds one
             qbase = __ldcg(&h->solo.qbase);
@@ -1310,7 +1307,7 @@ __global__ void __launch_bounds__(NT, MINB) bfs_kernel(BfsArgs a)
                             nxt, qnext_base, bnext_base);
         }
         // end of level: flush the staged vertices and add the block's degree sum
-        flush_level(s_lf, wb, qn_buf, bn_buf, NT / 32, a, nxt, qnext_base, bnext_base);
+        flush_level(s_lf, wb, qn_buf, bn_buf, BFS_THREADS / 32, a, nxt, qnext_base, bnext_base);
         {
             const unsigned long long t = warp_sum(my_mf);
             my_mf = 0;
@@ -1442,7 +1439,7 @@ static int vec_ok(const BfsArgs &a)
 int bfs_pick_blocks(int num_sms, int minb)
 {
     int per_sm = 0;
-    const void *k = minb == 2 ? (const void *)bfs_kernel<BFS_THREADS, 2> : (const void *)bfs_kernel<BFS_THREADS, 3>;
+    const void *k = minb == 2 ? (const void *)bfs_kernel<2> : (const void *)bfs_kernel<3>;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, BFS_THREADS, 0) != cudaSuccess ||
         per_sm < 1)
         per_sm = 1;
@@ -1450,10 +1447,9 @@ int bfs_pick_blocks(int num_sms, int minb)
 }
 
 namespace {
-// How a search is launched: the kernel, its threads per block and its grid.
+// How a search is launched: the kernel and its grid.
 struct BfsLaunch {
     const void *kern;
-    int threads;
     int blocks;
 };
 
@@ -1463,23 +1459,25 @@ struct BfsLaunch {
 // (edgefactor 16) on 1 / 16 / 64 / 152 / 304 blocks of 512 threads: SCALE 10
 // 41 / 42 / 45 / 49 / 63; SCALE 14 92 / 59 / 61 / 67 / 82; SCALE 17 401 / 86 /
 // 72 / 77 / 97; SCALE 20 - / 240 / 122 / 107 / 132; SCALE 21 - / 486 / 212 /
-// 164 / 174; SCALE 22 - / 936 / 304 / 193 / 184.  Above kWideNnz two blocks'
-// worth of warps per SM are needed, as one block of 1024 threads.
-BfsLaunch pick_launch(int64_t nnz, const gb_bfs_options &o, int num_sms, int blocks2, int blocks3, int cap)
+// 164 / 174; SCALE 22 - / 936 / 304 / 193 / 184.  From 2^22 vertices the work asks for two blocks' worth
+// of warps per SM, whatever the edges: us for eight searches on 152 / 304 blocks of 512 / 152 of
+// 1024 threads, SCALE 22 with 46 M entries 1634 / 1521 / 1570, with 122 M 1725 / 1566 / 1598, SCALE 23 with 94 M
+// 2308 / 2068 / 2143; SCALE 21 with 60 M 1220 / 1254 / 1332, with 82 M 1039 / 1110 / -. (Blocks of
+// 1024 threads halved the barriers' arrivals; they lose since a block
+// takes one atomic per list at the end of a level.)
+BfsLaunch pick_launch(int64_t n, int64_t nnz, const gb_bfs_options &o, int num_sms, int blocks2, int blocks3, int cap)
 {
     constexpr int64_t kPerBlock = int64_t(1) << 15;  // CSR entries per block of a small graph
-    constexpr int64_t kWideNnz = int64_t(100) << 20;
+    constexpr int64_t kWideN = int64_t(1) << 22;
     const int one = std::max(1, std::min(blocks2, num_sms));
     if (o.blocks_per_sm == 3) {
         const int b = cap > 0 ? std::min(cap, blocks3) : blocks3;
-        return {(const void *)bfs_kernel<BFS_THREADS, 3>, BFS_THREADS, b};
+        return {(const void *)bfs_kernel<3>, b};
     }
-    if (o.blocks_per_sm == 2 && nnz >= kWideNnz && cap <= 0 && blocks2 >= 2 * num_sms)
-        return {(const void *)bfs_kernel<BFS_WIDE, 1>, BFS_WIDE, num_sms};
-    int b = o.blocks_per_sm == 1 || nnz < kWideNnz ? one : blocks2;
+    int b = o.blocks_per_sm == 1 || n < kWideN ? one : blocks2;
     if (cap > 0) b = std::min(b, cap);
     b = (int)std::min<int64_t>(b, std::max<int64_t>(1, (nnz + kPerBlock - 1) / kPerBlock));
-    return {(const void *)bfs_kernel<BFS_THREADS, 2>, BFS_THREADS, b};
+    return {(const void *)bfs_kernel<2>, b};
 }
 }  // namespace
 
@@ -1576,10 +1574,10 @@ gb_status bfs_impl(const gb_graph *g, int64_t root, int32_t *parent, int32_t *le
     a.vec_col = (reinterpret_cast<uintptr_t>(a.col) & 15u) == 0;  // allocated with col_alloc_entries
     a.timeout_ns = timeout_ns();
     void *args[] = {&a};
-    const BfsLaunch L = pick_launch(g->nnz, o, ctx->num_sms, ctx->bfs_blocks2, ctx->bfs_blocks, grid);
-    a.useg = open_list_seg(n, (int64_t)L.blocks * (L.threads / 32));
+    const BfsLaunch L = pick_launch(n, g->nnz, o, ctx->num_sms, ctx->bfs_blocks2, ctx->bfs_blocks, grid);
+    a.useg = open_list_seg(n, (int64_t)L.blocks * (BFS_THREADS / 32));
     if (a.useg == 0 || !a.hd) a.ulist = nullptr;  // the list walks read hd
-    GB_CUDA(cudaLaunchCooperativeKernel(L.kern, dim3(L.blocks), dim3(L.threads), args, 0, s));
+    GB_CUDA(cudaLaunchCooperativeKernel(L.kern, dim3(L.blocks), dim3(BFS_THREADS), args, 0, s));
     note_launch();
     return GB_OK;
 }
@@ -1672,7 +1670,7 @@ gb_status bfs_noalloc_impl(const int64_t *off, const int32_t *col, int64_t n, in
             GB_CUDA(cudaGetSymbolAddress((void **)&nd.scratch, g_noalloc_scratch));
             GB_CUDA(cudaDeviceGetAttribute(&nd.num_sms, cudaDevAttrMultiProcessorCount, dev));
             int per_sm = 0;
-            GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bfs_kernel<BFS_THREADS, 2>,
+            GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bfs_kernel<2>,
                                                                   BFS_THREADS, 0));
             nd.blocks = nd.num_sms * std::max(1, std::min(per_sm, 2));
             nd.ready = true;
@@ -1724,8 +1722,8 @@ gb_status bfs_noalloc_impl(const int64_t *off, const int32_t *col, int64_t n, in
     // the scratch holds no open list, so any grid will do; one block per SM at most
     gb_bfs_options one = o;
     one.blocks_per_sm = 1;
-    const BfsLaunch L = pick_launch(nnz, one, d.num_sms, d.blocks, d.blocks, 0);
-    GB_CUDA(cudaLaunchCooperativeKernel(L.kern, dim3(L.blocks), dim3(L.threads), args, 0, s));
+    const BfsLaunch L = pick_launch(n, nnz, one, d.num_sms, d.blocks, d.blocks, 0);
+    GB_CUDA(cudaLaunchCooperativeKernel(L.kern, dim3(L.blocks), dim3(BFS_THREADS), args, 0, s));
     note_launch();
     DevStatus hst;
     GB_CUDA(cudaMemcpyAsync(&hst, ws + kNaStatus, sizeof(hst), cudaMemcpyDeviceToHost, s));
