@@ -64,7 +64,8 @@ __device__ __forceinline__ unsigned ld_volatile_u32(const unsigned *p)
 // ---------------------------------------------------------------------------
 struct GridBarrier {
     unsigned count;
-    unsigned pad;
+    unsigned pad[31];  // a line of its own: the blocks that wait read it all the time, beside
+                       // the atomics on the level's counters of the blocks still at work
 };
 
 __device__ __forceinline__ void red_release_add_u32(unsigned *p, unsigned v)
@@ -94,11 +95,13 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned &target, DevS
         red_release_add_u32(&b->count, 1u);
         uint64_t t0 = 0;
         unsigned spins = 0;
-        while ((int)(ld_acquire_u32(&b->count) - target) < 0) {
-            if (status_code(st) != 0) {
-                ok = 0;
-                break;
-            }
+        for (;;) {
+            // both reads in flight together (an acquire holds back later reads, not
+            // earlier ones): the status after the barrier would cost it one more latency
+            const int code = status_code(st);
+            const bool passed = (int)(ld_acquire_u32(&b->count) - target) >= 0;
+            if (code != 0) ok = 0;
+            if (passed || !ok) break;
             // the clock from the first poll on, every eighth: a poll is an L2 round
             // trip, so a limit below a few microseconds runs out within them
             if ((++spins & 7u) == 1) {
@@ -113,7 +116,7 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned &target, DevS
             }
             __nanosleep(32);
         }
-        s_ok = ok && status_code(st) == 0;
+        s_ok = ok;
     }
     __syncthreads();
     return s_ok != 0;
