@@ -212,7 +212,7 @@ gb_status graph_prepare_batched(gb_graph *g, gb_stream s);
  *                      bottom-up -> top-down when the frontier shrinks below
  *                      n/beta vertices (Beamer et al., SC 2012).  A
  *                      frontier of hubs (16 times the mean degree) switches
- *                      at up to four times that ratio, at most 64.
+ *                      at 1.4 times that ratio.
  *   big_degree         frontier vertices of larger degree are split over the
  *                      whole grid in top-down steps.
  *   ms_alpha, ms_beta  the same switch for the multi-source BFS, on all edges

@@ -141,12 +141,12 @@ struct BfsArgs {
 // The switch to bottom-up, for a frontier of qn vertices with mf edges, mu edges
 // left unvisited.  alpha is the ratio at which it pays for a frontier of
 // ordinary vertices.  One of hubs, with HUB_MEAN times the mean degree and more, is
-// worth up to four times as much (a ratio of at most 64): an open vertex
+// worth 1.4 times as much (a ratio of at most 64): an open vertex
 // then meets the frontier at its first test, its highest-degree
 // neighbour, while every edge of a hub costs top-down its atomic whether or not it
 // finds a vertex.  SCALE 26, a frontier of 16,304 vertices and 150 M edges (just below 1/14): that
-// level 1.68 ms top-down, the search 2.32 ms; bottom-up 1.50 ms in all. At a ratio
-// of 128 another root's search went from 1.31 to 2.77 ms, so the line is 64.
+// level 1.68 ms top-down, 0.90 bottom-up, the search 2.32 -> 1.47 ms. Not further: SCALE 24,
+// 2,406 vertices with about 1/21, 0.28 ms top-down, 0.38 bottom-up.
 constexpr float HUB_MEAN = 16.0f;
 __device__ __forceinline__ bool go_bottom_up(float mf, float mu, float qn, const BfsArgs &a)
 {
@@ -156,7 +156,7 @@ __device__ __forceinline__ bool go_bottom_up(float mf, float mu, float qn, const
 void set_switch(BfsArgs &a, const gb_bfs_options &o)
 {
     a.alpha = (float)o.alpha;
-    a.alpha_hub = (float)std::max(o.alpha, std::min(4.0 * o.alpha, 64.0));
+    a.alpha_hub = (float)std::max(o.alpha, std::min(1.4 * o.alpha, 64.0));
     a.hub_deg = HUB_MEAN * (float)((double)a.nnz / (double)std::max<int64_t>(a.nnzv > 0 ? a.nnzv : a.n, 1));
     a.beta = (float)o.beta;
 }
