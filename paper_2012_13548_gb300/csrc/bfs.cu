@@ -548,8 +548,9 @@ __device__ __noinline__ void canonical_rescan(const BfsArgs &a, const unsigned *
 {
     const int lane = (int)lane_id();
     unsigned long long examined = 0;
-    for (int64_t i0 = gwarp * 32; i0 < qn; i0 += nwarps * 32) {
-        const int64_t i = i0 + lane;
+    const int rn = rows_per_warp(qn, nwarps);
+    for (int64_t i0 = gwarp * rn; i0 < qn; i0 += nwarps * rn) {
+        const int64_t i = lane < rn ? i0 + lane : qn;
         int32_t u = 0;
         int64_t s = 0, e = 0;
         if (i < qn && GB_OK_IDX(a.st, qbase + i, a.n, 226)) {
@@ -598,8 +599,9 @@ __device__ __noinline__ void canonical_edges(const BfsArgs &a, const unsigned *F
         for (int64_t j = cs + lane; j < e; j += 32)
             if (j >= su) edge(j, be.u);
     }
-    for (int64_t i0 = gwarp * 32; i0 < qn; i0 += nwarps * 32) {
-        const int64_t i = i0 + lane;
+    const int rn = rows_per_warp(qn, nwarps);
+    for (int64_t i0 = gwarp * rn; i0 < qn; i0 += nwarps * rn) {
+        const int64_t i = lane < rn ? i0 + lane : qn;
         int32_t u = 0;
         int64_t s = 0, d = 0;
         if (i < qn && GB_OK_IDX(a.st, qb + i, a.n, 231)) {
@@ -1116,9 +1118,10 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
                     }
                 }
             }
-            // (b) the other frontier vertices, 32 per warp, edges gathered as one stream
-            for (int64_t i0 = gwarp * 32; i0 < qn; i0 += nwarps * 32) {
-                const int64_t i = i0 + lane;
+            // (b) the other frontier vertices, up to 32 per warp, edges gathered as one stream
+            const int rn = rows_per_warp(qn, nwarps);
+            for (int64_t i0 = gwarp * rn; i0 < qn; i0 += nwarps * rn) {
+                const int64_t i = (int)lane < rn ? i0 + lane : qn;
                 int32_t u = 0;
                 int64_t s = 0, d = 0;
                 if (i < qn && GB_OK_IDX(a.st, qbase + i, a.n, 208)) {

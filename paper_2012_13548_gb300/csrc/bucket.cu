@@ -412,7 +412,7 @@ __global__ void bk_list_kernel(const BkDesc *__restrict__ desc, const unsigned *
             if (i == 0) ctl->nseg = nd;
         } else {
             if (d.count <= (unsigned)BK_CAP || rem <= low) continue;
-            const unsigned want = (d.count + BK_SPLIT - 1) / BK_SPLIT;
+            const unsigned want = (d.count - 1) / BK_SPLIT + 1;  // rounded up; a sum could pass 2^32
             bits = 32 - __clz(want - 1) + max(0, rem - field);
             bits = min(min(bits, BK_BITS), rem - low);
             gbase = atomicAdd(&ctl->npiece, 1u << bits);
@@ -427,7 +427,7 @@ __global__ void bk_list_kernel(const BkDesc *__restrict__ desc, const unsigned *
         sg.pr = d.pr;
         sg.pad = 0;
         segs[q] = sg;
-        const unsigned nt = (d.count + BK_TILE - 1) / BK_TILE;
+        const unsigned nt = d.count ? (d.count - 1) / BK_TILE + 1 : 0u;
         const unsigned t0 = atomicAdd(&ctl->ntile, nt);
         for (unsigned t = 0; t < nt; ++t) tiles[t0 + t] = make_uint2(q, t);
     }

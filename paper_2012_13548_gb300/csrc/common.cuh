@@ -155,6 +155,16 @@ __device__ __forceinline__ T warp_inclusive_scan(T v)
     return v;
 }
 
+// How many of `cnt` rows a warp takes at a time: 32 if that leaves none of
+// `nwarps` warps without, else fewer.  A warp streams its rows' edges in rounds of
+// dependent memory accesses, 2-3 us each, and a level lasts as long as its longest
+// warp: 32 rows of up to 256 entries in one warp while thousands had none were half of
+// a wide level's time.
+__device__ __forceinline__ int rows_per_warp(int64_t cnt, int64_t nwarps)
+{
+    return cnt >= 32 * nwarps ? 32 : (int)((cnt + nwarps - 1) / nwarps);
+}
+
 // Loads that bypass L1: data written by other blocks of the same kernel.
 __device__ __forceinline__ unsigned ldcg_u32(const unsigned *p) { return __ldcg(p); }
 __device__ __forceinline__ int ldcg_i32(const int *p) { return __ldcg(p); }

@@ -719,9 +719,10 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                     }
                 }
             }
-            // (1b) other active vertices, 32 per warp, adjacency gathered as one stream
-            for (int64_t i0 = gwarp * 32; i0 < na; i0 += nwarps * 32) {
-                const int64_t i = i0 + lane;
+            // (1b) other active vertices, up to 32 per warp, adjacency gathered as one stream
+            const int rn = rows_per_warp(na, nwarps);
+            for (int64_t i0 = gwarp * rn; i0 < na; i0 += nwarps * rn) {
+                const int64_t i = (int)lane < rn ? i0 + lane : na;
                 int64_t gv = 0, s = 0, d = 0, vo = 0;
                 int g = 0;
                 T f = 0;
@@ -774,8 +775,9 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
             // a level that does not grow, each also scans its row for its
             // smallest-id parents
             const bool by_rows = a.canonical && !by_edges;
-            for (int64_t i0 = gwarp * 32; i0 < nn; i0 += nwarps * 32) {
-                const int64_t i = i0 + lane;
+            const int rnn = by_rows ? rows_per_warp(nn, nwarps) : 32;
+            for (int64_t i0 = gwarp * rnn; i0 < nn; i0 += nwarps * rnn) {
+                const int64_t i = (int)lane < rnn ? i0 + lane : nn;
                 int64_t gu = 0, lu = 0, rs = 0, re = 0;
                 int g = 0;
                 T nw = 0;

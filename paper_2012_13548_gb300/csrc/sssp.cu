@@ -430,17 +430,6 @@ __device__ __forceinline__ int stream_owner(int64_t excl, int64_t k)
     return owner;
 }
 
-// How many of `cnt` rows a warp takes at a time: 32 if there are enough for every
-// warp, else fewer, so that all warps take part.  A step of a stream is a chain of
-// five memory latencies (entry, distance, minimum, stamp, queue), and a
-// round lasts as long as its longest warp: 32 rows of up to 1024 entries in
-// one warp while most had none took most of a round's time.
-__device__ __forceinline__ int rows_per_warp(int64_t cnt, int64_t nwarps)
-{
-    const int64_t r = (cnt + nwarps - 1) / nwarps;
-    return r > 32 ? 32 : (int)r;
-}
-
 // Warp-collective: relax the edges [so + (k - eo)] of a 32-row stream of
 // `total` slots (row starts s0, exclusive prefixes excl, distances du, ids u),
 // two slots per lane per step.
