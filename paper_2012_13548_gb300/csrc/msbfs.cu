@@ -680,19 +680,23 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
             for (int pass = 0; pass < (by_edges ? 2 : 1); ++pass) {
             // (1a) big active vertices in 256-edge chunks
             if (nc > 0) {
-                const int64_t per = (nc + nwarps - 1) / nwarps;
+                // eight rounds a chunk: where there are warps enough, each takes a half, a
+                // quarter or an eighth
+                const int ps = nc * 8 <= nwarps ? 3 : nc * 4 <= nwarps ? 2 : nc * 2 <= nwarps ? 1 : 0;
+                const int64_t per = ((nc << ps) + nwarps - 1) / nwarps;
                 const int64_t c0 = gwarp * per;
-                const int64_t c1 = c0 + per < nc ? c0 + per : nc;
+                const int64_t c1 = c0 + per < (nc << ps) ? c0 + per : (nc << ps);
                 if (c0 < c1) {
                     int64_t lo = 0, hi = nb;
                     while (hi - lo > 1) {
                         const int64_t mid = (lo + hi) >> 1;
-                        if ((int64_t)(__ldcg(&a.bigq[bbase + mid]) >> 32) <= c0) lo = mid;
+                        if ((int64_t)(__ldcg(&a.bigq[bbase + mid]) >> 32) <= c0 >> ps) lo = mid;
                         else hi = mid;
                     }
                     int64_t ow = lo;
                     unsigned long long be = __ldcg(&a.bigq[bbase + ow]);
-                    for (int64_t c = c0; c < c1; ++c) {
+                    for (int64_t cc = c0; cc < c1; ++cc) {
+                        const int64_t c = cc >> ps;
                         while (ow + 1 < nb && (int64_t)(__ldcg(&a.bigq[bbase + ow + 1]) >> 32) <= c) {
                             ++ow;
                             be = __ldcg(&a.bigq[bbase + ow]);
@@ -702,10 +706,11 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                         const MsGraph &G = s_g[g];
                         const int64_t lv = gv - G.voff;
                         const T f = ld_mask(&M[gv]);
-                        const int64_t s = G.off[lv] + (c - (int64_t)(be >> 32)) * MS_BIG_CHUNK;
+                        const int64_t s = G.off[lv] + (c - (int64_t)(be >> 32)) * MS_BIG_CHUNK +
+                                          ((cc & ((1 << ps) - 1)) * MS_BIG_CHUNK >> ps);
                         const int64_t eu = G.off[lv + 1];
-                        const int64_t e = s + MS_BIG_CHUNK < eu ? s + MS_BIG_CHUNK : eu;
-                        if (lane == 0) my_edges += (unsigned long long)(e - s);
+                        const int64_t e = s + (MS_BIG_CHUNK >> ps) < eu ? s + (MS_BIG_CHUNK >> ps) : eu;
+                        if (lane == 0 && e > s) my_edges += (unsigned long long)(e - s);
                         for (int64_t b = s; b < e; b += 32) {
                             const int64_t j = b + lane;
                             const bool valid = j < e;
