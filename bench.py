@@ -695,12 +695,14 @@ def batched_vs_plain(args, gb, torch, scale, dist):
 
 
 def kernel1_bytes(m, scale, nnz, n):
-    """Algorithmic HBM bytes of kernel 1: read tuples, write 2m keys, histogram
-    read, P sort passes (read+write 16 bytes per key), count + write passes
-    (read keys twice), write columns and offsets."""
+    """Algorithmic HBM bytes of kernel 1 by buckets: the tuples read twice (digit
+    counts, move); above 2^21 keys 8-byte keys written and read twice for the
+    second digit; 4-byte entries written, read and written by the bucket
+    sorts and read by the compaction; columns and offsets written.  The further
+    splits of long buckets are not counted."""
     nk = 2 * m
-    passes = (2 * scale + 7) // 8
-    return 16 * m + 8 * nk + 8 * nk + passes * 16 * nk + 16 * nk + 4 * nnz + 8 * (n + 1)
+    keys = 24 * nk if nk > 1 << 21 else 0
+    return 32 * m + keys + 16 * nk + 4 * nnz + 8 * (n + 1)
 
 
 def read_traffic(scale, alg_bytes_per_launch):
