@@ -640,11 +640,10 @@ struct SoloBuf {
     int32_t pre[SOLO_Q];
     struct {
         unsigned long long mf;
-        int cnt, dmax;
+        int cnt, dmax, stop;
     } c[3];
     unsigned long long big;
     int wsum[32];
-    int stop;
 };
 static_assert(sizeof(SoloBuf) <= sizeof(WarpBuf) * (BFS_THREADS / 32), "SoloBuf lies over the warp buffers");
 static_assert(SOLO_Q == 2 * BFS_THREADS, "two frontier vertices per thread in the prefix sum");
@@ -742,6 +741,9 @@ __device__ __forceinline__ void solo_min_parent(const BfsArgs &a, int64_t j, int
 // level claimed (a minimum), so no rescan follows.  The stretch ends when the
 // frontier is empty or too wide for it, when the rule asks for bottom-up, or
 // after a quarter of the wait limit, so that the waiting blocks stay within it.
+// Whether it ends is part of the level's record in the ring, as its counts are: one
+// flag for all levels could be set at the next level before a slow warp has read it for
+// this one, and the warps would part at the block's barriers.
 constexpr int SOLO_ROW = 2 * TD_E;
 __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l, int64_t qbase, int64_t qn,
                                             int64_t bnext_base, double mf, double mu, unsigned *Fn, LevelCtl *nxt)
@@ -761,10 +763,9 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
         sb.deg[0][i] = (int32_t)(a.off[u + 1] - s0);
     }
     if (tid == 0) {
-        sb.c[0].cnt = sb.c[0].dmax = 0;
+        sb.c[0].cnt = sb.c[0].dmax = sb.c[0].stop = 0;
         sb.c[0].mf = 0;
         sb.big = 0;
-        sb.stop = 0;
     }
     __syncthreads();
     unsigned long long edges = 0, touched = 0;
@@ -779,7 +780,7 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
         const int64_t qnext = qbase + qn;
         const int slot1 = slot == 2 ? 0 : slot + 1;
         if (tid == 0) {  // its last readers passed the previous level's barrier
-            sb.c[slot1].cnt = sb.c[slot1].dmax = 0;
+            sb.c[slot1].cnt = sb.c[slot1].dmax = sb.c[slot1].stop = 0;
             sb.c[slot1].mf = 0;
         }
         unsigned long long mfs = 0;
@@ -848,7 +849,7 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
             touched += (unsigned long long)q;
             if (l < kStatLevels || (x & 15) == 15) {
                 const uint64_t now = globaltimer_ns();
-                if (now - t_start > a.timeout_ns / 4) sb.stop = 1;
+                if (now - t_start > a.timeout_ns / 4) sb.c[slot].stop = 1;
                 if (l < kStatLevels) {
                     a.stats->level_ns[l] = now - h->t0;
                     a.stats->level_frontier[l] = qn;
@@ -872,7 +873,7 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
         const int64_t cnt = sb.c[slot].cnt;
         const unsigned long long nmf = sb.c[slot].mf;
         dm = sb.c[slot].dmax;
-        const bool stop = sb.stop != 0;
+        const bool stop = sb.c[slot].stop != 0;
         prev_qn = qn;
         qbase = qnext;
         qn = cnt;

@@ -19,9 +19,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture(autouse=True)
 def _reset_options():
-    gb.bfs_set_options(canonical_parents=0, big_degree=256, blocks_per_sm=2)
+    gb.bfs_set_options(canonical_parents=0, big_degree=256, blocks_per_sm=2, timeout_ms=5000.0)
     yield
-    gb.bfs_set_options(canonical_parents=0, big_degree=256, blocks_per_sm=2)
+    gb.bfs_set_options(canonical_parents=0, big_degree=256, blocks_per_sm=2, timeout_ms=5000.0)
     gb.gb_device_status()
 
 
@@ -84,4 +84,24 @@ def test_narrow_levels(name, big_degree, canonical):
         st = gb.bfs_last_stats()
         assert st["nlevels"] == l_ref.max() + 1 == st["td_levels"] + st["bu_levels"]
         assert st["reached"] == n
+    g.free()
+
+
+@pytest.mark.parametrize("name", ["path", "mesh", "wide_mesh"])
+@pytest.mark.parametrize("canonical", [0, 1])
+def test_stretches_that_the_wait_limit_cuts_short(name, canonical):
+    # a quarter of the limit ends a stretch, so each of these searches is many stretches
+    rng = np.random.default_rng(len(name))
+    n, pairs = GRAPHS[name](rng)
+    off, col, root = _csr(n, pairs, rng)
+    p_ref, l_ref = oracle.bfs(off, col, root)
+    g = gb.graph_from_csr(torch.as_tensor(off).cuda(), torch.as_tensor(col).cuda())
+    gb.bfs_set_options(canonical_parents=canonical, timeout_ms=1.0)
+    for _ in range(10):
+        parent, level = gb.bfs(g, root)
+        gb.gb_device_status()
+        assert np.array_equal(level.cpu().numpy(), l_ref)
+        if canonical:
+            assert np.array_equal(parent.cpu().numpy(), p_ref)
+    assert gb.bfs_validate(g, root, parent, level)["code"] == 0
     g.free()
