@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "barrier.h"
 #include "gb300bfs.h"
 #include "internal.h"
 
@@ -60,7 +61,8 @@ __device__ __forceinline__ unsigned ld_volatile_u32(const unsigned *p)
 // writes) and waits with acquire loads.  Every wait is bounded by
 // `timeout_ns` of the global timer: on expiry the block records
 // GB_ERR_TIMEOUT, and every block leaves early once any block has recorded an
-// error; grid_sync then returns false.
+// error; grid_sync then returns false.  An error recorded before a barrier stops
+// every block at that barrier at the latest (barrier.h).
 // ---------------------------------------------------------------------------
 struct GridBarrier {
     unsigned count;
@@ -96,12 +98,10 @@ __device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned &target, DevS
         uint64_t t0 = 0;
         unsigned spins = 0;
         for (;;) {
-            // both reads in flight together (an acquire holds back later reads, not
-            // earlier ones): the status after the barrier would cost it one more latency
-            const int code = status_code(st);
-            const bool passed = (int)(ld_acquire_u32(&b->count) - target) >= 0;
-            if (code != 0) ok = 0;
-            if (passed || !ok) break;
+            const BarrierLook look =
+                barrier_look([&] { return (int)(ld_acquire_u32(&b->count) - target) >= 0; }, [&] { return status_code(st); });
+            if (look == BARRIER_ERROR) ok = 0;
+            if (look != BARRIER_WAIT) break;
             // the clock from the first poll on, every eighth: a poll is an L2 round
             // trip, so a limit below a few microseconds runs out within them
             if ((++spins & 7u) == 1) {
