@@ -61,6 +61,11 @@ constexpr int BBUF = 32;            // per-warp buffer of discovered big-degree 
 constexpr int SOLO_Q = 1024;
 constexpr int SOLO_E = 1024;
 constexpr int SOLO_E_SHORT = 4096;
+// The other blocks wait for a whole stretch, which a quarter of the wait limit (ns)
+// ends: below SOLO_SHORT_WAIT the clock is read after every level, not every 16th (16
+// levels of 25 us, the longest in canonical mode, would leave nothing of such a limit), and
+// below SOLO_MIN_WAIT, where one level is a quarter, every level takes the grid.
+constexpr uint64_t SOLO_SHORT_WAIT = 1000000, SOLO_MIN_WAIT = 100000;
 constexpr int SITE_BFS_BAR = 20;
 constexpr int SITE_BFS_LEVELS = 21;
 
@@ -847,7 +852,7 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
         if (tid == 0) {
             edges += (unsigned long long)total;
             touched += (unsigned long long)q;
-            if (l < kStatLevels || (x & 15) == 15) {
+            if (l < kStatLevels || (x & 15) == 15 || a.timeout_ns < SOLO_SHORT_WAIT) {
                 const uint64_t now = globaltimer_ns();
                 if (now - t_start > a.timeout_ns / 4) sb.c[slot].stop = 1;
                 if (l < kStatLevels) {
@@ -1049,7 +1054,8 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
         }
 
         // Narrow levels: block 0 runs them alone, the others wait.
-        if (td && qn <= SOLO_Q && (mf <= (double)SOLO_E || (mf <= (double)SOLO_E_SHORT && mf <= 4.0 * (double)qn))) {
+        if (td && qn <= SOLO_Q && a.timeout_ns >= SOLO_MIN_WAIT &&
+            (mf <= (double)SOLO_E || (mf <= (double)SOLO_E_SHORT && mf <= 4.0 * (double)qn))) {
             if (blockIdx.x == 0)
                 solo_levels(a, reinterpret_cast<SoloBuf &>(s_wb), l, qbase, qn, bnext_base, mf, mu, Fn, nxt);
             if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_BFS_BAR)) return;

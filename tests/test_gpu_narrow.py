@@ -105,3 +105,24 @@ def test_stretches_that_the_wait_limit_cuts_short(name, canonical):
             assert np.array_equal(parent.cpu().numpy(), p_ref)
     assert gb.bfs_validate(g, root, parent, level)["code"] == 0
     g.free()
+
+
+@pytest.mark.parametrize("limit_ms", [0.2, 0.05])
+@pytest.mark.parametrize("canonical", [0, 1])
+def test_a_short_wait_limit_holds_for_levels_run_by_one_block(canonical, limit_ms):
+    # the other blocks wait for a whole stretch of levels of up to 25 us: it has to end
+    # well within their limit, as a level of the whole grid does
+    n, pairs = GRAPHS["wide_mesh"](None)
+    off, col, root = _csr(n, pairs, np.random.default_rng(8))
+    p_ref, l_ref = oracle.bfs(off, col, root)
+    g = gb.graph_from_csr(torch.as_tensor(off).cuda(), torch.as_tensor(col).cuda())
+    gb.bfs_set_options(canonical_parents=canonical)
+    gb.bfs(g, root)
+    gb.bfs_set_options(timeout_ms=limit_ms)
+    for _ in range(3):
+        parent, level = gb.bfs(g, root)
+        gb.gb_device_status()
+        assert np.array_equal(level.cpu().numpy(), l_ref)
+        if canonical:
+            assert np.array_equal(parent.cpu().numpy(), p_ref)
+    g.free()
