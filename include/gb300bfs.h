@@ -17,8 +17,9 @@
  *     passes.  The library owns gb_graph and gb_server objects.
  *   - Work is stream-ordered on the gb_stream given (a cudaStream_t; NULL is
  *     the legacy default stream).  Outputs are valid once that stream has
- *     synchronised.  Calls that must return a size computed on the device
- *     (graph_build_csr) synchronise the stream themselves and say so.
+ *     synchronised.  Calls that build a graph (or add to one) synchronise the
+ *     stream themselves after their last kernel and say so: the graph may be
+ *     used on any stream once they return.
  *   - Errors detected inside a kernel (an edge endpoint out of range, a
  *     bounded device-side wait that ran out) are recorded in a per-device
  *     status word; gb_device_status() synchronises a stream and returns and
@@ -128,12 +129,13 @@ gb_status kron_generate(int scale, int edgefactor, double a, double b, double c,
  * duplicate edges are dropped (Sec. 2.1 lets the kernels after generation
  * disregard them).  Offsets are int64 [n+1]: an empty row repeats the previous
  * offset and off[n] = nnz (Sec. 2.2).  Columns are int32 [nnz].
- * Synchronises `s` (the column count is needed on the host).  Returns
+ * Synchronises `s` (the column count is needed on the host, and the graph is
+ * complete on return).  Returns
  * GB_ERR_RANGE if an endpoint is outside [0, 2^scale).  *out receives a
  * library-owned graph; free it with graph_free.  Besides the CSR every graph
  * holds four arrays the search reads: a degree >= 1 bitmap (n/8 bytes), the
- * list of the vertices of degree >= 1 in ascending order (4 bytes each; the
- * first bottom-up level walks it), a hub per vertex (4 * n bytes: a neighbour
+ * list of the vertices of degree >= 1 in ascending order (held at its bound,
+ * 4 * min(n, nnz) bytes; the first bottom-up level walks it), a hub per vertex (4 * n bytes: a neighbour
  * of largest degree among the first 128 of its row, tested first by the
  * bottom-up step) and, for the bottom-up list walks, each hub again beside
  * the vertex's degree saturated at 65535 (8 * n bytes).  The column array is padded to a multiple of 4
@@ -191,7 +193,8 @@ gb_status graph_csr_view(const gb_graph *g, const int64_t **off, const int32_t *
  * lines.  bfs_batch searches a graph that has the copy on it, with the same
  * results (levels, and parents as original ids), and builds it by itself for
  * graphs of 2^25 or more vertices.  It adds 8 (n+1) + 4 nnz + 8 n bytes to the
- * graph until graph_free; GB_ERR_NOMEM leaves the graph as it was.  Part of
+ * graph until graph_free; GB_ERR_NOMEM leaves the graph as it was.
+ * Synchronises `s`, also when bfs_batch builds it.  Part of
  * kernel 1 in the sense of Sec. 4.3 (a structure built once per graph), so
  * not part of the searches' time.  Calls on one graph must not overlap. */
 gb_status graph_prepare_batched(gb_graph *g, gb_stream s);

@@ -582,7 +582,8 @@ gb_status build_batched_layout(gb_graph *g, cudaStream_t s)
                                                           std::min<int64_t>(n, g->nnz / (RL_LONG + 1) + 1),
                                                           tmpg.rl_col);
     note_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    // searches on other streams see the copy from here on
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e);
     g->rl_perm = tmpg.rl_perm;
     g->rl_inv = tmpg.rl_inv;
     g->rl_off = tmpg.rl_off;
@@ -615,16 +616,16 @@ gb_status build_graph_aux(gb_graph *g, cudaStream_t s)
     const int64_t per = (int64_t)rows * (HUB_THREADS / 32);  // rows a block takes at a time
     const unsigned hb = (unsigned)std::min<int64_t>((n + per - 1) / per, (int64_t)ctx->num_sms * 64);
     hub_kernel<<<hb, HUB_THREADS, 0, s>>>(g->off, g->col, key, n, g->nnz, g->hub, g->hd, rows, ctx->status);
-    note_launch(3);
+    // the list at its bound (a vertex of it has an entry), so that the one wait below comes
+    // after the last kernel: other streams may search the graph once this returns
+    GB_CUDA(gb::dmalloc_async(&g->nzl, std::max<int64_t>(std::min(n, g->nnz), 4) * sizeof(int32_t), s));
+    nzl_write_kernel<<<(unsigned)nb, NZL_THREADS, 0, s>>>(g->nz, nw, base, g->nzl);
+    note_launch(4);
     GB_CUDA(cudaGetLastError());
     unsigned long long nnzv = 0;
     GB_CUDA(cudaMemcpyAsync(&nnzv, base + nb, sizeof(nnzv), cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
     g->nnzv = (int64_t)nnzv;
-    GB_CUDA(gb::dmalloc_async(&g->nzl, std::max<int64_t>(g->nnzv, 4) * sizeof(int32_t), s));
-    nzl_write_kernel<<<(unsigned)nb, NZL_THREADS, 0, s>>>(g->nz, nw, base, g->nzl);
-    note_launch();
-    GB_CUDA(cudaGetLastError());
     return GB_OK;
 }
 

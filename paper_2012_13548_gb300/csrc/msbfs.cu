@@ -1128,7 +1128,7 @@ gb_status msbfs_impl(const gb_graph *g, const int64_t *roots, int k, int32_t *pa
 {
     // A graph whose frontier masks (8 n bytes) outgrow the L2 is searched on its
     // degree-ordered copy, built at the first batched call if not yet there.
-    if (!g->rl_col && g->n >= MS_LAYOUT_MIN_N) {
+    if (g->n >= MS_LAYOUT_MIN_N) {  // under its lock: another thread may be building it
         gb_status rc = prepare_batched(const_cast<gb_graph *>(g), s);
         if (rc != GB_OK) return rc;
     }
