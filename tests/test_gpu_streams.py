@@ -61,7 +61,7 @@ def test_shortest_paths_on_another_stream():
     off, col, wgt = oracle.csr_build_weighted(e_ref, w_ref, spec.scale)
     root = int(np.diff(off).argmax())
     d_ref, _ = oracle.sssp(off, col, wgt, root)
-    e, w = torch.as_tensor(e_ref).cuda(), torch.as_tensor(w_ref).cuda()
+    e, w = torch.as_tensor(e_ref).cuda(), torch.as_tensor(w_ref, dtype=torch.float32).cuda()
     dist = torch.empty(1 << spec.scale, dtype=torch.float64, device="cuda")
     parent = torch.empty(1 << spec.scale, dtype=torch.int32, device="cuda")
     build, search = torch.cuda.Stream(), torch.cuda.Stream()
