@@ -92,6 +92,13 @@ int64_t gb_sort_portion(void);
 gb_status gb_debug_fail_allocations(int64_t skip, int64_t count);
 int64_t gb_debug_live_allocations(void);
 
+/* How this thread's last graph build sorted its tuples (library bookkeeping, for
+ * tests; the paper has no counterpart).  *digits: 0 for the radix sort, else
+ * the digits of the bucket sort, 1 or 2.  *splits: how often the bucket sort
+ * had to split long buckets beyond the first time, in the build and in the
+ * weight-ordered rows together. */
+gb_status gb_debug_build_route(int *digits, int *splits);
+
 /* Synchronise `s`, then return and clear the device status word: GB_OK, or
  * the first GB_ERR_RANGE / GB_ERR_TIMEOUT a kernel recorded since the last
  * call. */

@@ -94,6 +94,7 @@ def lib():
             "gb_set_sort_portion": (ctypes.c_int, [_i64]),
             "gb_debug_fail_allocations": (ctypes.c_int, [_i64, _i64]),
             "gb_debug_live_allocations": (_i64, []),
+            "gb_debug_build_route": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
             "gb_sort_portion": (_i64, []),
             "gb_device_status": (ctypes.c_int, [_vp]),
             "kron_generate": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_double,
@@ -156,6 +157,7 @@ def exported_symbols():
     """Names of the C-ABI functions this binding wraps."""
     return ["gb_last_error", "gb_abi_version", "gb_kernel_launches", "gb_set_sort_portion",
             "gb_sort_portion", "gb_debug_fail_allocations", "gb_debug_live_allocations",
+            "gb_debug_build_route",
             "gb_device_status", "kron_generate",
             "graph_build_csr", "graph_build_csr_counting", "graph_from_csr", "graph_generate_csr",
             "graph_free", "graph_info", "graph_csr_view", "graph_prepare_batched",
@@ -268,6 +270,15 @@ def debug_fail_allocations(skip=0, count=0):
 def debug_live_allocations():
     """Device blocks the library holds now (allocated and not yet freed)."""
     return int(lib().gb_debug_live_allocations())
+
+
+def debug_build_route():
+    """How this thread's last graph build sorted its tuples: (digits, splits), digits 0
+    for the radix sort, 1 or 2 for the bucket sort, splits the times that long buckets
+    had to be split beyond the first."""
+    d, s = ctypes.c_int(), ctypes.c_int()
+    _check(lib().gb_debug_build_route(ctypes.byref(d), ctypes.byref(s)))
+    return d.value, s.value
 
 
 def gb_device_status(stream=None):

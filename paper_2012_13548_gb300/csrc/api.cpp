@@ -24,6 +24,7 @@ std::atomic<long long> g_live_allocs{0};  // device blocks the library holds
 std::mutex g_fail_mu;                      // injected allocation failures
 long long g_fail_skip = 0, g_fail_count = 0;
 thread_local std::string t_err;
+thread_local int t_digits = 0, t_splits = 0;  // of the last graph build
 std::mutex g_ctx_mu;
 std::vector<Context *> g_ctx;  // indexed by device
 
@@ -161,6 +162,12 @@ void set_error(const std::string &msg) { t_err = msg; }
 void note_launch(unsigned long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 unsigned long long launches() { return g_launches.load(std::memory_order_relaxed); }
 const std::string &last_error() { return t_err; }
+void note_build(int digits)
+{
+    t_digits = digits;
+    t_splits = 0;
+}
+void note_split() { ++t_splits; }
 
 gb_status cuda_fail(cudaError_t e, const char *what)
 {
@@ -290,6 +297,17 @@ gb_status gb_debug_fail_allocations(int64_t skip, int64_t count)
     return GB_OK;
 }
 
+gb_status gb_debug_build_route(int *digits, int *splits)
+{
+    if (!digits || !splits) {
+        set_error("gb_debug_build_route: NULL");
+        return GB_ERR_INVALID;
+    }
+    *digits = t_digits;
+    *splits = t_splits;
+    return GB_OK;
+}
+
 int64_t gb_debug_live_allocations(void) { return (int64_t)g_live_allocs.load(); }
 
 int64_t gb_sort_portion(void) { return sort_portion(); }
@@ -333,6 +351,7 @@ gb_status graph_build_csr(const int64_t *edges, int64_t m, int scale, gb_graph *
             return GB_ERR_INVALID;
         }
         *out = nullptr;
+        note_build(0);
         gb_graph *g = new gb_graph();
         gb_status rc = build_csr(edges, m, scale, g, as_stream(s));
         if (rc != GB_OK) {
@@ -354,6 +373,7 @@ gb_status graph_build_csr_counting(const int64_t *edges, int64_t m, int scale, g
             return GB_ERR_INVALID;
         }
         *out = nullptr;
+        note_build(0);
         gb_graph *g = new gb_graph();
         gb_status rc = build_csr_counting(edges, m, scale, g, as_stream(s));
         if (rc != GB_OK) {
@@ -387,6 +407,7 @@ gb_status graph_build_csr_weighted(const int64_t *edges, const float *w, int64_t
             return GB_ERR_INVALID;
         }
         *out = nullptr;
+        note_build(0);
         gb_graph *g = new gb_graph();
         gb_status rc = build_csr_weighted(edges, w, m, scale, g, as_stream(s));
         if (rc != GB_OK) {
@@ -489,6 +510,7 @@ gb_status graph_generate_csr(int scale, int edgefactor, double a, double b, doub
             return GB_ERR_INVALID;
         }
         *out = nullptr;
+        note_build(0);
         gb_graph *g = new gb_graph();
         gb_status rc = kron_csr(scale, edgefactor, a, b, c, seed_gen, seed_perm, g, as_stream(s));
         if (rc != GB_OK) {

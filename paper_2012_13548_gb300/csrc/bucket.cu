@@ -8,12 +8,16 @@
 //   1. from about 2 M keys up the buckets are split once more by the next digit.  What
 //      is left of a key then fits 32 bits (64 with a weight), so from here on
 //      an entry moves 4 bytes, not 8;
-//   2. buckets longer than CAP keys (rows of high degree) are split by further
-//      digits, as many bits as their length asks for, twice if need be;
+//   2. buckets longer than CAP keys (rows of high degree) are split by a further
+//      digit, as many bits as their length asks for;
 //   3. every bucket of at most CAP keys is sorted by one block in shared memory, by
 //      counting (count_sort below).  Repeated entries are marked, the kept ones
 //      counted per 4096 positions, and the first position of every row in the
-//      bucket's key range recorded;
+//      bucket's key range recorded.  What is still too long then (columns crowded
+//      in a part of their range) is split again, from the highest bit that its
+//      keys differ in, until nothing is (split_rest): every such split parts
+//      a bucket's keys, and one whose keys do not differ is a repeated pair, which
+//      needs no sort;
 //   4. a scan of those counts, then one pass that drops the marked entries and
 //      one that turns the row positions into offsets.
 //
@@ -25,11 +29,10 @@
 // one shared-memory atomic, a tile's place one global atomic per digit, and
 // three quarters of the key's bits never need a pass of their own.
 //
-// SCALE 26 (1.07 G tuples), whole kernel 1: 125.7 ms by the LSD sort, 65 ms by
-// buckets; SCALE 22 with weights (least weight per pair and weight-ordered rows): 48 -> 8.7 ms.
-//
-// Buckets that two extra splits leave longer than CAP (more than CAP copies of
-// a stretch of keys) raise a flag and the caller takes the LSD sort.
+// SCALE 26 (1.07 G tuples), whole kernel 1: 125.7 ms by the LSD sort, 54.5 ms by
+// buckets; SCALE 22 with weights (least weight per pair and weight-ordered rows): 48 -> 7.3 ms.
+// SCALE 20 with the vertices as the generator's quadrants number them, whose long rows
+// crowd at low columns: 1.92 and 1.46 ms (renumbered at random: 1.88 and 1.11).
 #include "bucket.h"
 
 #include <algorithm>
@@ -57,10 +60,11 @@ constexpr int LF_THREADS = 256;
 constexpr int LF_WARPS = LF_THREADS / 32;
 constexpr int WBITS = 25;  // bits of a weight in units of 2^-24
 constexpr int POS_TILE = 4096;
-constexpr int SITE_K1_RANGE = 10, SITE_SP_W = 45, SITE_BK_POS = 16;
+constexpr int SITE_BK_POS = 16;
 
 // A bucket: its place, its length, and which keys it holds.  Of its stored keys
-// the lowest `pr >> 56` bits count, the bits above them are `prefix`; of those
+// the lowest `pr >> 56` bits count, the bits above them are `prefix` (its lowest 56 bits;
+// (row, weight, column) keys may have more, whose rows the sort does not ask for); of those
 // key ranges of 2^rem keys it holds the `span` ones from `lo` on.
 struct BkDesc {
     uint32_t start, count;
@@ -68,9 +72,13 @@ struct BkDesc {
     uint32_t lo;
     uint16_t span, rem;
 };
-__device__ __forceinline__ uint64_t desc_pr(uint64_t prefix, int rem) { return prefix | ((uint64_t)rem << 56); }
+constexpr uint64_t kPrefixMask = (uint64_t(1) << 56) - 1;
+__device__ __forceinline__ uint64_t desc_pr(uint64_t prefix, int rem)
+{
+    return (prefix & kPrefixMask) | ((uint64_t)rem << 56);
+}
 __device__ __forceinline__ int desc_bits(uint64_t pr) { return (int)(pr >> 56); }
-__device__ __forceinline__ uint64_t desc_prefix(uint64_t pr) { return pr & ((uint64_t(1) << 56) - 1); }
+__device__ __forceinline__ uint64_t desc_prefix(uint64_t pr) { return pr & kPrefixMask; }
 __device__ __forceinline__ BkDesc whole_desc(uint32_t start, uint32_t count, uint64_t prefix, int rem)
 {
     BkDesc d;
@@ -89,23 +97,16 @@ struct BkSeg {
     uint32_t start, count, gbase;
     uint16_t bits, shift;
     uint64_t pr;
-    uint64_t pad;
+    unsigned long long differ;  // the bits that its keys differ in (split_rest)
 };
 
 struct BkCtl {
-    unsigned nseg, ntile, npiece, ndesc, overflow, pad[3];
+    unsigned nseg, ntile, npiece, ndesc, overflow, pad[3];  // overflow: pieces too long for a sort
 };
 
 __device__ __forceinline__ uint64_t low_mask(int bits)
 {
     return bits >= 64 ? ~uint64_t(0) : (uint64_t(1) << bits) - 1;
-}
-
-__device__ __forceinline__ uint32_t weight_units_or0(float w)
-{
-    if (!(w > 0.0f && w <= 1.0f)) return 0u;
-    const uint32_t k = __float2uint_rn(w * 16777216.0f);
-    return k < 1u ? 1u : k;
 }
 
 // ---- step 0 ---------------------------------------------------------------
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(BK_THREADS, 2) bk_part0_kernel(const int64_t *
             bin[2 * j] = ok ? (int)(a >> sh) : -1;
             bin[2 * j + 1] = ok ? (int)(b >> sh) : -1;
             if (WEIGHTED) {
-                uint32_t wu = weight_units_or0(w[j]);
+                uint32_t wu = weight_units(w[j]);
                 if (wu == 0u) {
                     record_error(st, GB_ERR_RANGE, SITE_SP_W, (long long)(t * TUP + j * BK_THREADS + threadIdx.x));
                     wu = 1u;
@@ -391,10 +392,19 @@ __global__ void __launch_bounds__(BK_THREADS, 2) bk_part0_kernel(const int64_t *
 
 // Lists the buckets to split and the tiles that cover them.  forced > 0: all of
 // them by that many bits, the pieces of bucket i at i << forced; else those
-// longer than BK_CAP, down to single rows (`field` bits hold what is not the
+// longer than BK_CAP.  BY_LENGTH: down to single rows (`field` bits hold what is not the
 // row) and from there by as many bits as bring a row of the bucket's length to
 // BK_SPLIT keys: long buckets are long by one row as a rule, and bits of the row
-// do not split it.  low: bits that do not tell entries apart.
+// do not split it.  BY_DIFFERENCE: by bits that bk_digit_kernel chooses.  low: bits
+// that do not tell entries apart.
+constexpr int BY_LENGTH = 0, BY_DIFFERENCE = -1;
+// Bits that bring `count` keys to BK_SPLIT a piece, if they spread evenly.
+__device__ __forceinline__ int split_bits(unsigned count)
+{
+    const unsigned want = (count - 1) / BK_SPLIT + 1;  // rounded up; a sum could pass 2^32
+    return 32 - __clz(want - 1);
+}
+
 __global__ void bk_list_kernel(const BkDesc *__restrict__ desc, const unsigned *__restrict__ ndesc_dev, unsigned ndesc,
                                int forced, int field, int low, BkSeg *__restrict__ segs, uint2 *__restrict__ tiles,
                                BkCtl *__restrict__ ctl)
@@ -403,19 +413,20 @@ __global__ void bk_list_kernel(const BkDesc *__restrict__ desc, const unsigned *
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < nd; i += gridDim.x * blockDim.x) {
         const BkDesc d = desc[i];
         const int rem = desc_bits(d.pr);
-        int bits;
-        unsigned gbase, q;
-        if (forced) {
+        int bits = 0;
+        unsigned gbase = 0, q;
+        if (forced > 0) {
             bits = forced;
             gbase = i << forced;
             q = i;
             if (i == 0) ctl->nseg = nd;
         } else {
             if (d.count <= (unsigned)BK_CAP || rem <= low) continue;
-            const unsigned want = (d.count - 1) / BK_SPLIT + 1;  // rounded up; a sum could pass 2^32
-            bits = 32 - __clz(want - 1) + max(0, rem - field);
-            bits = min(min(bits, BK_BITS), rem - low);
-            gbase = atomicAdd(&ctl->npiece, 1u << bits);
+            if (forced == BY_LENGTH) {
+                bits = split_bits(d.count) + max(0, rem - field);
+                bits = min(min(bits, BK_BITS), rem - low);
+                gbase = atomicAdd(&ctl->npiece, 1u << bits);
+            }
             q = atomicAdd(&ctl->nseg, 1u);
         }
         BkSeg sg;
@@ -425,11 +436,69 @@ __global__ void bk_list_kernel(const BkDesc *__restrict__ desc, const unsigned *
         sg.bits = (uint16_t)bits;
         sg.shift = (uint16_t)(rem - bits);
         sg.pr = d.pr;
-        sg.pad = 0;
+        sg.differ = 0;
         segs[q] = sg;
         const unsigned nt = d.count ? (d.count - 1) / BK_TILE + 1 : 0u;
         const unsigned t0 = atomicAdd(&ctl->ntile, nt);
         for (unsigned t = 0; t < nt; ++t) tiles[t0 + t] = make_uint2(q, t);
+    }
+}
+
+// The bits in which the keys of every listed bucket differ from its first.  A block a tile.
+template <typename K>
+__global__ void __launch_bounds__(BK_THREADS) bk_differ_kernel(const K *__restrict__ keys, BkSeg *__restrict__ segs,
+                                                               const uint2 *__restrict__ tiles,
+                                                               const BkCtl *__restrict__ ctl)
+{
+    const unsigned nt = ctl->ntile;
+    for (unsigned t = blockIdx.x; t < nt; t += gridDim.x) {
+        const uint2 tl = tiles[t];
+        const uint32_t start = segs[tl.x].start, count = segs[tl.x].count;
+        const K first = keys[start];
+        const unsigned o0 = tl.y * BK_TILE, left = count - o0;
+        uint64_t d = 0;
+#pragma unroll
+        for (int j = 0; j < BK_ITEMS; ++j) {
+            const unsigned i = j * BK_THREADS + threadIdx.x;
+            if (i < left) d |= (uint64_t)(keys[start + o0 + i] ^ first);
+        }
+        const unsigned lo = __reduce_or_sync(kFull, (unsigned)d), hi = __reduce_or_sync(kFull, (unsigned)(d >> 32));
+        if ((threadIdx.x & 31) == 0 && (lo | hi)) atomicOr(&segs[tl.x].differ, ((unsigned long long)hi << 32) | lo);
+    }
+}
+
+// The digit of every listed bucket: from the highest bit that its keys differ in, eight
+// times as many pieces as its length asks for (a first split by length
+// left it crowded), none if only the bits that do not count differ.  What its keys share above the
+// digit goes into its prefix; rawoff (if given): the rows that begin in the part of its
+// key range left out so are empty, and lie before or after all its keys.
+template <typename K>
+__global__ void bk_digit_kernel(const K *__restrict__ keys, BkSeg *__restrict__ segs, BkCtl *__restrict__ ctl, int low,
+                                int scale, unsigned *__restrict__ rawoff)
+{
+    const unsigned nseg = ctl->nseg;
+    for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < nseg; q += gridDim.x * blockDim.x) {
+        BkSeg sg = segs[q];
+        const int rem = desc_bits(sg.pr);
+        const unsigned long long differ = sg.differ & low_mask(rem) & ~low_mask(low);
+        const int top = differ ? 64 - __clzll((long long)differ) : low;
+        const int bits = min(min(split_bits(sg.count) + 3, BK_BITS), top - low);
+        const uint64_t old = desc_prefix(sg.pr);
+        const uint64_t pre = (old << (rem - top)) | (((uint64_t)keys[sg.start] & low_mask(rem)) >> top);
+        if (rawoff) {  // a key counts the pairs (u, v) from here on
+            const uint64_t vmask = low_mask(scale);
+            const uint64_t lo = old << (rem - low), hi = lo + (uint64_t(1) << (rem - low));
+            const uint64_t nlo = pre << (top - low), nhi = nlo + (uint64_t(1) << (top - low));
+            for (uint64_t r = (lo + vmask) >> scale; r < (hi + vmask) >> scale; ++r) {
+                if (r << scale <= nlo) rawoff[r] = sg.start;
+                else if (r << scale >= nhi) rawoff[r] = sg.start + sg.count;
+            }
+        }
+        sg.pr = desc_pr(pre, top);
+        sg.bits = (uint16_t)bits;
+        sg.shift = (uint16_t)(top - bits);
+        sg.gbase = atomicAdd(&ctl->npiece, 1u << bits);
+        segs[q] = sg;
     }
 }
 
@@ -637,7 +706,7 @@ struct LeafArgs {
     unsigned ndesc;
     const unsigned *ndesc2;      // and *ndesc2 pieces of the longer ones, read from src2
     int scale;
-    BkCtl *ctl2;           // its overflow is set if a piece is too long for a sort here
+    BkCtl *ctl2;           // its overflow counts the pieces too long for a sort here
     unsigned *tile_cnt;    // kept entries per POS_TILE positions
     unsigned *rawoff;      // [n + 1] first position of every row
     uint2 *wadj;           // MODE 2
@@ -836,7 +905,7 @@ __global__ void __launch_bounds__(LF_THREADS, sizeof(K) == 4 ? 6 : 4) bk_leaf_ke
         const int bits = desc_bits(d.pr), rem = d.rem;
         const bool big = d.count > (unsigned)BK_CAP;
         if (big && rem > LOW) {
-            if (piece && tid == 0) a.ctl2->overflow = 1;
+            if (piece && tid == 0) atomicAdd(&a.ctl2->overflow, 1u);
             continue;
         }
         Leaf<K> lf;
@@ -935,7 +1004,7 @@ struct BkResult {
     DevStatus status;
 };
 
-// base[i] = kept entries before tile i; their total, whether pieces are left that
+// base[i] = kept entries before tile i; their total, how many pieces are left that
 // need a further split, and the device status to *res.
 __global__ void __launch_bounds__(PS_THREADS) bk_posscan_kernel(const unsigned *__restrict__ cnt, unsigned nt,
                                                                 const unsigned *__restrict__ sums,
@@ -1117,20 +1186,28 @@ struct Level {
     BkCtl *ctl = nullptr;
 };
 
+// rawoff: BY_DIFFERENCE only.
 template <typename KIN, typename KOUT>
 gb_status split(Context *ctx, const Level &lv, const BkDesc *desc, const unsigned *ndesc_dev, unsigned ndesc, int forced,
-                int field, int low, int64_t nk, const KIN *in, KOUT *out, cudaStream_t s)
+                int field, int low, int64_t nk, const KIN *in, KOUT *out, cudaStream_t s, int scale = 0,
+                unsigned *rawoff = nullptr)
 {
     const int sms = ctx->num_sms;
     const int64_t most = ndesc_dev ? nk / (BK_SPLIT / 2) + 2 : (int64_t)ndesc;
     const int lb = (int)std::max<int64_t>(1, std::min<int64_t>((most + 255) / 256, sms * 4));
     bk_list_kernel<<<lb, 256, 0, s>>>(desc, ndesc_dev, ndesc, forced, field, low, lv.segs, lv.tiles, lv.ctl);
-    const int64_t tiles = nk / BK_TILE + 1 + (forced ? (int64_t)ndesc : nk / BK_CAP);
+    const int64_t tiles = nk / BK_TILE + 1 + (forced > 0 ? (int64_t)ndesc : nk / BK_CAP);
     const int hb = (int)std::min<int64_t>(tiles, sms * 4), pb = (int)std::min<int64_t>(tiles, sms * 2);
-    const int64_t nseg = forced ? (int64_t)ndesc : nk / BK_CAP + 1;
+    const int64_t nseg = forced > 0 ? (int64_t)ndesc : nk / BK_CAP + 1;
+    if (forced == BY_DIFFERENCE) {
+        bk_differ_kernel<KIN><<<hb, BK_THREADS, 0, s>>>(in, lv.segs, lv.tiles, lv.ctl);
+        bk_digit_kernel<KIN><<<(int)std::min<int64_t>((nseg + 255) / 256, sms * 4), 256, 0, s>>>(in, lv.segs, lv.ctl, low,
+                                                                                             scale, rawoff);
+        note_launch(2);
+    }
     bk_hist_kernel<KIN><<<hb, BK_THREADS, 0, s>>>(in, lv.segs, lv.tiles, lv.ctl, lv.cnt);
     bk_scan_kernel<<<(int)std::min<int64_t>(nseg, sms * 8), SC_THREADS, 0, s>>>(
-        lv.segs, lv.ctl, forced == 0, lv.cnt, lv.cursor, lv.desc);
+        lv.segs, lv.ctl, forced <= 0, lv.cnt, lv.cursor, lv.desc);
     constexpr int smem = PartShared<KOUT, sizeof(KIN) != sizeof(KOUT)>::bytes;
     GB_CUDA(smem_limit(bk_part_kernel<KIN, KOUT>, smem));
     bk_part_kernel<KIN, KOUT><<<pb, BK_THREADS, smem, s>>>(in, lv.segs, lv.tiles, lv.ctl, lv.cursor, out, (unsigned)nk,
@@ -1203,10 +1280,63 @@ Level level_at(unsigned char *b, const LevelPlan &p)
     return l;
 }
 
+// Why by the bits that differ: splits at fixed digits took 10 bits whether or not keys
+// differed in them, gave up after two, and the LSD sort began anew (SCALE 20 as
+// drawn 3.1 ms; unit weights beside a row of 10^5, whose weight bits are all
+// equal, 6.6 ms, now 3.2).  Where length alone asks for a second split (rows beyond
+// 2^10 pieces) a turn costs 20 us more than a third fixed digit did, for its two
+// launches more.
+// What the sorts of `from`'s pieces left because it was too long, `left` pieces with
+// their keys in ka: split from the bits they differ in and sorted into kb, until nothing is left.
+// Every turn a piece gives up at least the bit that parts its keys, so there are at most 64.
+// look(ctl, &left): waits for the stream and reads ctl's overflow.
+template <typename K, int MODE, typename Look>
+gb_status split_rest(Context *ctx, LeafArgs la, Level from, unsigned left, int low, int64_t nk, K *ka, K *kb,
+                     Look look, cudaStream_t s)
+{
+    const int64_t desc_x = nk / (BK_SPLIT / 2) + 2;  // as many descriptors as `from` has
+    Scratch tmp(s);
+    unsigned char *prev = nullptr;
+    K *in = ka, *out = kb;
+    for (int turn = 0; left; ++turn) {
+        if (turn == 64) {
+            set_error("kernel 1: a bucket that no digit splits");
+            return GB_ERR_CUDA;
+        }
+        // bk_digit_kernel takes less than 1/64 as many pieces as keys
+        const int64_t pieces = std::min<int64_t>(nk / 64 + 8, (int64_t)left << BK_BITS);
+        Arena ar;
+        LevelPlan p = plan_zeroed(ar, pieces);
+        const size_t zeroed = ar.used;
+        plan_rest(ar, p, left, nk / BK_TILE + 1 + left, pieces, desc_x);
+        unsigned char *ws = nullptr;
+        GB_CUDA(tmp.alloc(&ws, ar.used));
+        GB_CUDA(cudaMemsetAsync(ws, 0, zeroed, s));
+        const Level lv = level_at(ws, p);
+        gb_status rc = split<K, K>(ctx, lv, from.desc, &from.ctl->ndesc, 0, BY_DIFFERENCE, 0, low, nk, in, out, s, la.scale,
+                                   la.rawoff);
+        if (rc != GB_OK) return rc;
+        la.ndesc = 0;
+        la.desc2 = lv.desc;
+        la.ndesc2 = &lv.ctl->ndesc;
+        la.ctl2 = lv.ctl;
+        rc = leaves<K, MODE>(ctx, la, desc_x, out, out, kb, s);
+        if (rc != GB_OK) return rc;
+        rc = look(lv.ctl, &left);
+        if (rc != GB_OK) return rc;
+        if (prev) GB_CUDA(tmp.drop(prev));
+        prev = ws;
+        from = lv;
+        std::swap(in, out);
+        note_split();
+    }
+    return GB_OK;
+}
+
 // Steps 0-4 for one key type.
 template <typename K, bool WEIGHTED>
 gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, const BucketPlan &bp, gb_graph *g,
-                bool *overflow, cudaStream_t s)
+                cudaStream_t s)
 {
     constexpr int MODE = WEIGHTED ? 1 : 0;
     constexpr int LOW = WEIGHTED ? WBITS : 0;
@@ -1219,7 +1349,7 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     const int64_t n0 = int64_t(1) << bp.p0, n1 = int64_t(1) << total_bits;
     const int rowbits = std::max(0, scale - total_bits);  // of a bucket after step 1
     const int64_t seg_x = nk / BK_CAP + 1, desc_x = nk / (BK_SPLIT / 2) + 2, tile_x = nk / BK_TILE + 1 + seg_x;
-    const int64_t piece2 = split_pieces(nk, rowbits), piece3 = split_pieces(nk, rowbits - BK_BITS);
+    const int64_t piece2 = split_pieces(nk, rowbits);
 
     Arena ar;
     const size_t o_cnt0 = ar.take(BK_BINS * 4);
@@ -1227,7 +1357,7 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     const size_t o_pos = ar.take((size_t)npos * 4 + 4);
     LevelPlan l1{};
     if (bp.p1) l1 = plan_zeroed(ar, n1);
-    LevelPlan l2 = plan_zeroed(ar, piece2), l3 = plan_zeroed(ar, piece3);
+    LevelPlan l2 = plan_zeroed(ar, piece2);
     const size_t zeroed = ar.used;
     const size_t o_cur0 = ar.take(BK_BINS * 4);
     const size_t o_desc0 = ar.take(BK_BINS * sizeof(BkDesc));
@@ -1238,7 +1368,6 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     const size_t o_kept = ar.take((size_t)npos * (POS_TILE / 32) * sizeof(uint2));
     if (bp.p1) plan_rest(ar, l1, n0, nk / BK_TILE + 1 + n0, n1, n1);
     plan_rest(ar, l2, seg_x, tile_x, piece2, desc_x);
-    plan_rest(ar, l3, seg_x, tile_x, piece3, desc_x);
 
     Scratch tmp(s);
     unsigned char *ws = nullptr;
@@ -1291,7 +1420,7 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     }
     // steps 2 and 3: the buckets of at most BK_CAP keys, and the pieces of the longer
     // ones, moved to ka and sorted back into their places in kb
-    const Level lv2 = level_at(ws, l2), lv3 = level_at(ws, l3);
+    const Level lv2 = level_at(ws, l2);
     LeafArgs la{};
     la.desc = leaf_desc;
     la.ndesc = (unsigned)n1;
@@ -1301,7 +1430,7 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     la.scale = scale;
     la.tile_cnt = reinterpret_cast<unsigned *>(ws + o_pos);
     la.rawoff = reinterpret_cast<unsigned *>(ws + o_raw);
-    rc = split<K, K>(ctx, lv2, leaf_desc, nullptr, (unsigned)n1, 0, field, LOW, nk, kb, ka, s);
+    rc = split<K, K>(ctx, lv2, leaf_desc, nullptr, (unsigned)n1, BY_LENGTH, field, LOW, nk, kb, ka, s);
     if (rc != GB_OK) return rc;
     rc = leaves<K, MODE>(ctx, la, n1 + desc_x, kb, ka, kb, s);
     if (rc != GB_OK) return rc;
@@ -1310,30 +1439,20 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     BkResult *res = reinterpret_cast<BkResult *>(ws + o_res);
     const unsigned psb = (unsigned)((npos + PS_CHUNK - 1) / PS_CHUNK);
     BkResult hr;
-    const auto positions = [&]() -> gb_status {
+    const auto positions = [&](const BkCtl *ctl, unsigned *left) -> gb_status {
         bk_possum_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums);
-        bk_posscan_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums, base, la.ctl2, ctx->status, res);
+        bk_posscan_kernel<<<psb, PS_THREADS, 0, s>>>(la.tile_cnt, (unsigned)npos, sums, base, ctl, ctx->status, res);
         note_launch(2);
         GB_CUDA(cudaGetLastError());
         GB_CUDA(cudaMemcpyAsync(&hr, res, sizeof(hr), cudaMemcpyDeviceToHost, s));
         GB_CUDA(cudaStreamSynchronize(s));
+        *left = hr.status.code == 0 ? hr.overflow : 0;  // an error: no further work on these keys
         return GB_OK;
     };
-    rc = positions();
+    unsigned left = 0;
+    rc = positions(lv2.ctl, &left);
+    if (rc == GB_OK) rc = split_rest<K, MODE>(ctx, la, lv2, left, LOW, nk, ka, kb, positions, s);
     if (rc != GB_OK) return rc;
-    if (hr.overflow) {
-        // rows of 64 K entries and more in one bucket: their pieces are split once more
-        rc = split<K, K>(ctx, lv3, lv2.desc, &lv2.ctl->ndesc, 0, 0, field, LOW, nk, ka, kb, s);
-        if (rc != GB_OK) return rc;
-        la.ndesc = 0;
-        la.desc2 = lv3.desc;
-        la.ndesc2 = &lv3.ctl->ndesc;
-        la.ctl2 = lv3.ctl;
-        rc = leaves<K, MODE>(ctx, la, desc_x, kb, kb, kb, s);
-        if (rc != GB_OK) return rc;
-        rc = positions();
-        if (rc != GB_OK) return rc;
-    }
     const DevStatus &hst = hr.status;
     const unsigned nnz = hr.nnz;
     if (hst.code != 0) {
@@ -1344,8 +1463,6 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
                                                 : "graph_build_csr: device error during the build");
         return (gb_status)hst.code;
     }
-    *overflow = hr.overflow != 0;
-    if (hr.overflow) return GB_OK;
     g->nnz = (int64_t)nnz;
     GB_CUDA(gb::dmalloc_async(&g->off, (n + 1) * sizeof(int64_t), s));
     GB_CUDA(gb::dmalloc_async(&g->col, col_alloc_entries(g->nnz) * sizeof(int32_t), s));
@@ -1379,43 +1496,38 @@ bool bucket_plan(int64_t m, int scale, bool weighted, BucketPlan *out)
     } else {
         b.p0 = std::max((p + 1) / 2, 2 * scale + low - 64);
         if (b.p0 > BK_BITS) return false;  // a weighted key does not fit 64 bits below the first digit
-        b.p1 = p - b.p0;
-        if (b.p1 < 1) {
-            b.p1 = 1;
-            if (b.p0 + 1 > 2 * scale) return false;
-        }
+        b.p1 = p - b.p0;                   // p > BK_BITS >= p0
     }
     *out = b;
     return true;
 }
 
 gb_status bucket_build(const int64_t *edges, const float *w, int64_t m, int scale, const BucketPlan &plan, gb_graph *g,
-                       bool *overflow, cudaStream_t s)
+                       cudaStream_t s)
 {
-    return w ? build<uint64_t, true>(edges, w, m, scale, plan, g, overflow, s)
-             : build<uint32_t, false>(edges, nullptr, m, scale, plan, g, overflow, s);
+    note_build(plan.p1 ? 2 : 1);
+    return w ? build<uint64_t, true>(edges, w, m, scale, plan, g, s)
+             : build<uint32_t, false>(edges, nullptr, m, scale, plan, g, s);
 }
 
-gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, bool *overflow, cudaStream_t s)
+bool bucket_order_fits(int64_t nnz) { return nnz >= 1 && nnz < (int64_t(1) << 32); }
+
+gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, cudaStream_t s)
 {
     Context *ctx = context();
-    *overflow = true;
     const int64_t nnz = g->nnz, n = g->n;
-    if (nnz < 1 || nnz >= (int64_t(1) << 32)) return GB_OK;
     // 2^q rows a bucket, BK_MEAN entries on average
     int q = 0;
     while (q < BK_ROWBITS && q + 1 < g->scale && (nnz >> (g->scale - q - 1)) <= BK_MEAN && q + 1 + WBITS + g->scale <= 60) ++q;
     const int field = WBITS + g->scale, rem = q + field;
-    if (rem > 64) return GB_OK;
     const unsigned nd = (unsigned)((n + (int64_t(1) << q) - 1) >> q);
     const int64_t seg_x = nnz / BK_CAP + 1, desc_x = nnz / (BK_SPLIT / 2) + 2, tile_x = nnz / BK_TILE + 1 + seg_x;
-    const int64_t piece2 = split_pieces(nnz, q), piece3 = split_pieces(nnz, q - BK_BITS);
+    const int64_t piece2 = split_pieces(nnz, q);
     Arena ar;
-    LevelPlan l2 = plan_zeroed(ar, piece2), l3 = plan_zeroed(ar, piece3);
+    LevelPlan l2 = plan_zeroed(ar, piece2);
     const size_t zeroed = ar.used;
     const size_t o_desc = ar.take((size_t)nd * sizeof(BkDesc));
     plan_rest(ar, l2, seg_x, tile_x, piece2, desc_x);
-    plan_rest(ar, l3, seg_x, tile_x, piece3, desc_x);
     Scratch tmp(s);
     unsigned char *ws = nullptr;
     uint64_t *ka = nullptr, *kb = nullptr;
@@ -1424,7 +1536,7 @@ gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, bool *overflow, cu
     GB_CUDA(tmp.alloc(&kb, (size_t)nnz));
     GB_CUDA(cudaMemsetAsync(ws, 0, zeroed, s));
     BkDesc *desc = reinterpret_cast<BkDesc *>(ws + o_desc);
-    const Level lv2 = level_at(ws, l2), lv3 = level_at(ws, l3);
+    const Level lv2 = level_at(ws, l2);
     bk_rows_kernel<<<(int)std::min<int64_t>((nd + 255) / 256, ctx->num_sms * 8), 256, 0, s>>>(g->off, n, q, rem, nd, desc);
     bk_rowkeys_kernel<<<ctx->num_sms * 8, 256, 0, s>>>(g->off, g->col, g->wgt, n, nnz, g->scale, q, kb);
     note_launch(2);
@@ -1437,27 +1549,18 @@ gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, bool *overflow, cu
     la.ctl2 = lv2.ctl;
     la.scale = g->scale;
     la.wadj = wadj;
-    gb_status rc = split<uint64_t, uint64_t>(ctx, lv2, desc, nullptr, nd, 0, field, 0, nnz, kb, ka, s);
+    gb_status rc = split<uint64_t, uint64_t>(ctx, lv2, desc, nullptr, nd, BY_LENGTH, field, 0, nnz, kb, ka, s);
     if (rc != GB_OK) return rc;
     rc = leaves<uint64_t, 2>(ctx, la, nd + desc_x, kb, ka, kb, s);
     if (rc != GB_OK) return rc;
-    unsigned ovf = 0;
-    GB_CUDA(cudaMemcpyAsync(&ovf, &lv2.ctl->overflow, sizeof(ovf), cudaMemcpyDeviceToHost, s));
-    GB_CUDA(cudaStreamSynchronize(s));
-    if (ovf) {
-        rc = split<uint64_t, uint64_t>(ctx, lv3, lv2.desc, &lv2.ctl->ndesc, 0, 0, field, 0, nnz, ka, kb, s);
-        if (rc != GB_OK) return rc;
-        la.ndesc = 0;
-        la.desc2 = lv3.desc;
-        la.ndesc2 = &lv3.ctl->ndesc;
-        la.ctl2 = lv3.ctl;
-        rc = leaves<uint64_t, 2>(ctx, la, desc_x, kb, kb, kb, s);
-        if (rc != GB_OK) return rc;
-        GB_CUDA(cudaMemcpyAsync(&ovf, &lv3.ctl->overflow, sizeof(ovf), cudaMemcpyDeviceToHost, s));
+    const auto look = [&](const BkCtl *ctl, unsigned *left) -> gb_status {
+        GB_CUDA(cudaMemcpyAsync(left, &ctl->overflow, sizeof(*left), cudaMemcpyDeviceToHost, s));
         GB_CUDA(cudaStreamSynchronize(s));
-    }
-    *overflow = ovf != 0;
-    return GB_OK;
+        return GB_OK;
+    };
+    unsigned left = 0;
+    rc = look(lv2.ctl, &left);
+    return rc == GB_OK ? split_rest<uint64_t, 2>(ctx, la, lv2, left, 0, nnz, ka, kb, look, s) : rc;
 }
 
 }  // namespace gb

@@ -16,13 +16,14 @@ struct BucketPlan {
 bool bucket_plan(int64_t m, int scale, bool weighted, BucketPlan *out);
 
 // The CSR (and, with w, the weights) of the tuples into g, and its auxiliary
-// arrays.  *overflow: some bucket stayed too long; nothing was built and the
-// caller takes the LSD sort.  Synchronises the stream.
+// arrays.  Synchronises the stream.
 gb_status bucket_build(const int64_t *edges, const float *w, int64_t m, int scale, const BucketPlan &plan, gb_graph *g,
-                       bool *overflow, cudaStream_t s);
+                       cudaStream_t s);
 
+// Whether the rows of nnz entries can be ordered by weight by buckets (fewer than 2^32).
+bool bucket_order_fits(int64_t nnz);
 // (column, weight) of every entry of g into wadj, each row by ascending weight
-// (ties by column).  *overflow as above.  Synchronises the stream.
-gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, bool *overflow, cudaStream_t s);
+// (ties by column).  The caller synchronises the stream.
+gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, cudaStream_t s);
 
 }  // namespace gb

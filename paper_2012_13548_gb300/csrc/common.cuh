@@ -52,6 +52,18 @@ __device__ __forceinline__ unsigned ld_volatile_u32(const unsigned *p)
     return *(volatile const unsigned *)p;
 }
 
+// Sites of kernel 1's input errors (DevStatus::where): an endpoint, a weight.
+constexpr int SITE_K1_RANGE = 10, SITE_SP_W = 45;
+
+// Weight w in (0, 1] as units of 2^-24, rounded to the nearest unit and at
+// least one; 0 for a weight outside (0, 1] or NaN.
+__device__ __forceinline__ uint32_t weight_units(float w)
+{
+    if (!(w > 0.0f && w <= 1.0f)) return 0u;
+    const uint32_t k = __float2uint_rn(w * 16777216.0f);
+    return k < 1u ? 1u : k;
+}
+
 // ---------------------------------------------------------------------------
 // Software grid barrier for cooperative (all-blocks-resident) launches.
 // Arrivals only ever add to one counter: the k-th barrier of a launch is

@@ -1,8 +1,8 @@
 // Kernel 1 (Sec. 2.2): the undirected CSR graph from the Kronecker tuples.
 //
 // Tuples in memory are sorted by buckets (bucket.cu).  The steps below serve
-// the inputs that it does not take (SCALE 27 and more, 2^31 tuples and more,
-// buckets that stay too long), a caller's own sort portions, and the generator fused with kernel 1:
+// the inputs that it does not take (SCALE 27 and more, 2^31 tuples and more),
+// a caller's own sort portions, and the generator fused with kernel 1:
 //
 //   1. symmetrise: tuple (u,v) becomes keys (u << S | v) and (v << S | u),
 //      S = scale, so one key holds an ordered pair in 2*S contiguous bits;
@@ -32,7 +32,6 @@ namespace {
 constexpr int FIN_THREADS = 256;
 constexpr int FIN_ITEMS = 16;
 constexpr int FIN_TILE = FIN_THREADS * FIN_ITEMS;  // 4096 keys
-constexpr int SITE_K1_RANGE = 10;
 
 // Both directed keys of every tuple, and the digit counts of the radix
 // sort's passes over them (plan.passes of them; 0: none), so that the sort
@@ -701,11 +700,8 @@ gb_status build_csr(const int64_t *edges, int64_t m, int scale, gb_graph *g, cud
     if (nk == 0) return empty_csr(g, s);
     // a caller that set a portion size asks for the LSD sort in portions
     BucketPlan bp;
-    if (sort_portion() == SORT_PORTION_DEFAULT && bucket_plan(m, scale, false, &bp)) {
-        bool overflow = false;
-        const gb_status rc = bucket_build(edges, nullptr, m, scale, bp, g, &overflow, s);
-        if (rc != GB_OK || !overflow) return rc;
-    }
+    if (sort_portion() == SORT_PORTION_DEFAULT && bucket_plan(m, scale, false, &bp))
+        return bucket_build(edges, nullptr, m, scale, bp, g, s);
     uint64_t *k0 = nullptr, *k1 = nullptr;
     unsigned long long *hist = nullptr;
     SortPlan plan = sort_plan(0, 2 * scale);

@@ -49,6 +49,11 @@ gb_status cuda_fail(cudaError_t e, const char *what);
 void note_launch(unsigned long long n = 1);
 unsigned long long launches();
 
+// What this thread's last graph build did (gb_debug_build_route): a build starts
+// with note_build(0), the bucket sort notes its digits and every further split.
+void note_build(int digits);
+void note_split();
+
 // Process-wide BFS options.
 gb_bfs_options &options();
 uint64_t timeout_ns();

@@ -43,9 +43,10 @@
 // Kernel 1's weights: graph_build_csr_weighted builds the CSR as kernel 1 does
 // and then gives each entry the least weight among the tuples joining its pair
 // (the bucket sort of bucket.cu carries the weight below the key, and sorts the rows
-// once more by weight; where it does not serve, each tuple finds its two entries by
-// bisection of the sorted rows and the weight-sorted rows come from one radix sort of
-// (row << 25 | weight) keys carrying the columns).
+// once more by weight; where the key and the weight do not fit it, each tuple finds its two
+// entries by bisection of the sorted rows, and for 2^32 entries and more, or a caller's own
+// sort portions, the weight-sorted rows come from one radix sort of (row << 25 | weight) keys
+// carrying the columns).
 #include "bucket.h"
 #include "common.cuh"
 #include "internal.h"
@@ -65,20 +66,11 @@ constexpr int64_t SP_LIGHT = 128;  // edges per chunk of a light prefix
 constexpr unsigned long long SP_INF = ~0ull;
 constexpr double kUnit = 5.9604644775390625e-8;  // 2^-24: one weight unit
 constexpr int SITE_SP_BAR = 40, SITE_SP_NEAR = 41, SITE_SP_FAR = 42, SITE_SP_BIGQ = 43,
-              SITE_SP_ROUNDS = 44, SITE_SP_W = 45, SITE_SP_FIND = 46;
+              SITE_SP_ROUNDS = 44, SITE_SP_FIND = 46;
 
 // ---------------------------------------------------------------------------
 // Kernel 1's weights
 // ---------------------------------------------------------------------------
-
-// Weight w in (0, 1] as units of 2^-24, rounded to the nearest unit and at
-// least one; 0 for a weight outside (0, 1] or NaN.
-__device__ __forceinline__ uint32_t weight_units(float w)
-{
-    if (!(w > 0.0f && w <= 1.0f)) return 0u;
-    const uint32_t k = __float2uint_rn(w * 16777216.0f);
-    return k < 1u ? 1u : k;
-}
 
 // Index of column v in the sorted row [lo, hi), or -1.
 __device__ __forceinline__ int64_t find_in_row(const int32_t *__restrict__ col, int64_t lo, int64_t hi,
@@ -1107,7 +1099,7 @@ int sssp_pick_blocks(int num_sms)
 
 namespace {
 
-// Kernel 1 by the LSD sort, then each entry's least weight.
+// Kernel 1 without the weights, then each entry's least weight.
 gb_status attach_weights(const int64_t *edges, const float *w, int64_t m, int scale, gb_graph *g, cudaStream_t s)
 {
     gb_status rc = build_csr(edges, m, scale, g, s);
@@ -1142,28 +1134,24 @@ gb_status build_csr_weighted(const int64_t *edges, const float *w, int64_t m, in
     Context *ctx = context();
     if (!ctx) return GB_ERR_CUDA;
     BucketPlan bp;
-    bool overflow = true;
     const bool buckets = sort_portion() == SORT_PORTION_DEFAULT;
+    gb_status rc;
     if (buckets && bucket_plan(m, scale, true, &bp)) {
         g->n = int64_t(1) << scale;
         g->scale = scale;
         g->device = ctx->device;
         GB_CUDA(cudaMemsetAsync(ctx->status, 0, sizeof(DevStatus), s));
-        const gb_status rc = bucket_build(edges, w, m, scale, bp, g, &overflow, s);
-        if (rc != GB_OK) return rc;
+        rc = bucket_build(edges, w, m, scale, bp, g, s);
+    } else {
+        rc = attach_weights(edges, w, m, scale, g, s);
     }
-    if (overflow) {
-        const gb_status rc = attach_weights(edges, w, m, scale, g, s);
-        if (rc != GB_OK) return rc;
-    }
+    if (rc != GB_OK) return rc;
     const int64_t nnz = g->nnz;
     GB_CUDA(gb::dmalloc_async(&g->wadj, std::max<int64_t>(nnz, 4) * sizeof(uint2), s));
-    overflow = true;
-    if (buckets && nnz > 0) {
-        const gb_status rc = bucket_weight_order(g, g->wadj, &overflow, s);
+    if (buckets && bucket_order_fits(nnz)) {
+        rc = bucket_weight_order(g, g->wadj, s);
         if (rc != GB_OK) return rc;
-    }
-    if (overflow && nnz > 0) {
+    } else if (nnz > 0) {
         // the rows by ascending weight: one sort of (row << 25 | weight) keys with the columns
         uint64_t *k0 = nullptr, *k1 = nullptr, *ks = nullptr;
         uint32_t *v0 = nullptr, *v1 = nullptr, *vs = nullptr;
@@ -1184,6 +1172,7 @@ gb_status build_csr_weighted(const int64_t *edges, const float *w, int64_t m, in
     GB_CUDA(cudaStreamSynchronize(s));
     return GB_OK;
 }
+
 gb_status sssp_impl(const gb_graph *g, int64_t root, double delta, double *dist, int32_t *parent,
                     SsspDevStats *stats, cudaStream_t s)
 {
