@@ -226,8 +226,9 @@ gb_status graph_prepare_batched(gb_graph *g, gb_stream s);
  *   big_degree         frontier vertices of larger degree are split over the
  *                      whole grid in top-down steps.
  *   ms_alpha, ms_beta  the same switch for the multi-source BFS, on all edges
- *                      of the graph; where its masks fit the L2 it stays
- *                      top-down up to four times as many edges (to a ratio of 4).
+ *                      of the graph.  ms_alpha's default, 16, leaves the
+ *                      ratio to the library: 16, and 4 where the masks fit
+ *                      the L2 (64 MB); any other value is taken as it is.
  *   timeout_ms         limit of every device-side wait (grid barriers, the
  *                      radix-sort look-back); on expiry the kernel records
  *                      GB_ERR_TIMEOUT and returns.

@@ -33,7 +33,7 @@ gb_bfs_options g_opt = {
     14.0,    // alpha
     24.0,    // beta
     256,     // big_degree
-    16.0,    // ms_alpha
+    kMsAlphaDefault,  // ms_alpha
     32.0,    // ms_beta
     5000.0,  // timeout_ms
     2,       // blocks_per_sm

@@ -54,7 +54,8 @@ unsigned long long launches();
 void note_build(int digits);
 void note_split();
 
-// Process-wide BFS options.
+// Process-wide BFS options.  ms_alpha's default leaves the ratio to the library.
+constexpr double kMsAlphaDefault = 16.0;
 gb_bfs_options &options();
 uint64_t timeout_ns();
 

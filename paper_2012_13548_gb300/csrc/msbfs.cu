@@ -1010,15 +1010,15 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
 // bottom-up.  A top-down edge is one atomic on a mask, 0.05 ns while the masks
 // (`bytes` of them) stay in the L2, and a bottom-up level of few active vertices
 // reads nearly every entry to the end, 0.014 ns each: there the line lies
-// near 4, not ms_alpha's default of 16, whose place is graphs whose masks
+// near 4, not 16, whose place is graphs whose masks
 // do not fit.  SCALE 22, 64 roots, 4552 active vertices with 1/15 of
 // the edges: that level 1.80 ms bottom-up, 0.48 top-down (the call 5.29 -> 3.74 ms).
-// A lower ms_alpha is kept.  (In canonical mode the level costs twice as much
+// Only ms_alpha's default is read so: any other value is the ratio itself.  (In canonical mode the level costs twice as much
 // top-down, 0.94 ms, and the call still gains: 5.34 -> 4.27 ms.)
 constexpr int64_t MS_L2_MASKS = int64_t(64) << 20;
 float switch_ratio(const gb_bfs_options &o, int64_t bytes)
 {
-    return (float)(bytes <= MS_L2_MASKS ? std::min(o.ms_alpha, std::max(4.0, o.ms_alpha / 4.0)) : o.ms_alpha);
+    return (float)(o.ms_alpha == kMsAlphaDefault && bytes <= MS_L2_MASKS ? 4.0 : o.ms_alpha);
 }
 
 template <typename T>
