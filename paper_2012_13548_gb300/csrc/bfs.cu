@@ -74,7 +74,7 @@ constexpr int SITE_BFS_LEVELS = 21;
 #ifdef GB_CHECKED
 #define GB_OK_IDX(st, i, bound, site) \
     ((int64_t)(i) >= 0 && (int64_t)(i) < (int64_t)(bound) \
-         ? true : (record_error((st), GB_ERR_RANGE, (site), (long long)(i)), false))
+         ? true : (grid_error((st), GB_ERR_RANGE, (site), (long long)(i)), false))
 #else
 #define GB_OK_IDX(st, i, bound, site) true
 #endif
@@ -141,6 +141,7 @@ struct BfsArgs {
     int vec_out;  // parent, level, hub and the state bytes allow 16-byte vector access
     int vec_col;  // col is 16-byte aligned and padded to a multiple of 4 entries
     uint64_t timeout_ns;
+    int solo_q, solo_clock;  // see set_wait
 };
 
 // The switch to bottom-up, for a frontier of qn vertices with mf edges, mu edges
@@ -156,6 +157,15 @@ constexpr float HUB_MEAN = 16.0f;
 __device__ __forceinline__ bool go_bottom_up(float mf, float mu, float qn, const BfsArgs &a)
 {
     return mf * a.alpha > mu || (mf * a.alpha_hub > mu && mf > qn * a.hub_deg);
+}
+
+// The wait limit, and what follows from it for narrow levels: the widest frontier that one
+// block takes (none below SOLO_MIN_WAIT), and after which levels it reads the clock.
+void set_wait(BfsArgs &a)
+{
+    a.timeout_ns = timeout_ns();
+    a.solo_q = a.timeout_ns >= SOLO_MIN_WAIT ? SOLO_Q : -1;
+    a.solo_clock = a.timeout_ns < SOLO_SHORT_WAIT ? 0 : 15;
 }
 
 void set_switch(BfsArgs &a, const gb_bfs_options &o)
@@ -852,7 +862,7 @@ __device__ __forceinline__ void solo_levels(const BfsArgs &a, SoloBuf &sb, int l
         if (tid == 0) {
             edges += (unsigned long long)total;
             touched += (unsigned long long)q;
-            if (l < kStatLevels || (x & 15) == 15 || a.timeout_ns < SOLO_SHORT_WAIT) {
+            if (l < kStatLevels || (x & a.solo_clock) == a.solo_clock) {
                 const uint64_t now = globaltimer_ns();
                 if (now - t_start > a.timeout_ns / 4) sb.c[slot].stop = 1;
                 if (l < kStatLevels) {
@@ -956,7 +966,7 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
     const int64_t n = a.n, nw = a.nw;
     WsHeader *h = a.hdr;
     const int32_t root = a.root;
-    unsigned bar_target = grid_barrier_base(&h->bar);
+    grid_barrier_begin(&h->bar);
     __shared__ WarpBuf s_wb[BFS_THREADS / 32];
     __shared__ unsigned long long s_mf;
     __shared__ LevelFlush s_lf;
@@ -993,7 +1003,7 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
             a.bigq[0] = be;
         }
     }
-    if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_BFS_BAR)) return;
+    if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_BFS_BAR)) return;
     if (gtid == 0) {
         h->t0 = globaltimer_ns();
         a.stats->init_ns = 0;
@@ -1014,7 +1024,7 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
         const int64_t qn = (int64_t)ldcg_u64(&cur->qcnt);
         if (qn == 0) break;
         if (l > n) {
-            if (gtid == 0) record_error(a.st, GB_ERR_TIMEOUT, SITE_BFS_LEVELS, l);
+            if (gtid == 0) grid_error(a.st, GB_ERR_TIMEOUT, SITE_BFS_LEVELS, l);
             break;
         }
         const double mf = (double)ldcg_u64(&cur->mf);
@@ -1054,11 +1064,11 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
         }
 
         // Narrow levels: block 0 runs them alone, the others wait.
-        if (td && qn <= SOLO_Q && a.timeout_ns >= SOLO_MIN_WAIT &&
+        if (td && qn <= a.solo_q &&
             (mf <= (double)SOLO_E || (mf <= (double)SOLO_E_SHORT && mf <= 4.0 * (double)qn))) {
             if (blockIdx.x == 0)
                 solo_levels(a, reinterpret_cast<SoloBuf &>(s_wb), l, qbase, qn, bnext_base, mf, mu, Fn, nxt);
-            if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_BFS_BAR)) return;
+            if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_BFS_BAR)) return;
             l = (int)__ldcg(&h->solo.l) - 1;  // the loop adds one
             qbase = __ldcg(&h->solo.qbase);
             prev_qn = __ldcg(&h->solo.prev_qn);
@@ -1337,7 +1347,7 @@ __global__ void __launch_bounds__(BFS_THREADS, MINB) bfs_kernel(BfsArgs a)
         qbase += qn;
         bbase += nb;
         if (gtid == 0) atomicAdd(&h->acc[td ? 4 : 5], 1ull);
-        if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_BFS_BAR)) return;
+        if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_BFS_BAR)) return;
         if (gtid == 0 && l < kStatLevels) {
             const uint64_t now = globaltimer_ns();
             a.stats->level_ns[l] = now - h->t0;
@@ -1582,7 +1592,7 @@ gb_status bfs_impl(const gb_graph *g, int64_t root, int32_t *parent, int32_t *le
     a.canonical = o.canonical_parents;
     a.vec_out = vec_ok(a);
     a.vec_col = (reinterpret_cast<uintptr_t>(a.col) & 15u) == 0;  // allocated with col_alloc_entries
-    a.timeout_ns = timeout_ns();
+    set_wait(a);
     void *args[] = {&a};
     const BfsLaunch L = pick_launch(n, g->nnz, o, ctx->num_sms, ctx->bfs_blocks2, ctx->bfs_blocks, grid);
     a.useg = open_list_seg(n, (int64_t)L.blocks * (BFS_THREADS / 32));
@@ -1727,7 +1737,7 @@ gb_status bfs_noalloc_impl(const int64_t *off, const int32_t *col, int64_t n, in
     a.canonical = o.canonical_parents;
     a.vec_out = vec_ok(a);
     a.vec_col = 0;  // a caller's columns: neither alignment nor padding is known
-    a.timeout_ns = timeout_ns();
+    set_wait(a);
     void *args[] = {&a};
     // the scratch holds no open list, so any grid will do; one block per SM at most
     gb_bfs_options one = o;

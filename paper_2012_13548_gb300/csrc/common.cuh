@@ -42,6 +42,13 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p)
     return v;
 }
 
+__device__ __forceinline__ uint64_t ld_acquire_u64(const unsigned long long *p)
+{
+    uint64_t v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v)
 {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -73,45 +80,66 @@ __device__ __forceinline__ uint32_t weight_units(float w)
 // writes) and waits with acquire loads.  Every wait is bounded by
 // `timeout_ns` of the global timer: on expiry the block records
 // GB_ERR_TIMEOUT, and every block leaves early once any block has recorded an
-// error; grid_sync then returns false.  An error recorded before a barrier stops
-// every block at that barrier at the latest (barrier.h).
+// error; grid_sync then returns false.  An error recorded before a barrier (with
+// grid_error) stops every block at that barrier at the latest (barrier.h).
 // ---------------------------------------------------------------------------
 struct GridBarrier {
-    unsigned count;
-    unsigned pad[31];  // a line of its own: the blocks that wait read it all the time, beside
+    unsigned long long word;
+    unsigned pad[30];  // a line of its own: the blocks that wait read it all the time, beside
                        // the atomics on the level's counters of the blocks still at work
 };
 
-__device__ __forceinline__ void red_release_add_u32(unsigned *p, unsigned v)
+__device__ __forceinline__ void red_release_add_u64(unsigned long long *p, uint64_t v)
 {
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// The counter value this launch starts from (a multiple of gridDim.x: every
-// earlier launch on the same barrier passed all its barriers).  Call once at
-// kernel entry, before the block's first grid_sync.
-__device__ __forceinline__ unsigned grid_barrier_base(GridBarrier *b)
+// What thread 0 of a block keeps of the barrier, in shared memory: as registers of every
+// thread for the whole kernel it made the searches spill.
+struct BlockBarrier {
+    BarrierState state;
+    int failed;  // a thread of this block has recorded an error in this launch
+};
+__device__ __forceinline__ BlockBarrier &block_barrier()
 {
-    __shared__ unsigned s_base;
-    if (threadIdx.x == 0) s_base = (ld_acquire_u32(&b->count) / gridDim.x) * gridDim.x;
+    __shared__ BlockBarrier s_bar;
+    return s_bar;
+}
+
+// record_error in a kernel with grid barriers.
+__device__ __forceinline__ void grid_error(DevStatus *st, int code, int where, long long detail)
+{
+    block_barrier().failed = 1;
+    record_error(st, code, where, detail);
+}
+
+// Call once at kernel entry, before the block's first grid_sync and grid_error.  No
+// kernel records an error before its first barrier but by not arriving there, so the
+// error count is the earlier launches'.
+__device__ __forceinline__ void grid_barrier_begin(GridBarrier *b)
+{
+    if (threadIdx.x == 0) {
+        block_barrier().state = barrier_start(ld_acquire_u64(&b->word), gridDim.x);
+        block_barrier().failed = 0;
+    }
     __syncthreads();
-    return s_base;
 }
 
-__device__ __forceinline__ bool grid_sync(GridBarrier *b, unsigned &target, DevStatus *st,
-                                          uint64_t timeout_ns, int site)
+__device__ __forceinline__ bool grid_sync(GridBarrier *b, DevStatus *st, uint64_t timeout_ns, int site)
 {
     __shared__ int s_ok;
-    target += gridDim.x;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        red_release_add_u32(&b->count, 1u);
+        red_release_add_u64(&b->word, barrier_arrival(block_barrier().failed != 0));
+        BarrierState state = block_barrier().state;
+        state.target += gridDim.x;
+        block_barrier().state.target = state.target;
         uint64_t t0 = 0;
         unsigned spins = 0;
         for (;;) {
             const BarrierLook look =
-                barrier_look([&] { return (int)(ld_acquire_u32(&b->count) - target) >= 0; }, [&] { return status_code(st); });
+                barrier_look(state, [&] { return status_code(st); }, [&] { return ld_acquire_u64(&b->word); });
             if (look == BARRIER_ERROR) ok = 0;
             if (look != BARRIER_WAIT) break;
             // the clock from the first poll on, every eighth: a poll is an L2 round

@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
         s_voff[i] = i < a.ng ? s_g[i].voff : s_g[a.ng - 1].voff + s_g[a.ng - 1].n;
     __syncthreads();
     const MsSlots *S = a.slots ? &s_slots : nullptr;
-    unsigned bar_target = grid_barrier_base(&a.hdr->bar);
+    grid_barrier_begin(&a.hdr->bar);
     MsWarpBuf &wb = s_wb[threadIdx.x >> 5];
     int qn_buf = 0, bn_buf = 0;
 
@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                     a.huge[atomicAdd(&h->nhuge, 1ull)] = (int32_t)i;
             }
         }
-        if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_MS_BAR)) return;
+        if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_MS_BAR)) return;
         // roots: bit b of graph g at its root, one thread each; roots that
         // coincide share one entry (the first to set a bit makes it).  One
         // thread placing them all, a chain of some ten memory accesses each,
@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
             if (threadIdx.x == 0)
                 h->acc[2] = (unsigned long long)a.ng * (unsigned long long)a.k;  // the roots themselves
         }
-        if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_MS_BAR)) return;
+        if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_MS_BAR)) return;
     }
     if (a.stats && gtid == 0) h->t0 = globaltimer_ns();
 
@@ -643,7 +643,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
         const int64_t na = (int64_t)ldcg_u64(&cur->na);
         if (na == 0) break;
         if (l - a.l0 > ntot) {
-            if (gtid == 0) record_error(a.st, GB_ERR_TIMEOUT, SITE_MS_LEVELS, l);
+            if (gtid == 0) grid_error(a.st, GB_ERR_TIMEOUT, SITE_MS_LEVELS, l);
             break;
         }
         const int64_t prev_na = l > 0 ? (int64_t)ldcg_u64(&h->na_hist[(l - 1) & 3]) : 0;
@@ -771,7 +771,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
             if (pass == 0) {
                 ms_flush_q(wb, qn_buf, nxt, act_next);
                 ms_flush_b(wb, bn_buf, nxt, bigq_next);
-                if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_MS_BAR)) return;
+                if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_MS_BAR)) return;
                 nn = (int64_t)ldcg_u64(&nxt->na);
                 by_edges = a.canonical && nn > na;
             }
@@ -911,7 +911,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
             h->na_hist[l & 3] = (unsigned long long)na;
             atomicAdd(&h->acc[td ? 4 : 5], 1ull);
         }
-        if (!grid_sync(&h->bar, bar_target, a.st, a.timeout_ns, SITE_MS_BAR)) return;
+        if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_MS_BAR)) return;
         // per-level device time, active vertices and step
         if (a.stats && gtid == 0 && l - a.l0 < kStatLevels) {
             const uint64_t now = globaltimer_ns();

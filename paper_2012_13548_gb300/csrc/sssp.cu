@@ -232,7 +232,7 @@ __device__ __forceinline__ void list_big(const SpArgs &a, SpQueueCtl *q, SpBig *
     const int64_t bi = (int64_t)(old >> 32);
     if (bi < a.bigcap)
         reinterpret_cast<unsigned long long *>(bq)[bi] = (unsigned long long)(uint32_t)v | ((old & 0xffffffffull) << 32);
-    else record_error(a.st, GB_ERR_RANGE, SITE_SP_BIGQ, bi);
+    else grid_error(a.st, GB_ERR_RANGE, SITE_SP_BIGQ, bi);
 }
 
 __device__ __forceinline__ void flush_near(const SpArgs &a, SpWarp &wb, SpFill &f, unsigned qid)
@@ -243,7 +243,7 @@ __device__ __forceinline__ void flush_near(const SpArgs &a, SpWarp &wb, SpFill &
     for (int i = lane_id(); i < f.near; i += 32) {
         const int32_t v = wb.near[i];
         if (base + i < a.n) a.nq[(int64_t)(qid & 1) * a.n + base + i] = v;
-        else record_error(a.st, GB_ERR_RANGE, SITE_SP_NEAR, base + i);
+        else grid_error(a.st, GB_ERR_RANGE, SITE_SP_NEAR, base + i);
         list_big(a, q, a.bq + (int64_t)(qid & 1) * a.bigcap, v, a.off[v + 1] - a.off[v]);
     }
     __syncwarp();
@@ -256,7 +256,7 @@ __device__ __forceinline__ void flush_far(const SpArgs &a, SpWarp &wb, SpFill &f
     const int64_t base = stage_base(&a.hdr->farcnt[epoch & 1], f.far);
     for (int i = lane_id(); i < f.far; i += 32) {
         if (base + i < a.n) a.fq[(int64_t)(epoch & 1) * a.n + base + i] = wb.far[i];
-        else record_error(a.st, GB_ERR_RANGE, SITE_SP_FAR, base + i);
+        else grid_error(a.st, GB_ERR_RANGE, SITE_SP_FAR, base + i);
     }
     __syncwarp();
     f.far = 0;
@@ -271,7 +271,7 @@ __device__ __forceinline__ void flush_settle(const SpArgs &a, SpWarp &wb, SpFill
     for (int i = lane_id(); i < f.settle; i += 32) {
         const int32_t v = wb.settle[i];
         if (base + i < a.n) a.sq[base + i] = v;
-        else record_error(a.st, GB_ERR_RANGE, SITE_SP_NEAR, base + i);
+        else grid_error(a.st, GB_ERR_RANGE, SITE_SP_NEAR, base + i);
         list_big(a, &a.hdr->settle, a.bq + 2 * a.bigcap, v, a.off[v + 1] - a.off[v]);
     }
     __syncwarp();
@@ -472,7 +472,7 @@ __device__ __noinline__ void pull_settle(const SpArgs &a, const int32_t *ids, in
         const int64_t base = stage_base(out_cnt, f.near);
         for (int i = lane; i < f.near; i += 32) {
             if (base + i < a.n) __stcg(&out[base + i], wb.near[i]);
-            else record_error(a.st, GB_ERR_RANGE, SITE_SP_FAR, base + i);
+            else grid_error(a.st, GB_ERR_RANGE, SITE_SP_FAR, base + i);
         }
         __syncwarp();
         f.near = 0;
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
     __shared__ SpWarp s_wb[SP_THREADS / 32];
     SpWarp &wb = s_wb[threadIdx.x >> 5];
     SpFill f;
-    unsigned bar = grid_barrier_base(&h->bar);
+    grid_barrier_begin(&h->bar);
     unsigned long long processed = 0, scanned = 0, won = 0, reached = 0;
     const uint64_t t_start = globaltimer_ns();
     const uint64_t pol = stream_policy();
@@ -606,7 +606,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
             reinterpret_cast<unsigned long long *>(a.bq)[a.bigcap] = (unsigned long long)(uint32_t)a.root;
         }
     }
-    if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
+    if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
 
     unsigned qcur = 1, epoch = 1;
     unsigned long long T = a.delta;
@@ -625,12 +625,12 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
     };
     for (;; ++rounds) {
         if (rounds > a.max_rounds) {  // cannot happen: every queued vertex had its distance lowered
-            if (gtid == 0) record_error(a.st, GB_ERR_TIMEOUT, SITE_SP_ROUNDS, rounds);
+            if (gtid == 0) grid_error(a.st, GB_ERR_TIMEOUT, SITE_SP_ROUNDS, rounds);
             return;
         }
         // a bound on the whole search: the error makes every block leave at its next barrier
         if (gtid == 0 && globaltimer_ns() - t_start > a.run_limit_ns)
-            record_error(a.st, GB_ERR_TIMEOUT, SITE_SP_ROUNDS, rounds);
+            grid_error(a.st, GB_ERR_TIMEOUT, SITE_SP_ROUNDS, rounds);
         const unsigned qnext = qcur + 1;
         // the counters of queue qcur+2; their last readers finished two barriers ago
         if (gtid == 0) {
@@ -660,7 +660,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
                 reinterpret_cast<unsigned long long *>(LB)[old >> 32] =
                     (unsigned long long)(uint32_t)u | ((old & 0xffffffffull) << 32);
             }
-            if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
+            if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
             const unsigned long long lc = __ldcg(&h->light[qcur & 1]);
             const int64_t nlb = (int64_t)(lc >> 32), nch = nlb > 0 ? (int64_t)(lc & 0xffffffffull) : 0;
             for (int64_t c = gwarp; c < nch; c += nwarps) {
@@ -710,7 +710,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
         flush_near(a, wb, f, qnext);
         flush_far(a, wb, f, epoch);
         flush_settle(a, wb, f);
-        if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
+        if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
         phase_end(0);
         if (__ldcg(&h->q[qnext & 3].cnt) > 0) {
             qcur = qnext;
@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
             }
         }
         flush_far(a, wb, f, e);
-        if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
+        if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
         phase_end(1);
         // ---- the least far distance >= T
         if (gtid == 0) {  // every block read the settle list before the barrier above
@@ -798,7 +798,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
             mn = x < mn ? x : mn;
         }
         if (lane == 0 && mn != SP_INF) atomicMin(&h->minfar, mn);
-        if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
+        if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
         phase_end(2);
         const unsigned long long mf = __ldcg(&h->minfar);
         if (mf == SP_INF) break;  // nothing left to settle
@@ -825,7 +825,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
         }
         flush_near(a, wb, f, qnext);
         flush_far(a, wb, f, e + 1);
-        if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
+        if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
         phase_end(3);
         if (gtid == 0) h->minfar = SP_INF;  // every block read it before the barrier above
         ++buckets;
@@ -919,7 +919,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
         atomicAdd(&h->acc[2], won);
         atomicAdd(&h->acc[3], reached);
     }
-    if (!grid_sync(&h->bar, bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
+    if (!grid_sync(&h->bar, a.st, a.timeout_ns, SITE_SP_BAR)) return;
     if (gtid == 0 && a.stats) {
         a.stats->rounds = (unsigned long long)rounds + 1;
         a.stats->buckets = (unsigned long long)buckets + 1;

@@ -1,4 +1,4 @@
-"""The order of a waiting block's two reads at a grid barrier (csrc/barrier.h), on the host.
+"""What a waiting block concludes at a grid barrier (csrc/barrier.h), on the host.
 
 Another block records an error and then arrives; every place of those two steps between
 the waiting block's reads is tried.  A block that passes has to have seen an error recorded
@@ -17,16 +17,21 @@ PROGRAM = r"""
 #include <cstdio>
 // The other block's steps: 1 records an error (if `fails`), 2 arrives.  Step k is made
 // before the waiting block's read number at[k].
-static int run(bool fails, int at1, int at2)
+static int run(bool fails, int at1, int at2, uint64_t start)
 {
-    int reads = 0, status = 0, count = 0;
+    // three blocks, two have arrived
+    gb::BarrierState b = gb::barrier_start(start, 3);
+    b.target += 3;
+    start += gb::barrier_arrival(false);
+    uint64_t word = start + gb::barrier_arrival(false);
+    int reads = 0, status = 0;
     auto others = [&] {
         if (at1 == reads && fails) status = -5;
-        if (at2 == reads) count = 1;
+        if (at2 == reads) word += gb::barrier_arrival(fails);
         ++reads;
     };
     for (int look = 0; look < 20; ++look) {
-        const gb::BarrierLook l = gb::barrier_look([&] { others(); return count == 1; }, [&] { others(); return status; });
+        const gb::BarrierLook l = gb::barrier_look(b, [&] { others(); return status; }, [&] { others(); return word; });
         if (l != gb::BARRIER_WAIT) return l;
     }
     return gb::BARRIER_WAIT;
@@ -34,14 +39,20 @@ static int run(bool fails, int at1, int at2)
 int main()
 {
     int bad = 0;
-    for (int a1 = 0; a1 < 12; ++a1)
-        for (int a2 = a1; a2 < 12; ++a2) {
-            bad += run(true, a1, a2) != gb::BARRIER_ERROR;
-            bad += run(false, a1, a2) != gb::BARRIER_PASSED;
-        }
-    // an error and no arrival: the wait ends
-    bad += run(true, 3, 1000) != gb::BARRIER_ERROR;
-    bad += run(false, 3, 1000) != gb::BARRIER_WAIT;
+    // the words that a launch may start from: none, after other launches, errors among
+    // them (their count about to wrap too), more arrivals than 32 bits hold
+    const uint64_t starts[] = {0, 24, 24 + (uint64_t(5) << 48), (uint64_t(0xffff) << 48) + 3, 0xffffffffull,
+                               uint64_t(3) * 0x55555556ull, uint64_t(3) << 40};
+    for (uint64_t start : starts) {
+        for (int a1 = 0; a1 < 12; ++a1)
+            for (int a2 = a1; a2 < 12; ++a2) {
+                bad += run(true, a1, a2, start) != gb::BARRIER_ERROR;
+                bad += run(false, a1, a2, start) != gb::BARRIER_PASSED;
+            }
+        // an error and no arrival: the wait ends
+        bad += run(true, 3, 1000, start) != gb::BARRIER_ERROR;
+        bad += run(false, 3, 1000, start) != gb::BARRIER_WAIT;
+    }
     std::printf("%d\n", bad);
     return bad != 0;
 }
