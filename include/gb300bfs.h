@@ -218,11 +218,12 @@ gb_status graph_prepare_batched(gb_graph *g, gb_stream s);
  *                      the level array).  It selects the same for sssp
  *                      (smallest-id neighbour on a shortest path).
  *   alpha, beta        direction switch: top-down -> bottom-up when the
- *                      frontier's edges exceed (unexplored edges)/alpha;
+ *                      frontier's edges exceed (unexplored edges)/alpha
+ *                      and the frontier grows;
  *                      bottom-up -> top-down when the frontier shrinks below
  *                      n/beta vertices (Beamer et al., SC 2012).  A
  *                      frontier of hubs (16 times the mean degree) switches
- *                      at 1.4 times that ratio.
+ *                      at 1.4 times that ratio, at most 64.
  *   big_degree         frontier vertices of larger degree are split over the
  *                      whole grid in top-down steps.
  *   ms_alpha, ms_beta  the same switch for the multi-source BFS, on all edges

@@ -152,7 +152,11 @@ struct BfsArgs {
 // neighbour, while every edge of a hub costs top-down its atomic whether or not it
 // finds a vertex.  SCALE 26, a frontier of 16,304 vertices and 150 M edges (just below 1/14): that
 // level 1.68 ms top-down, 0.90 bottom-up, the search 2.32 -> 1.47 ms. Not further: SCALE 24,
-// 2,406 vertices with about 1/21, 0.28 ms top-down, 0.38 bottom-up.
+// 2,406 vertices with about 1/21, 0.28 ms top-down, 0.38 bottom-up.  In canonical
+// mode and for a caller's arrays no hub is tested first, but a hub's edges cost top-down
+// twice, for the claims and for the smallest parents: us a search over 64 roots with
+// the rule / without it, canonical, SCALE 20 122.5 / 122.8, SCALE 22 235.1 / 235.6, SCALE 24
+// 618 / 621 (slowest root 849 / 1015); bfs_noalloc, SCALE 20, 153.1 / 154.3.
 constexpr float HUB_MEAN = 16.0f;
 __device__ __forceinline__ bool go_bottom_up(float mf, float mu, float qn, const BfsArgs &a)
 {
