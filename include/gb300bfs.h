@@ -308,7 +308,9 @@ gb_status bfs_noalloc(const int64_t *off, const int32_t *col, int64_t n, int64_t
  * synchronises the stream of that call.
  *   nlevels          number of BFS levels (max level + 1)
  *   edges_examined   adjacency entries read (top-down: frontier degrees;
- *                    bottom-up: neighbours tested before the first hit)
+ *                    bottom-up: neighbours tested before the first hit; the
+ *                    second look for the smallest parent in canonical mode
+ *                    is not counted)
  *   vertices_touched frontier vertices expanded plus unvisited vertices
  *                    tested
  *   reached          vertices with level >= 0 (summed over roots)

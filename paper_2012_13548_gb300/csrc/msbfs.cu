@@ -710,7 +710,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                                           ((cc & ((1 << ps) - 1)) * MS_BIG_CHUNK >> ps);
                         const int64_t eu = G.off[lv + 1];
                         const int64_t e = s + (MS_BIG_CHUNK >> ps) < eu ? s + (MS_BIG_CHUNK >> ps) : eu;
-                        if (lane == 0 && e > s) my_edges += (unsigned long long)(e - s);
+                        if (lane == 0 && e > s && pass == 0) my_edges += (unsigned long long)(e - s);
                         for (int64_t b = s; b < e; b += 32) {
                             const int64_t j = b + lane;
                             const bool valid = j < e;
@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                     f = ld_mask(&M[gv]);
                 }
                 my_touched += (i < na && pass == 0);
-                my_edges += d;
+                if (pass == 0) my_edges += d;
                 const int64_t incl = warp_inclusive_scan(d);
                 const int64_t total = __shfl_sync(kFull, incl, 31);
                 const int64_t excl = incl - d;
@@ -796,7 +796,8 @@ __global__ void __launch_bounds__(MS_THREADS, 2) ms_kernel(MsArgs<T> a)
                         re = s_g[g].off[lu + 1];
                     }
                 }
-                if (by_rows) ms_rows(s_g, S, M, g, orig_id(s_g[g], lu), rs, re, nw, my_edges);
+                unsigned long long again = 0;  // like pass 1, no part of the search's edges
+                if (by_rows) ms_rows(s_g, S, M, g, orig_id(s_g[g], lu), rs, re, nw, again);
                 if (i < nn) {
                     st_mask(&a.seen[gu], (T)(ld_mask(&a.seen[gu]) | nw));
                     if (a.hist && l + 1 < MS_HIST)

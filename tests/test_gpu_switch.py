@@ -48,3 +48,18 @@ def test_ms_alpha_acts_as_it_is_set(ms_alpha, step):
         _, levels = gb.bfs_batch(g, [0, 0])
         assert gb.bfs_last_stats()["level_dir"][:2] == ["td", step]
         assert np.array_equal(levels[1].cpu().numpy(), oracle.bfs(off, col, 0)[1])
+
+
+@pytest.mark.parametrize("canonical", [0, 1])
+def test_edges_examined_counts_the_frontiers_edges_once(canonical):
+    # top-down only: every reached vertex's row, however the smallest parents are found
+    rng = np.random.default_rng(2)
+    graphs = [hubs(12, 7, 300, 3000, rng)[:3], hubs(13, 300, 20, 9000, rng)[:3]]
+    gb.bfs_set_options(canonical_parents=canonical, alpha=1e-9, beta=1e-9, ms_alpha=1e-9, ms_beta=1e-9)
+    for g, off, col in graphs:
+        _, level = oracle.bfs(off, col, 0)
+        rows = int(np.diff(off)[level >= 0].sum())
+        gb.bfs(g, 0)
+        assert gb.bfs_last_stats()["edges_examined"] == rows
+        gb.bfs_batch(g, [0, 0])
+        assert gb.bfs_last_stats()["edges_examined"] == rows
