@@ -99,6 +99,11 @@ int64_t gb_debug_live_allocations(void);
  * weight-ordered rows together. */
 gb_status gb_debug_build_route(int *digits, int *splits);
 
+/* How many settle steps of this thread's last sssp call read the heavy edges from
+ * the rows of the unsettled vertices (library bookkeeping, for tests;
+ * synchronises the call's stream).  GB_ERR_INVALID before the first call. */
+gb_status gb_debug_sssp_pulls(int64_t *pulls);
+
 /* Synchronise `s`, then return and clear the device status word: GB_OK, or
  * the first GB_ERR_RANGE / GB_ERR_TIMEOUT a kernel recorded since the last
  * call. */

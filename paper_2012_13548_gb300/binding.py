@@ -95,6 +95,7 @@ def lib():
             "gb_debug_fail_allocations": (ctypes.c_int, [_i64, _i64]),
             "gb_debug_live_allocations": (_i64, []),
             "gb_debug_build_route": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
+            "gb_debug_sssp_pulls": (ctypes.c_int, [ctypes.POINTER(_i64)]),
             "gb_sort_portion": (_i64, []),
             "gb_device_status": (ctypes.c_int, [_vp]),
             "kron_generate": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_double,
@@ -157,7 +158,7 @@ def exported_symbols():
     """Names of the C-ABI functions this binding wraps."""
     return ["gb_last_error", "gb_abi_version", "gb_kernel_launches", "gb_set_sort_portion",
             "gb_sort_portion", "gb_debug_fail_allocations", "gb_debug_live_allocations",
-            "gb_debug_build_route",
+            "gb_debug_build_route", "gb_debug_sssp_pulls",
             "gb_device_status", "kron_generate",
             "graph_build_csr", "graph_build_csr_counting", "graph_from_csr", "graph_generate_csr",
             "graph_free", "graph_info", "graph_csr_view", "graph_prepare_batched",
@@ -279,6 +280,13 @@ def debug_build_route():
     d, s = ctypes.c_int(), ctypes.c_int()
     _check(lib().gb_debug_build_route(ctypes.byref(d), ctypes.byref(s)))
     return d.value, s.value
+
+
+def debug_sssp_pulls():
+    """Settle steps of this thread's last sssp call that started from the unsettled end."""
+    n = _i64()
+    _check(lib().gb_debug_sssp_pulls(ctypes.byref(n)))
+    return n.value
 
 
 def gb_device_status(stream=None):

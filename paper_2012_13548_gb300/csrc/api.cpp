@@ -457,6 +457,21 @@ gb_status sssp(const gb_graph *g, int64_t root, double delta, double *dist, int3
     });
 }
 
+gb_status gb_debug_sssp_pulls(int64_t *pulls)
+{
+    return guarded([&]() -> gb_status {
+        if (!pulls || !t_sssp.valid || !t_sssp.dev) {
+            set_error("gb_debug_sssp_pulls: NULL, or no sssp call on this thread yet");
+            return GB_ERR_INVALID;
+        }
+        SsspDevStats h;
+        GB_CUDA(cudaStreamSynchronize(t_sssp.stream));
+        GB_CUDA(cudaMemcpy(&h, t_sssp.dev, sizeof(h), cudaMemcpyDeviceToHost));
+        *pulls = (int64_t)h.pulls;
+        return GB_OK;
+    });
+}
+
 gb_status sssp_last_stats(gb_sssp_stats *out)
 {
     return guarded([&]() -> gb_status {

@@ -225,6 +225,7 @@ struct SsspDevStats {
     unsigned long long reached;    // vertices with a finite distance
     unsigned long long delta;      // bucket width in units of 2^-24
     unsigned long long phase_ns[4];  // device time: expansion rounds, settle steps, far minima, far splits
+    unsigned long long pulls;        // settle steps from the unsettled end (gb_debug_sssp_pulls)
 };
 gb_status sssp_impl(const gb_graph *g, int64_t root, double delta, double *dist, int32_t *parent,
                     SsspDevStats *stats, cudaStream_t s);

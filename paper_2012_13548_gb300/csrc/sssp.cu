@@ -928,6 +928,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_MINB) sssp_kernel(SpArgs a)
         a.stats->won = __ldcg(&h->acc[2]);
         a.stats->reached = __ldcg(&h->acc[3]);
         a.stats->delta = a.delta;
+        a.stats->pulls = pulls;
         for (int k = 0; k < 4; ++k) a.stats->phase_ns[k] = ph[k];
     }
 }

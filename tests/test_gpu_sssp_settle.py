@@ -3,7 +3,8 @@
 A bucket's heavy edges are read from the settled rows or from the rows of what is
 still unsettled, whichever is less; rows below and above 64 and 1024 entries, buckets
 from one unit of the weights to the whole search, equal weights (ties at every
-bound), unreachable parts.
+bound), unreachable parts.  How often the second end is taken follows from the final
+distances; the searches have to take it as often, and the cases hold both.
 """
 import numpy as np
 import pytest
@@ -42,6 +43,30 @@ def graph(kind, rng):
     return scale, np.stack([u, v]).astype(np.int64)
 
 
+def expected_pulls(off, dist, delta):
+    """The settle steps from the unsettled end: those where the degrees of the vertices
+    that the bucket settles exceed a quarter of what is left (the unsettled degrees and
+    the length of the list of vertices to look at: all at first, then those that
+    the last such step left)."""
+    units = dist * 2.0 ** 24                       # whole numbers
+    width = max(1.0, np.floor(delta * 2.0 ** 24 + 0.5))
+    deg = np.diff(off)
+    n, nnz, settled, listed, pulls, before = len(deg), int(off[-1]), 0.0, float(len(deg)), 0, 0
+    top = width
+    while True:
+        below = units < top
+        settled = int(deg[below].sum())
+        if settled - before > 0.25 * (nnz - settled + listed):
+            pulls += 1
+            listed = float(np.count_nonzero(~below & (deg > 0)))
+        before = settled
+        left = units[~below]
+        least = left.min() if left.size else np.inf
+        if not np.isfinite(least):
+            return pulls
+        top = (least // width + 1) * width
+
+
 @pytest.mark.parametrize("weights", ["any", "one", "tiny"])
 @pytest.mark.parametrize("kind", ["hubs", "middle", "path", "parts"])
 def test_distances_equal_the_oracle(kind, weights):
@@ -55,7 +80,7 @@ def test_distances_equal_the_oracle(kind, weights):
     edges = torch.as_tensor(e).cuda()
     deg = np.diff(off)
     roots = [int(deg.argmax()), int(np.nonzero(deg > 0)[0][0]), int(rng.choice(np.nonzero(deg > 0)[0]))]
-    saved = gb.bfs_get_options()
+    saved, ends = gb.bfs_get_options(), set()
     try:
         for r in roots:
             d_ref, _ = oracle.sssp(off, col, wr, r)
@@ -63,10 +88,15 @@ def test_distances_equal_the_oracle(kind, weights):
                 for canonical in (0, 1):
                     gb.bfs_set_options(canonical_parents=canonical)
                     dist, parent = gb.sssp(G, r, delta)
+                    pulls = gb.debug_sssp_pulls()
+                    assert pulls == expected_pulls(off, d_ref, delta)
+                    ends.add(pulls > 0)
                     assert np.array_equal(dist.cpu().numpy(), d_ref), (r, delta, canonical)
                     if canonical:
                         assert np.array_equal(parent.cpu().numpy(), oracle.sssp_tree(off, col, wr, r, d_ref))
                     assert gb.sssp_validate(G, r, parent, dist, edges)["code"] == 0
     finally:
         gb.bfs_set_options(**saved)
+    if weights == "any" and kind != "middle":   # rows of every length: some searches never pull
+        assert ends == {True, False}
     gb.gb_device_status()
