@@ -38,11 +38,11 @@ PLAIN_SPACE = {
     "blocks_per_sm": [1, 2, 3],
 }
 MS_SPACE = {
-    "ms_alpha": [1.0, 4.0, 16.0, 64.0, 256.0],
+    "ms_alpha": [1.0, 4.0, 16.0, 64.0, 256.0],  # 16, the default, leaves the ratio to the library
     "ms_beta": [2.0, 8.0, 32.0, 128.0],
 }
 SSSP_SPACE = {
-    "delta": [0.03, 0.05, 0.075, 0.1, 0.125, 0.15, 0.2, 0.3],
+    "delta": [0.03, 0.05, 0.0625, 0.075, 0.0875, 0.1, 0.125, 0.15, 0.2, 0.3],
 }
 
 
