@@ -83,3 +83,14 @@ def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(binding, "LIB_PATH", os.path.join(ROOT, "no_such_dir", "lib.so"))
     with pytest.raises(RuntimeError, match="missing"):
         binding.lib()
+
+
+def test_the_index_checking_variant_compiles(tmp_path):
+    # build_ext --checked: the checks are code that the ordinary build never sees
+    import subprocess
+    from paper_2012_13548_gb300 import build_ext
+    cmd = [build_ext._nvcc()] + build_ext.ARCH + ["-O0", "-std=c++17", "-DGB_CHECKED", "-I", build_ext.INCLUDE,
+                                                  "-I", build_ext.CSRC, "-c", os.path.join(build_ext.CSRC, "bfs.cu"),
+                                                  "-o", str(tmp_path / "bfs.o")]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
