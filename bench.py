@@ -572,7 +572,7 @@ def run_ours(args, dist):
     mean_ms = statistics.mean(flat_ms)
     achieved = mean_bytes / (mean_ms * 1e-3) / 1e9
     traffic, traffic_note = read_traffic(scale, mean_bytes)
-    k1_bytes = kernel1_bytes(edges.shape[1], scale, g.nnz, n)
+    k1_bytes = kernel1_bytes(edges.shape[1], g.nnz, n)
 
     # end to end through the public API from pinned host memory
     e2e = None if args.no_e2e else run_e2e(args, gb, torch, edges, scale, roots, m_r, dist)
@@ -694,15 +694,10 @@ def batched_vs_plain(args, gb, torch, scale, dist):
             "invalid_trees": int(dist.max(float(bad)))}
 
 
-def kernel1_bytes(m, scale, nnz, n):
-    """Algorithmic HBM bytes of kernel 1 by buckets: the tuples read twice (digit
-    counts, move); above 2^21 keys 8-byte keys written and read twice for the
-    second digit; 4-byte entries written, read and written by the bucket
-    sorts and read by the compaction; columns and offsets written.  The further
-    splits of long buckets are not counted."""
-    nk = 2 * m
-    keys = 24 * nk if nk > 1 << 21 else 0
-    return 32 * m + keys + 16 * nk + 4 * nnz + 8 * (n + 1)
+def kernel1_bytes(m, nnz, n):
+    """HBM bytes that kernel 1 cannot do without: the tuples read once, columns
+    and offsets written once."""
+    return 16 * m + 4 * nnz + 8 * (n + 1)
 
 
 def read_traffic(scale, alg_bytes_per_launch):
@@ -736,7 +731,7 @@ def kernel_source_hash(main="bfs.cu"):
     import hashlib
     import re
     h = hashlib.sha256()
-    for f in (main, "common.cuh"):
+    for f in (main, "common.cuh", "barrier.h"):
         src = open(os.path.join(ROOT, "paper_2012_13548_gb300", "csrc", f)).read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
         src = re.sub(r"//[^\n]*", " ", src)
