@@ -151,7 +151,9 @@ gb_status kron_generate(int scale, int edgefactor, double a, double b, double c,
  * of largest degree among the first 128 of its row, tested first by the
  * bottom-up step) and, for the bottom-up list walks, each hub again beside
  * the vertex's degree saturated at 65535 (8 * n bytes).  The column array is padded to a multiple of 4
- * entries. */
+ * entries.  Temporaries: about 27 * m bytes, 32 * m where the radix sort
+ * serves (SCALE 27 and more, 2^31 tuples and more, a caller's own sort
+ * portions). */
 gb_status graph_build_csr(const int64_t *edges, int64_t m, int scale, gb_graph **out,
                           gb_stream s);
 
@@ -404,7 +406,11 @@ gb_status kron_weights(int64_t m, uint64_t seed_weight, float *w, gb_stream s);
  * weight outside (0, 1] (NaN included).  Synchronises `s`; the graph also
  * holds 12 * nnz bytes for the weights: one weight per CSR entry and every
  * row again as (column, weight) pairs by ascending weight, which the search
- * reads (built by one radix sort; temporaries about 24 * nnz bytes). */
+ * reads.  Temporaries: about 35 * m bytes while the tuples are sorted, then
+ * about 17 * nnz while the rows are ordered by weight; SCALE 25 and 26 (whose
+ * keys leave no room for the weight) 27 * m and 17 * nnz, larger graphs and
+ * a caller's own sort portions 32 * m and, from 2^32 entries on or with
+ * portions, 24 * nnz (radix sorts). */
 gb_status graph_build_csr_weighted(const int64_t *edges, const float *w, int64_t m, int scale,
                                    gb_graph **out, gb_stream s);
 
@@ -426,7 +432,7 @@ gb_status graph_weights_view(const gb_graph *g, const uint32_t **wgt);
  * smallest-id one when the canonical_parents option is set; -1 if
  * unreachable).  The distances are those of Dijkstra's algorithm exactly; in
  * canonical mode the parent array is the unique canonical tree of them.
- * Allocates about 40 * n bytes of stream-ordered scratch.  GB_ERR_RANGE for
+ * Allocates about 48 * n bytes of stream-ordered scratch.  GB_ERR_RANGE for
  * a root outside [0, n); GB_ERR_INVALID for an unweighted graph. */
 gb_status sssp(const gb_graph *g, int64_t root, double delta, double *dist, int32_t *parent,
                gb_stream s);

@@ -152,7 +152,10 @@ struct BfsArgs {
 // neighbour, while every edge of a hub costs top-down its atomic whether or not it
 // finds a vertex.  SCALE 26, a frontier of 16,304 vertices and 150 M edges (just below 1/14): that
 // level 1.68 ms top-down, 0.90 bottom-up, the search 2.32 -> 1.47 ms. Not further: SCALE 24,
-// 2,406 vertices with about 1/21, 0.28 ms top-down, 0.38 bottom-up.  In canonical
+// 2,406 vertices with about 1/21, 0.28 ms top-down, 0.38 bottom-up.  Mean us a search over 128
+// roots with the factor 1 / 1.2 / 1.4 / 2 / 4: SCALE 20 104.9 / 104.9 / 104.9 / 105.5 / 106.3,
+// SCALE 22 162.5 / 161.9 / 161.9 / 162.3 / 166.0, SCALE 24 367.9 / 367.5 / 367.3 / 368.9 / 382.0, SCALE
+// 26 1177 / 1155 / 1156 / 1158 / 1201 (slowest root 2227 / 1791 / 1791 / 1895 / 2411).  In canonical
 // mode and for a caller's arrays no hub is tested first, but a hub's edges cost top-down
 // twice, for the claims and for the smallest parents: us a search over 64 roots with
 // the rule / without it, canonical, SCALE 20 122.5 / 122.8, SCALE 22 235.1 / 235.6, SCALE 24
@@ -275,7 +278,7 @@ __device__ __forceinline__ void flush_big(WarpBuf &wb, int &bn, const BfsArgs &a
 }
 
 // Block-collective, at the end of a level: what the warps still hold staged, with
-// one atomic per block and list.  Each of up to 9728 warps took one for
+// one atomic per block and list.  Each of 4864 warps (two blocks per SM) took one for
 // itself, 1.6 ns apiece on the same address: 8 us a list and level.
 struct LevelFlush {
     unsigned q[32];              // staged vertices of every warp, then where they go
@@ -746,11 +749,12 @@ __device__ __forceinline__ void solo_min_parent(const BfsArgs &a, int64_t j, int
 // and counters in that chain it took 7.5-10 us, whatever the frontier's size.
 // Here the frontier stays in shared memory with its row starts and degrees (a
 // discovered vertex's offsets are loaded beside the atomic that claims it), so
-// a level is two round trips to L2 (column, claim) and one block barrier.  A
-// frontier of short rows is dealt one vertex per thread; any other one edge
+// a level is two round trips to L2 (column, claim) and one block barrier, three where
+// the rows are short (their targets are tested before they are claimed).  A
+// frontier of short rows is dealt four or eight lanes a row; any other one edge
 // by edge, each thread finding its edges' vertices in the prefix of the
 // degrees, so that a hub does not hold one warp.  A 997 x 601 mesh (1,233
-// levels, frontiers of up to 1,000 vertices): 12.3 -> 6.3 ms, 10.0 -> 5.1 us a
+// levels, frontiers of up to 1,000 vertices): 12.3 -> 5.4 ms, 10.0 -> 4.4 us a
 // level; levels of three vertices 2.3 us.
 //
 // The frontier bitmaps are not kept during the stretch: nothing reads them
