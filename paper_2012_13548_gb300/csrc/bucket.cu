@@ -1369,18 +1369,18 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
     if (bp.p1) plan_rest(ar, l1, n0, nk / BK_TILE + 1 + n0, n1, n1);
     plan_rest(ar, l2, seg_x, tile_x, piece2, desc_x);
 
+    const size_t o_kb = ar.take((size_t)nk * sizeof(K));
+    const size_t o_ka = ar.take((size_t)nk * (bp.p1 ? sizeof(uint64_t) : sizeof(K)));
+
+    // all in one block: a build that repeats gets the same one from the pool, where blocks
+    // of several sizes, freed and taken between the graphs' arrays, made the pool
+    // map memory anew (SCALE 26: 54.3 to 59.1 ms in turns, so 54.2 to 54.5)
     Scratch tmp(s);
     unsigned char *ws = nullptr;
-    K *ka = nullptr, *kb = nullptr;  // entries after step 1 (kb), and a second buffer for the splits
-    uint64_t *k0 = nullptr;          // entries after step 0, where step 1 follows
     GB_CUDA(tmp.alloc(&ws, ar.used));
-    GB_CUDA(tmp.alloc(&kb, (size_t)nk));
-    if (bp.p1) {
-        GB_CUDA(tmp.alloc(&k0, (size_t)nk));
-        ka = reinterpret_cast<K *>(k0);
-    } else {
-        GB_CUDA(tmp.alloc(&ka, (size_t)nk));
-    }
+    K *kb = reinterpret_cast<K *>(ws + o_kb);  // entries after step 1
+    K *ka = reinterpret_cast<K *>(ws + o_ka);  // a second buffer for the splits,
+    uint64_t *k0 = reinterpret_cast<uint64_t *>(ws + o_ka);  // before them the entries after step 0, where step 1 follows
     GB_CUDA(cudaMemsetAsync(ws, 0, zeroed, s));
     unsigned *cnt0 = reinterpret_cast<unsigned *>(ws + o_cnt0), *cur0 = reinterpret_cast<unsigned *>(ws + o_cur0);
     unsigned *total = reinterpret_cast<unsigned *>(ws + o_total);
@@ -1528,12 +1528,11 @@ gb_status bucket_weight_order(const gb_graph *g, uint2 *wadj, cudaStream_t s)
     const size_t zeroed = ar.used;
     const size_t o_desc = ar.take((size_t)nd * sizeof(BkDesc));
     plan_rest(ar, l2, seg_x, tile_x, piece2, desc_x);
+    const size_t o_ka = ar.take((size_t)nnz * 8), o_kb = ar.take((size_t)nnz * 8);
     Scratch tmp(s);
     unsigned char *ws = nullptr;
-    uint64_t *ka = nullptr, *kb = nullptr;
     GB_CUDA(tmp.alloc(&ws, ar.used));
-    GB_CUDA(tmp.alloc(&ka, (size_t)nnz));
-    GB_CUDA(tmp.alloc(&kb, (size_t)nnz));
+    uint64_t *ka = reinterpret_cast<uint64_t *>(ws + o_ka), *kb = reinterpret_cast<uint64_t *>(ws + o_kb);
     GB_CUDA(cudaMemsetAsync(ws, 0, zeroed, s));
     BkDesc *desc = reinterpret_cast<BkDesc *>(ws + o_desc);
     const Level lv2 = level_at(ws, l2);
