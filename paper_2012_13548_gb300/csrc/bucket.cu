@@ -1280,16 +1280,16 @@ Level level_at(unsigned char *b, const LevelPlan &p)
     return l;
 }
 
-// Why by the bits that differ: splits at fixed digits took 10 bits whether or not keys
-// differed in them, gave up after two, and the LSD sort began anew (SCALE 20 as
-// drawn 3.1 ms; unit weights beside a row of 10^5, whose weight bits are all
-// equal, 6.6 ms, now 3.2).  Where length alone asks for a second split (rows beyond
-// 2^10 pieces) a turn costs 20 us more than a third fixed digit did, for its two
-// launches more.
 // What the sorts of `from`'s pieces left because it was too long, `left` pieces with
 // their keys in ka: split from the bits they differ in and sorted into kb, until nothing is left.
 // Every turn a piece gives up at least the bit that parts its keys, so there are at most 64.
 // look(ctl, &left): waits for the stream and reads ctl's overflow.
+// Why by the bits that differ: splits at fixed digits took 10 bits whether or not keys
+// differed in them, gave up after two, and the LSD sort began anew (SCALE 20 as
+// drawn 3.1 ms, now 1.46; unit weights beside a row of 10^5, whose weight bits are all
+// equal, 6.6 ms, now 3.2).  Where length alone asks for a second split (more than 2^10
+// pieces of one bucket) a turn costs 10 to 20 us more than a third fixed digit did, for its
+// two launches more.
 template <typename K, int MODE, typename Look>
 gb_status split_rest(Context *ctx, LeafArgs la, Level from, unsigned left, int low, int64_t nk, K *ka, K *kb,
                      Look look, cudaStream_t s)
@@ -1371,7 +1371,6 @@ gb_status build(const int64_t *edges, const float *w, int64_t m, int scale, cons
 
     const size_t o_kb = ar.take((size_t)nk * sizeof(K));
     const size_t o_ka = ar.take((size_t)nk * (bp.p1 ? sizeof(uint64_t) : sizeof(K)));
-
     // all in one block: a build that repeats gets the same one from the pool, where blocks
     // of several sizes, freed and taken between the graphs' arrays, made the pool
     // map memory anew (SCALE 26: 54.3 to 59.1 ms in turns, so 54.2 to 54.5)
