@@ -76,7 +76,8 @@ uint64_t gb_kernel_launches(void);
  * 1 <= keys <= 2^28 (the default, and what 0 restores).  Every portion size
  * gives the same result; smaller portions only add kernel launches, and a test
  * uses them to run the chained path, which the default reaches only above
- * 2^28 keys, on small inputs.  Process-wide; applies to later calls.
+ * 2^28 keys, on small inputs.  At the default, kernel 1 sorts by buckets
+ * wherever they serve; any other value asks for the radix sort there too.  Process-wide; applies to later calls.
  * GB_ERR_INVALID outside that range. */
 gb_status gb_set_sort_portion(int64_t keys);
 int64_t gb_sort_portion(void);
@@ -157,7 +158,7 @@ gb_status kron_generate(int scale, int edgefactor, double a, double b, double c,
 gb_status graph_build_csr(const int64_t *edges, int64_t m, int scale, gb_graph **out,
                           gb_stream s);
 
-/* Kernel 1 by counting sort instead of a radix sort of the edges (Sec. 2.2
+/* Kernel 1 by counting sort instead of a sort of the edges (Sec. 2.2
  * builds the CSR from the edges in sorted order; here the rows are counted,
  * the endpoints scattered into them, and each row sorted on its own): the
  * same graph as graph_build_csr, bit for bit, for the same arguments.  Row
